@@ -359,15 +359,15 @@ trk_status tracker_project_keypoints(trk_tracker *t, const float *states_dev, in
  *   S(p)   = 1 - prod_t (1 - a_t(p)) over every triangle of every link,
  *   L      = sum_p (S(p) - M(p))^2.
  * Triangles with a flagged vertex or zero area are left out.  FP32
- * arithmetic; the loss sums the tiles' squared errors in a fixed order and
- * the gradient sums are exact 64-bit fixed-point integers, so repeated calls
- * give identical results.
+ * arithmetic; the sums over pixel blocks and triangles are exact 64-bit
+ * fixed-point integers, so repeated calls give identical results.
  * ------------------------------------------------------------------------- */
 
 /* loss_dev[lam] = L of each candidate of params_dev [lam*d]; with grad_dev
  * [lam*d] not NULL also dL/dparams (physical units: rad, mm, rad of q-hat).
- * The backward recomputes the forward tile by tile: no per-pixel state is
- * kept between the passes.  sigma in [0.05, 64] px.  Asynchronous. */
+ * A call on more candidates than about two gigabytes of scratch hold takes
+ * them in slices (the results are the same).  sigma in [0.05, 64] px.
+ * Asynchronous. */
 trk_status soft_eval(trk_tracker *t, const float *params_dev, int32_t lam, const uint32_t *mask_packed_dev,
                      float sigma, float *loss_dev, float *grad_dev, void *stream);
 

@@ -6,47 +6,68 @@
 //   d_t(p)  signed distance (px) from pixel centre p to the boundary of
 //           projected triangle t (+ inside, - outside), unsnapped coordinates
 //   a_t(p)  sigmoid(d_t(p) / sigma), 0 where d_t(p) < -14 sigma
-//   S(p)    1 - prod_t (1 - a_t(p)) = 1 - exp(-sum_t softplus(d_t(p) / sigma))
+//   S(p)    1 - prod_t (1 - a_t(p)) = 1 - 1 / prod_t (1 + exp(d_t(p) / sigma))
 //   L       sum_p (S(p) - M(p))^2
 // and dL/dd_t(p) = 2 (S - M) (1 - S) sigmoid(d_t / sigma) / sigma, taken back
-// through the closest boundary feature to the projected vertices, through the
+// through the closest boundary point to the projected vertices, through the
 // pinhole to camera coordinates and through the kinematics to the state.
 // Everything is FP32.
 //
 // Launches per call (one row of kernels per population):
-//   k_soft_project  per (candidate, instrument): kinematics with the nine
-//                   state tangents carried along (forward mode), vertex
-//                   projection, screen box of the instrument
-//   k_soft_tribox   per (candidate, triangle): window of influence (bounding
-//                   box grown by 14 sigma) clipped to the image, and the union
-//                   of the windows of every chunk of 256 triangles
-//   k_soft_tile     per (candidate, 16x16 tile): pass 1 sums the softplus
-//                   terms of every triangle whose window meets the tile into
-//                   the tile's pixels and adds the tile's squared error to the
-//                   loss; with a gradient, pass 2 recomputes the same pairs
-//                   and scatters dL/d(u, v) to the vertices.  Nothing per pixel
-//                   leaves the tile: the backward recomputes instead of storing.
-//   k_soft_reduce   per (candidate, instrument): dL/dX per vertex, reduced per
-//                   kinematic frame to a 3x4 matrix G_f, contracted with the
-//                   frame tangents dT_f/dtheta_k; writes loss and gradient.
+//   k_soft_fk       per (candidate, instrument): kinematics with the nine
+//                   state tangents carried along (forward mode); clears the
+//                   candidate's accumulators
+//   k_soft_tris     a warp per group of 32 triangles: projection, edge
+//                   records, boxes; marks the 8x4-pixel blocks that the group
+//                   can reach and lists each marked block once
+//   k_soft_fwd      per listed block: the product over the triangles, the
+//                   block's squared error and, for a gradient, the factor
+//                   2 (S - M) (1 - S) / sigma of its pixels
+//   k_soft_bwd      per (group, part of its window): dL/d(u, v) of the
+//                   group's triangles, added to the vertices
+//   k_soft_reduce   dL/dX per vertex, reduced per kinematic frame to a 3x4
+//                   matrix G_f, contracted with the tangents dT_f/dtheta_k
+//
+// Both pair kernels put triangles on the lanes and walk the pixels together:
+// a triangle's record stays in registers (no shared-memory read per pair), the
+// two coordinates of a pixel in an edge's frame are one FMA each from the
+// previous ones, and nothing is exchanged between lanes per pair -- the forward
+// keeps one running product per pixel and lane, the backward one sum per
+// vertex coordinate and lane.
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 
 namespace trk {
 
 constexpr float kSoftCutoff = 14.0f;   // in units of sigma
-constexpr int kTile = 16;              // tile edge (px): one pixel per thread
+constexpr int kBlkW = 8, kBlkH = 4;    // pixel block of the pair kernels: one pixel per lane at its ends
+constexpr int kBlkPx = kBlkW * kBlkH;
 constexpr int kSoftThreads = 256;
-constexpr int kChunk = 256;            // triangles staged per pass
+constexpr int kFwdWarps = 4;           // most warps that share a block of the forward
+constexpr int kBwdSeg = 64;            // blocks of a group's window per backward unit ...
+constexpr int kBwdMaxSeg = 16;         // ... and at most this many units per group
+// With 1 + Q = prod (1 + exp): Q above kOne makes 1 - S < 2^-25, S is 1 in FP32
+// and the pixel's gradient factor 0, whatever the remaining triangles add.  The
+// forward stops early only at the larger kSaturated, so that a product formed
+// in another order cannot fall below kOne again.
+constexpr float kOne = 3.4e7f, kSaturated = 6.6e7f;
 // Gradient sums are accumulated in 64-bit fixed point, exact and so independent
 // of the order of the (atomic) additions: dL/d(u, v) per vertex in units of
-// 2^-32 (|sum| < 2^31), the per-frame G_f in units of 2^-24 (|sum| < 2^39).
-constexpr double kGvScale = 4294967296.0;
-constexpr double kGScale = 16777216.0;
-__device__ __forceinline__ long long to_fixed(float x, double scale) { return __double2ll_rn((double)x * scale); }
+// 2^-36 (|sum| < 2^27: with x_t = softplus(d_t / sigma) >= sigmoid, a pixel adds
+// at most 2 / sigma * sum_t sigmoid_t * exp(-sum_t x_t) <= 2 / (e sigma), so an
+// image of TRK_MAX_PIXELS at the smallest sigma, 0.05 px, stays below 2^25),
+// the per-frame G_f in units of 2^-24 (|sum| < 2^39) and the remainders in units
+// of 2^-56 (a gradient that nearly vanishes keeps its digits).
+constexpr float kGvScale = 68719476736.0f;
+constexpr float kRestScale = 4294967296.0f;
+constexpr float kGScale = 16777216.0f;
+constexpr double kLossScale = 4294967296.0;  // the loss, in units of 2^-32
+// (a power of two times a float is exact in FP32: no FP64 arithmetic needed)
+__device__ __forceinline__ long long to_fixed(float x, float scale) { return __float2ll_rn(x * scale); }
 
 // ---------------------------------------------------------------------------
 // Forward-mode kinematics: every lane carries the values and one tangent
@@ -238,31 +259,64 @@ struct SoftArgs {
     ChainDev ch;
     int nF, nI, V, T, d, lam;
     float fx, fy, cx, cy, z_near, guard, sigma;
-    int W, H, Wq, ntx, nty;
+    int W, H, Wq;
+    int nbx, nby, wpr;        // pixel blocks per row and column, bitmap words per block row
+    int ngroups, NTp;         // groups of 32 triangles (over all instruments), triangles padded to whole groups
     const float4 *verts;
     const int4 *tris;
     const float *params;      // [lam * d]
     const uint32_t *mask;
-    float4 *sv;               // [lam * nI * V]: u - cx, v - cy, Z, flag
-    longlong2 *gv;            // [lam * nI * V]: dL/du, dL/dv in fixed point (units of 2^-32)
+    float *Tf;                // [lam * nI * nF * 12] camera-from-frame transforms
     float *dT;                // [lam * nI * nF * 9 * 12]
-    short4 *box;              // [lam * nI * T]: window j0, i0, j1, i1 (j0 > j1: none)
-    int4 *cbox;               // [lam * nchunk]: union of the windows of each chunk
-    int nchunk;
-    int4 *ibox;               // [lam * nI]: window of the instrument
-    double *lpart;            // [lam * ntx * nty]: squared error of each tile
+    float4 *rec;              // [4][lam * NTp] edge records (struct TriRec)
+    float4 *box;              // [lam * NTp] centre and half extents of the triangle's bounding box
+    short4 *gwin;             // [lam * ngroups] blocks that the group can reach: bx0, by0, bx1, by1 (bx0 > bx1: none)
+    uint32_t *active;         // [lam * nby * wpr] bitmap of the listed blocks
+    int2 *items;              // [lam * nbx * nby] listed blocks: candidate, by << 16 | bx
+    int2 *units;              // [lam * ngroups * kBwdMaxSeg] backward units: candidate, group * kBwdMaxSeg + part
+    float *wp;                // [lam * nbx * nby * kBlkPx] 2 (S - M) (1 - S) / sigma of the listed blocks' pixels
+    unsigned *ctl;            // [5] blocks listed, forward ticket, forward exits, units listed, backward ticket
+    unsigned *rdone;          // [lam] finished blocks of k_soft_reduce
+    longlong2 *gv;            // [lam * nI * V]: dL/du, dL/dv in fixed point (units of 2^-36)
+    unsigned long long *G;    // [lam * nI * nF * 12][2] fixed point, units of 2^-24 and of 2^-56
+    unsigned long long *lsum; // [lam] loss in fixed point, units of 2^-32
     float *loss;              // [lam]
     float *grad;              // [lam * d] or NULL
 };
 
-__global__ void __launch_bounds__(kSoftThreads) k_soft_project(SoftArgs a)
+// Edge record of a drawable triangle, positively oriented, in image pixels: the
+// corners, the edges' unit directions and lengths, and
+// +1 / -1 for the mesh's corner order / the reverse (0: not drawn).
+struct TriRec {
+    float x[3], y[3], tx[3], ty[3], L[3], orient;
+};
+
+__device__ __forceinline__ TriRec load_rec(const SoftArgs &a, size_t i)
 {
-    const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    __shared__ float sT[kMaxFrames][12];
-    __shared__ int bx[4];
-    if (tid < 4) bx[tid] = (tid < 2) ? INT_MAX : INT_MIN;
+    const size_t n = (size_t)a.lam * a.NTp;
+    const float4 r0 = a.rec[i], r1 = a.rec[n + i], r2 = a.rec[2 * n + i], r3 = a.rec[3 * n + i];
+    TriRec r;
+    r.x[0] = r0.x; r.y[0] = r0.y; r.x[1] = r0.z; r.y[1] = r0.w;
+    r.x[2] = r1.x; r.y[2] = r1.y; r.tx[0] = r1.z; r.ty[0] = r1.w;
+    r.tx[1] = r2.x; r.ty[1] = r2.y; r.tx[2] = r2.z; r.ty[2] = r2.w;
+    r.L[0] = r3.x; r.L[1] = r3.y; r.L[2] = r3.z;
+    r.orient = r3.w;
+    return r;
+}
+
+// Kinematics of one instrument of one candidate on warp 0; meanwhile the other
+// warps clear the accumulators and count the mask (the loss starts at the
+// number of mask pixels: outside every triangle's reach S = 0 and the squared
+// error of a pixel is M).
+__global__ void __launch_bounds__(kSoftThreads) k_soft_fk(SoftArgs a)
+{
+    const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    __shared__ int s_m;
+    if (tid == 0) s_m = 0;
+    __syncthreads();
+    const size_t cb = (size_t)c * a.nI + b;
     if (tid < 32) {
-        const int lane = tid, dir = lane - 1;
+        const int dir = lane - 1;
         float st[9];
         for (int k = 0; k < 9; ++k) st[k] = a.params[(size_t)c * a.d + 9 * b + k];
         float T[kMaxFrames][12], dT[kMaxFrames][12];
@@ -270,375 +324,592 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_project(SoftArgs a)
             fk_tangent(a.ch, st, dir, T, dT);
             if (lane == 0)
                 for (int f = 0; f < a.nF; ++f)
-                    for (int e = 0; e < 12; ++e) sT[f][e] = T[f][e];
+                    for (int e = 0; e < 12; ++e) a.Tf[(cb * a.nF + f) * 12 + e] = T[f][e];
             else
                 for (int f = 0; f < a.nF; ++f)
-                    for (int e = 0; e < 12; ++e)
-                        a.dT[((((size_t)c * a.nI + b) * a.nF + f) * 9 + dir) * 12 + e] = dT[f][e];
+                    for (int e = 0; e < 12; ++e) a.dT[((cb * a.nF + f) * 9 + dir) * 12 + e] = dT[f][e];
+        }
+    } else {
+        const int t = tid - 32, nt = kSoftThreads - 32;
+        if (c == 0 && b == 0 && t < 5) a.ctl[t] = 0u;
+        if (b == 0) {
+            uint32_t *act = a.active + (size_t)c * a.nby * a.wpr;
+            for (int i = t; i < a.nby * a.wpr; i += nt) act[i] = 0u;
+            int m = 0;
+            for (int i = t; i < a.H * a.Wq; i += nt) m += __popc(a.mask[i]);
+            m = __reduce_add_sync(0xffffffffu, m);
+            if (lane == 0) atomicAdd(&s_m, m);
+            if (t == 0) a.rdone[c] = 0u;
+        }
+        if (a.grad) {
+            for (int v = t; v < a.V; v += nt) a.gv[cb * a.V + v] = make_longlong2(0, 0);
+            for (int e = t; e < a.nF * 24; e += nt) a.G[cb * a.nF * 24 + e] = 0ull;
         }
     }
     __syncthreads();
-    const float m = kSoftCutoff * a.sigma;
-    int j0 = INT_MAX, i0 = INT_MAX, j1 = INT_MIN, i1 = INT_MIN;
-    const size_t base = ((size_t)c * a.nI + b) * a.V;
-    for (int v = tid; v < a.V; v += blockDim.x) {
-        const float4 p = a.verts[v];
-        const float *M = sT[(int)p.w];
-        const float X = fmaf(M[0], p.x, fmaf(M[1], p.y, fmaf(M[2], p.z, M[3])));
-        const float Y = fmaf(M[4], p.x, fmaf(M[5], p.y, fmaf(M[6], p.z, M[7])));
-        const float Z = fmaf(M[8], p.x, fmaf(M[9], p.y, fmaf(M[10], p.z, M[11])));
-        float u = 0.0f, w = 0.0f, flag = 1.0f;
-        if (Z >= a.z_near) {
-            u = __fdiv_rn(a.fx * X, Z);
-            w = __fdiv_rn(a.fy * Y, Z);
-            if (fabsf(u) <= a.guard && fabsf(w) <= a.guard) {
-                flag = 0.0f;
-                j0 = min(j0, (int)ceilf(u + a.cx - m));
-                j1 = max(j1, (int)floorf(u + a.cx + m));
-                i0 = min(i0, (int)ceilf(w + a.cy - m));
-                i1 = max(i1, (int)floorf(w + a.cy + m));
-            }
-        }
-        a.sv[base + v] = make_float4(u, w, Z, flag);
-        a.gv[base + v] = make_longlong2(0, 0);
-    }
-    atomicMin(&bx[0], j0);
-    atomicMin(&bx[1], i0);
-    atomicMax(&bx[2], j1);
-    atomicMax(&bx[3], i1);
-    __syncthreads();
-    if (tid == 0)
-        a.ibox[(size_t)c * a.nI + b] = make_int4(max(bx[0], 0), max(bx[1], 0), min(bx[2], a.W - 1), min(bx[3], a.H - 1));
+    if (b == 0 && tid == 0) a.lsum[c] = (unsigned long long)s_m << 32;
 }
 
-// Window of influence of every triangle (none for a flagged vertex or zero
-// area), and the union of the windows of each chunk of kChunk triangles (one
-// block per chunk), so that a tile skips whole chunks that cannot reach it.
-__global__ void __launch_bounds__(kChunk) k_soft_tribox(SoftArgs a)
+// Projection of a mesh vertex: (u - cx, v - cy, Z, flag).  Explicit roundings:
+// the kernels that call it get the same bits.
+__device__ __forceinline__ float4 soft_project(const SoftArgs &a, const float *M, float4 p)
 {
-    const int c = blockIdx.y;
-    const int NT = a.nI * a.T;
-    const int t = blockIdx.x * kChunk + threadIdx.x;
-    __shared__ int cb[4];
-    if (threadIdx.x < 4) cb[threadIdx.x] = (threadIdx.x < 2) ? INT_MAX : INT_MIN;
+    const float X = __fmaf_rn(M[0], p.x, __fmaf_rn(M[1], p.y, __fmaf_rn(M[2], p.z, M[3])));
+    const float Y = __fmaf_rn(M[4], p.x, __fmaf_rn(M[5], p.y, __fmaf_rn(M[6], p.z, M[7])));
+    const float Z = __fmaf_rn(M[8], p.x, __fmaf_rn(M[9], p.y, __fmaf_rn(M[10], p.z, M[11])));
+    float4 o = make_float4(0.0f, 0.0f, Z, 1.0f);
+    if (Z >= a.z_near) {
+        o.x = __fdiv_rn(__fmul_rn(a.fx, X), Z);
+        o.y = __fdiv_rn(__fmul_rn(a.fy, Y), Z);
+        if (fabsf(o.x) <= a.guard && fabsf(o.y) <= a.guard) o.w = 0.0f;
+    }
+    return o;
+}
+
+__device__ __forceinline__ int bwd_segments(int blocks) { return min(kBwdMaxSeg, (blocks + kBwdSeg - 1) / kBwdSeg); }
+
+// A warp per group of 32 triangles.  Every lane projects its triangle's three
+// corners itself: cheaper than a pass of its own over the vertices and a gather.
+__global__ void __launch_bounds__(kSoftThreads) k_soft_tris(SoftArgs a)
+{
+    const int c = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    extern __shared__ float sT[];  // [nI * nF * 12]
+    for (int e = tid; e < a.nI * a.nF * 12; e += kSoftThreads) sT[e] = a.Tf[(size_t)c * a.nI * a.nF * 12 + e];
     __syncthreads();
-    short4 o = make_short4(1, 1, 0, 0);
-    if (t < NT) {
+    const int g = blockIdx.x * (kSoftThreads / 32) + (tid >> 5);
+    if (g >= a.ngroups) return;
+    const int t = g * 32 + lane;
+    const size_t ti = (size_t)c * a.NTp + t;
+    float lox = INFINITY, loy = INFINITY, hix = -INFINITY, hiy = -INFINITY;
+    float4 bx4 = make_float4(INFINITY, INFINITY, 0.0f, 0.0f);  // no block is near
+    if (t < a.nI * a.T) {
         const int b = t >= a.T;
         const int4 tri = a.tris[t - b * a.T];
-        const float4 *sv = a.sv + ((size_t)c * a.nI + b) * a.V;
-        const float4 p0 = sv[tri.x], p1 = sv[tri.y], p2 = sv[tri.z];
-        if (p0.w == 0.0f && p1.w == 0.0f && p2.w == 0.0f) {
-            const float A = (p1.x - p0.x) * (p2.y - p0.y) - (p1.y - p0.y) * (p2.x - p0.x);
-            if (A != 0.0f) {
-                const float m = kSoftCutoff * a.sigma;
-                const int j0 = max(0, (int)ceilf(fminf(p0.x, fminf(p1.x, p2.x)) + a.cx - m));
-                const int j1 = min(a.W - 1, (int)floorf(fmaxf(p0.x, fmaxf(p1.x, p2.x)) + a.cx + m));
-                const int i0 = max(0, (int)ceilf(fminf(p0.y, fminf(p1.y, p2.y)) + a.cy - m));
-                const int i1 = min(a.H - 1, (int)floorf(fmaxf(p0.y, fmaxf(p1.y, p2.y)) + a.cy + m));
-                if (j0 <= j1 && i0 <= i1) {
-                    o = make_short4((short)j0, (short)i0, (short)j1, (short)i1);
-                    atomicMin(&cb[0], j0);
-                    atomicMin(&cb[1], i0);
-                    atomicMax(&cb[2], j1);
-                    atomicMax(&cb[3], i1);
-                }
+        const float4 w0 = a.verts[tri.x], w1 = a.verts[tri.y], w2 = a.verts[tri.z];
+        const float *M = sT + b * a.nF * 12;
+        const float4 p0 = soft_project(a, M + 12 * (int)w0.w, w0), p1 = soft_project(a, M + 12 * (int)w1.w, w1),
+                     p2 = soft_project(a, M + 12 * (int)w2.w, w2);
+        const float A = (p1.x - p0.x) * (p2.y - p0.y) - (p1.y - p0.y) * (p2.x - p0.x);
+        if (p0.w == 0.0f && p1.w == 0.0f && p2.w == 0.0f && A != 0.0f) {
+            float x[3] = {p0.x, A > 0.0f ? p1.x : p2.x, A > 0.0f ? p2.x : p1.x};
+            float y[3] = {p0.y, A > 0.0f ? p1.y : p2.y, A > 0.0f ? p2.y : p1.y};
+            float tx[3], ty[3], L[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int k1 = k == 2 ? 0 : k + 1;
+                const float dx = x[k1] - x[k], dy = y[k1] - y[k];
+                L[k] = __fsqrt_rn(fmaf(dx, dx, dy * dy));
+                const float il = L[k] > 0.0f ? __frcp_rn(L[k]) : 0.0f;
+                tx[k] = dx * il;
+                ty[k] = dy * il;
             }
+            const size_t n = (size_t)a.lam * a.NTp;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {  // the edges come from the offsets, unrounded by the shift
+                x[k] += a.cx;
+                y[k] += a.cy;
+            }
+            a.rec[ti] = make_float4(x[0], y[0], x[1], y[1]);
+            a.rec[n + ti] = make_float4(x[2], y[2], tx[0], ty[0]);
+            a.rec[2 * n + ti] = make_float4(tx[1], ty[1], tx[2], ty[2]);
+            a.rec[3 * n + ti] = make_float4(L[0], L[1], L[2], A > 0.0f ? 1.0f : -1.0f);
+            lox = fminf(x[0], fminf(x[1], x[2]));
+            hix = fmaxf(x[0], fmaxf(x[1], x[2]));
+            loy = fminf(y[0], fminf(y[1], y[2]));
+            hiy = fmaxf(y[0], fmaxf(y[1], y[2]));
+            bx4 = make_float4(0.5f * (lox + hix), 0.5f * (loy + hiy), 0.5f * (hix - lox), 0.5f * (hiy - loy));
         }
-        a.box[(size_t)c * NT + t] = o;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) a.cbox[(size_t)c * a.nchunk + blockIdx.x] = make_int4(cb[0], cb[1], cb[2], cb[3]);
+    a.box[ti] = bx4;
+    for (int o = 16; o; o >>= 1) {
+        lox = fminf(lox, __shfl_xor_sync(0xffffffffu, lox, o));
+        loy = fminf(loy, __shfl_xor_sync(0xffffffffu, loy, o));
+        hix = fmaxf(hix, __shfl_xor_sync(0xffffffffu, hix, o));
+        hiy = fmaxf(hiy, __shfl_xor_sync(0xffffffffu, hiy, o));
+    }
+    short4 win = make_short4(1, 1, 0, 0);
+    if (lox <= hix) {
+        const float m = kSoftCutoff * a.sigma;
+        const int j0 = max(0, (int)floorf(lox - m)), j1 = min(a.W - 1, (int)ceilf(hix + m));
+        const int i0 = max(0, (int)floorf(loy - m)), i1 = min(a.H - 1, (int)ceilf(hiy + m));
+        if (j0 <= j1 && i0 <= i1)
+            win = make_short4((short)(j0 / kBlkW), (short)(i0 / kBlkH), (short)(j1 / kBlkW), (short)(i1 / kBlkH));
+    }
+    if (lane == 0) a.gwin[(size_t)c * a.ngroups + g] = win;
+    if (win.x > win.z) return;
+    // list the blocks of the window that no group has listed yet
+    const int w0 = win.x >> 5, nw = (win.z >> 5) - w0 + 1, rows = win.w - win.y + 1;
+    for (int e = lane; e < rows * nw; e += 32) {
+        const int by = win.y + e / nw, w = w0 + e % nw;
+        uint32_t need = 0xffffffffu;
+        if (w == w0) need &= 0xffffffffu << (win.x & 31);
+        if (w == (win.z >> 5)) need &= 0xffffffffu >> (31 - (win.z & 31));
+        uint32_t *word = a.active + ((size_t)c * a.nby + by) * a.wpr + w;
+        need &= ~__ldcg(word);
+        if (!need) continue;
+        uint32_t neu = need & ~atomicOr(word, need);
+        if (!neu) continue;
+        unsigned at = atomicAdd(&a.ctl[0], (unsigned)__popc(neu));
+        for (; neu; neu &= neu - 1) a.items[at++] = make_int2(c, by << 16 | (w * 32 + __ffs(neu) - 1));
+    }
+    if (a.grad) {
+        const int ns = bwd_segments(rows * (win.z - win.x + 1));
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&a.ctl[3], (unsigned)ns);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (lane < ns) a.units[at + lane] = make_int2(c, g * kBwdMaxSeg + lane);
+    }
 }
 
-// Staged triangle: positively oriented image-space vertices, edge data, window.
-struct SoftTriSmem {
-    float x[3][kChunk], y[3][kChunk];
-    float ex[3][kChunk], ey[3][kChunk], il[3][kChunk], il2[3][kChunk];
-    short4 win[kChunk];
-    int vid[3][kChunk];     // global vertex slots (into sv / gv)
-    int list[kChunk];
-    int wc[kChunk / 32];    // staged triangles per warp (the compaction's prefix)
-    int n;
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float ex2(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsq(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// |x| with the sign of s
+__device__ __forceinline__ float with_sign(float x, float s)
+{
+    return __uint_as_float(__float_as_uint(x) | (__float_as_uint(s) & 0x80000000u));
+}
+
+// Does the triangle's bounding box come within the cutoff of block (bx, by)?
+__device__ __forceinline__ bool box_near(float4 b, int bx, int by, float reach2)
+{
+    const float x = (float)(bx * kBlkW) + 0.5f * (kBlkW - 1), y = (float)(by * kBlkH) + 0.5f * (kBlkH - 1);
+    const float dx = fmaxf(fabsf(b.x - x) - (b.z + 0.5f * (kBlkW - 1)), 0.0f);
+    const float dy = fmaxf(fabsf(b.y - y) - (b.w + 0.5f * (kBlkH - 1)), 0.0f);
+    return fmaf(dx, dx, dy * dy) <= reach2;
+}
+
+// The edges of a triangle seen from a block: coordinates of the block's first
+// pixel along (a) and across (b, positive inside) each edge and the steps to
+// the next pixel, all in units of sigma / log2(e), so that 2^distance is the
+// sigmoid's exponential.
+struct BlockEdges {
+    float a[3], b[3], tx[3], ty[3], L[3];
 };
 
-// Signed distance of (px, py) to staged triangle n (FP32), with the feature
-// that realises it: kind 0 = edge line (inside) or segment interior
-// (outside), 1 = segment start vertex, 2 = segment end vertex; k = edge.
-__device__ __forceinline__ float soft_distance(const SoftTriSmem &S, int n, float px, float py, int &kind, int &kf)
+__device__ __forceinline__ BlockEdges block_edges(const TriRec &r, int bx, int by, float k)
 {
-    bool inside = true;
-    float hmin = INFINITY, dmin = INFINITY;
-    int kin = 0, kout = 0, kindout = 0;
+    const float X = (float)(bx * kBlkW), Y = (float)(by * kBlkH);
+    BlockEdges e;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float x0 = S.x[k][n], y0 = S.y[k][n], dx = S.ex[k][n], dy = S.ey[k][n];
-        const float rx = px - x0, ry = py - y0;
-        const float E = fmaf(dx, ry, -dy * rx);
-        const float h = E * S.il[k][n];
-        if (E < 0.0f) inside = false;
-        if (h < hmin) {
-            hmin = h;
-            kin = k;
-        }
-        const float s = fmaf(rx, dx, ry * dy) * S.il2[k][n];
-        float dist;
-        int kd;
-        if (s <= 0.0f) {
-            dist = sqrtf(fmaf(rx, rx, ry * ry));
-            kd = 1;
-        } else if (s >= 1.0f) {
-            const float qx = px - (x0 + dx), qy = py - (y0 + dy);
-            dist = sqrtf(fmaf(qx, qx, qy * qy));
-            kd = 2;
-        } else {
-            dist = fabsf(h);
-            kd = 0;
-        }
-        if (dist < dmin) {
-            dmin = dist;
-            kout = k;
-            kindout = kd;
-        }
+    for (int q = 0; q < 3; ++q) {
+        const float rx = X - r.x[q], ry = Y - r.y[q];
+        e.tx[q] = r.tx[q] * k;
+        e.ty[q] = r.ty[q] * k;
+        e.L[q] = r.L[q] * k;
+        e.a[q] = fmaf(rx, e.tx[q], ry * e.ty[q]);
+        e.b[q] = fmaf(ry, e.tx[q], -rx * e.ty[q]);
     }
-    if (inside) {
-        kind = 0;
-        kf = kin;
-        return hmin;
-    }
-    kind = kindout;
-    kf = kout;
-    return -dmin;
+    return e;
 }
 
-__device__ __forceinline__ float softplusf(float x) { return fmaxf(x, 0.0f) + log1pf(__expf(-fabsf(x))); }
-__device__ __forceinline__ float sigmoidf_(float x)
-{
-    const float e = __expf(-fabsf(x));
-    return x >= 0.0f ? 1.0f / (1.0f + e) : e / (1.0f + e);
-}
+// log2-scaled cutoff and unit of the distances
+constexpr float kLog2e = 1.44269504089f;
+constexpr float kCutLog2 = -kSoftCutoff * kLog2e;
 
-// Stage the triangles of chunk [t0, t0 + kChunk) whose window meets the tile,
-// in triangle order (a fixed order, so every sum over the staged triangles is
-// the same from run to run).
-__device__ void stage_chunk(const SoftArgs &a, int c, int t0, int tx0, int ty0, SoftTriSmem &S)
+// The product over one batch of triangles (one per lane) into the lane's 32
+// running products Q (1 + Q = product of 1 + exp(d / sigma)).  Per pixel: the
+// point's coordinates (a, b) in the three edge frames, the squared distance
+// b^2 + max(a - L, -a, 0)^2 to each edge, its minimum, the sign from the
+// smallest b (inside: every b >= 0, and there the nearest edge's line is
+// nearest at the edge), and one exponential.
+__device__ __forceinline__ void fwd_batch(BlockEdges &e, float (&Q)[kBlkPx])
 {
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int NT = a.nI * a.T;
-    const int t = t0 + tid;
-    bool hit = false;
-    short4 w = make_short4(1, 1, 0, 0);
-    if (t < NT) {
-        w = a.box[(size_t)c * NT + t];
-        hit = w.x <= w.z && w.x <= tx0 + kTile - 1 && w.z >= tx0 && w.y <= ty0 + kTile - 1 && w.w >= ty0;
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-    if ((tid & 31) == 0) S.wc[warp] = __popc(bal);
-    __syncthreads();
-    int base = 0;
-    for (int q = 0; q < warp; ++q) base += S.wc[q];
-    if (tid == 0) {
-        int n = 0;
-        for (int q = 0; q < kChunk / 32; ++q) n += S.wc[q];
-        S.n = n;
-    }
-    if (hit) {
-        const int slot = base + __popc(bal & ((1u << (tid & 31)) - 1u));
-        const int b = t >= a.T;
-        const int4 tri = a.tris[t - b * a.T];
-        const size_t vb = ((size_t)c * a.nI + b) * a.V;
-        const float4 p0 = a.sv[vb + tri.x], p1 = a.sv[vb + tri.y], p2 = a.sv[vb + tri.z];
-        const float A = (p1.x - p0.x) * (p2.y - p0.y) - (p1.y - p0.y) * (p2.x - p0.x);
-        float4 q[3] = {p0, A > 0.0f ? p1 : p2, A > 0.0f ? p2 : p1};
-        int id[3] = {tri.x, A > 0.0f ? tri.y : tri.z, A > 0.0f ? tri.z : tri.y};
+#pragma unroll
+    for (int py = 0; py < kBlkH; ++py) {
+#pragma unroll
+        for (int px = 0; px < kBlkW; ++px) {
+            float d2[3], bb[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float av = fmaf((float)px, e.tx[k], e.a[k]);
+                bb[k] = fmaf(-(float)px, e.ty[k], e.b[k]);
+                const float o = max3(av - e.L[k], -av, 0.0f);
+                d2[k] = fmaf(o, o, bb[k] * bb[k]);
+            }
+            const float m2 = fmaxf(min3(d2[0], d2[1], d2[2]), 1e-30f);
+            const float dist = fminf(m2 * rsq(m2), 64.0f);  // 2^64 saturates the pixel; no infinity enters the product
+            const float x = with_sign(dist, min3(bb[0], bb[1], bb[2]));
+            const float p = ex2(x);
+            float &q = Q[py * kBlkW + px];
+            if (x >= kCutLog2) q = fmaf(q, p, q + p);
+        }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            S.x[k][slot] = q[k].x + a.cx;
-            S.y[k][slot] = q[k].y + a.cy;
-            S.vid[k][slot] = (int)(vb + id[k]);
+            e.a[k] += e.ty[k];
+            e.b[k] += e.tx[k];
         }
+    }
+}
+
+// The lanes' products multiplied together: returns pixel `lane`'s.
+__device__ __forceinline__ float combine_lanes(const float (&Q)[kBlkPx], int lane)
+{
+    float v[16];
+    {
+        const bool up = lane & 16;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float mine = up ? Q[i + 16] : Q[i], give = up ? Q[i] : Q[i + 16];
+            const float got = __shfl_xor_sync(0xffffffffu, give, 16);
+            v[i] = fmaf(mine, got, mine + got);
+        }
+    }
+#pragma unroll
+    for (int s = 8; s; s >>= 1) {
+        const bool up = lane & s;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < s) {
+                const float mine = up ? v[i + s] : v[i], give = up ? v[i] : v[i + s];
+                const float got = __shfl_xor_sync(0xffffffffu, give, s);
+                v[i] = fmaf(mine, got, mine + got);
+            }
+    }
+    return v[0];
+}
+
+// Bound by instruction issue (67-82 % of the cycles; about 30 instructions per
+// 32 pairs).  640x512, 20k triangles, 64 candidates: 1.9 ms, where a pixel per
+// thread with the triangles in shared memory (four 16-byte reads, a branchy
+// distance of about 180 instructions and a log1p per pair) took 12 ms.
+// Persistent blocks over the listed pixel blocks.  The warps of a block share
+// the triangles of its pixel block group by group (group g belongs to warp
+// g mod warps); each warp collects the triangles that come near into full
+// batches of 32.  Every kCheck batches a warp looks whether the pixels are
+// saturated (see kSaturated) by its own products and the last ones the other
+// warps left in shared memory: those only grow, so a decision made on them
+// holds, and the results do not depend on when it is made.
+__global__ void __launch_bounds__(32 * kFwdWarps) k_soft_fwd(SoftArgs a)
+{
+    constexpr int kCheck = 6;
+    __shared__ int queue[kFwdWarps][64];
+    __shared__ float part[kFwdWarps][kBlkPx];
+    __shared__ int s_it;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const float k2 = kLog2e / a.sigma, inv_s = 1.0f / a.sigma;
+    const float reach = kSoftCutoff * a.sigma + 0.01f, reach2 = reach * reach;
+    const int n_items = (int)a.ctl[0];
+    int *qu = queue[warp];
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_it = (int)atomicAdd(&a.ctl[1], 1u);
+        part[warp][lane] = 0.0f;
+        __syncthreads();
+        if (s_it >= n_items) break;
+        const int2 it = a.items[s_it];
+        const int c = it.x, bx = it.y & 0xffff, by = it.y >> 16;
+        const short4 *gw = a.gwin + (size_t)c * a.ngroups;
+        const size_t tb = (size_t)c * a.NTp;
+        const int j = bx * kBlkW + (lane & (kBlkW - 1)), i = by * kBlkH + lane / kBlkW;
+        const bool on = j < a.W && i < a.H;
+        float Q[kBlkPx];
+#pragma unroll
+        for (int p = 0; p < kBlkPx; ++p) Q[p] = 0.0f;
+        int qn = 0, g0 = warp, batches = 0;
+        unsigned hits = 0;
+        int gb = 0;
+        for (;;) {
+            while (qn < 32) {
+                if (!hits) {
+                    if (g0 >= a.ngroups) break;
+                    gb = g0;
+                    const int g = gb + lane * nw;
+                    bool h = false;
+                    if (g < a.ngroups) {
+                        const short4 w = gw[g];
+                        h = w.x <= bx && bx <= w.z && w.y <= by && by <= w.w;
+                    }
+                    hits = __ballot_sync(0xffffffffu, h);
+                    g0 += 32 * nw;
+                    continue;
+                }
+                const int g = gb + (__ffs(hits) - 1) * nw;
+                hits &= hits - 1;
+                const int t = g * 32 + lane;
+                const bool h = box_near(a.box[tb + t], bx, by, reach2);
+                const unsigned m = __ballot_sync(0xffffffffu, h);
+                if (h) qu[qn + __popc(m & ((1u << lane) - 1u))] = t;
+                qn += __popc(m);
+            }
+            if (qn == 0) break;
+            __syncwarp();
+            // the last (up to) 32 of the queue, one per lane
+            const int n = min(qn, 32);
+            qn -= n;
+            BlockEdges e;
+            if (lane < n) {
+                e = block_edges(load_rec(a, tb + qu[qn + lane]), bx, by, k2);
+            } else {  // no triangle: far outside
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    e.a[k] = 0.0f;
+                    e.b[k] = -1e4f;
+                    e.tx[k] = e.ty[k] = e.L[k] = 0.0f;
+                }
+            }
+            __syncwarp();
+            fwd_batch(e, Q);
+            if (++batches % kCheck == 0) {
+                float q = combine_lanes(Q, lane);
+                part[warp][lane] = q;
+                volatile float(*pv)[kBlkPx] = part;
+                for (int w = 0; w < nw; ++w)
+                    if (w != warp) {
+                        const float o = pv[w][lane];
+                        q = fmaf(q, o, q + o);
+                    }
+                if (__all_sync(0xffffffffu, !on || q >= kSaturated)) break;
+            }
+        }
+        part[warp][lane] = combine_lanes(Q, lane);
+        __syncthreads();
+        if (warp == 0) {
+            float q = part[0][lane];
+            for (int w = 1; w < nw; ++w) {
+                const float o = part[w][lane];
+                q = fmaf(q, o, q + o);
+            }
+            float l = 0.0f, wpx = 0.0f;
+            const bool mv = on && ((a.mask[(size_t)i * a.Wq + (j >> 5)] >> (j & 31)) & 1u);
+            if (on) {
+                const bool sat = q >= kOne;
+                const float om = sat ? 0.0f : __frcp_rn(1.0f + q);  // 1 - S
+                const float S = sat ? 1.0f : q * om;
+                const float e = mv ? -om : S;
+                l = e * e;
+                wpx = 2.0f * e * om * inv_s;
+            }
+            if (a.grad) a.wp[(((size_t)c * a.nby + by) * a.nbx + bx) * kBlkPx + lane] = wpx;
+            const int m = __popc(__ballot_sync(0xffffffffu, mv));
+            for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+            if (lane == 0)  // squared error minus the mask pixels counted in advance: exact sums, in any order
+                atomicAdd(a.lsum + c, (unsigned long long)__double2ll_rn((double)l * kLossScale) -
+                                          ((unsigned long long)m << 32));
+        }
+    }
+    // the last block to run out of work writes the losses
+    if (tid == 0) {
+        __threadfence();
+        s_it = atomicAdd(&a.ctl[2], 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_it) {
+        __threadfence();
+        for (int c = tid; c < a.lam; c += blockDim.x)
+            a.loss[c] = (float)((double)(long long)__ldcg(a.lsum + c) * (1.0 / kLossScale));
+    }
+}
+
+// dL/d(u, v) of a group's triangles over a part of the group's window, one
+// triangle per lane.  With c the closest boundary point, at parameter t of edge
+// k, the signed distance d changes with c by -(p - c) / d, and c follows the
+// edge's ends by 1 - t and t.  The sums are kept in the edges' frames: Wb and
+// Wt for the part across the edge (all of it, and weighted by the position
+// along the edge), U0 and U1 for the part along it (only beyond an end).
+// Bound by instruction issue (82 %): 5.6 ms at 640x512, 20k triangles, 64
+// candidates (a warp per triangle and tile with its lanes on the pixels, six
+// values reduced over the warp for each: 24 ms, the forward again included).
+struct EdgeSums {
+    float U0[3], U1[3], Wb[3], Wt[3];
+};
+
+__device__ __forceinline__ void bwd_pixel(const BlockEdges &e, const float (&ar)[3], const float (&br)[3], int px,
+                                          float w, EdgeSums &s)
+{
+    float d2[3], bb[3], lo[3], hi[3], av[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        av[k] = fmaf((float)px, e.tx[k], ar[k]);
+        bb[k] = fmaf(-(float)px, e.ty[k], br[k]);
+        lo[k] = fminf(av[k], 0.0f);
+        hi[k] = fmaxf(av[k] - e.L[k], 0.0f);
+        d2[k] = fmaf(bb[k], bb[k], fmaf(lo[k], lo[k], hi[k] * hi[k]));
+    }
+    const float m2 = min3(d2[0], d2[1], d2[2]);
+    const bool k0 = d2[0] == m2, k1 = !k0 && d2[1] == m2;
+    const float m2c = fmaxf(m2, 1e-30f), ir = rsq(m2c);
+    const float mb = min3(bb[0], bb[1], bb[2]);
+    const float x = with_sign(m2c * ir, mb);
+    const float sg = rcp_(1.0f + ex2(-x));
+    // outside: d = -|p - c|, the sum grows along p - c; inside the other way
+    float g = __uint_as_float(__float_as_uint(w * sg * ir) ^ (~__float_as_uint(mb) & 0x80000000u));
+    g = x >= kCutLog2 ? g : 0.0f;
+    const float gk[3] = {k0 ? g : 0.0f, k1 ? g : 0.0f, (k0 || k1) ? 0.0f : g};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        s.U0[k] = fmaf(gk[k], lo[k], s.U0[k]);
+        s.U1[k] = fmaf(gk[k], hi[k], s.U1[k]);
+        const float h = gk[k] * bb[k];
+        s.Wb[k] += h;
+        s.Wt[k] = fmaf(h, av[k] - lo[k] - hi[k], s.Wt[k]);
+    }
+}
+
+__global__ void __launch_bounds__(128) k_soft_bwd(SoftArgs a)
+{
+    const int lane = threadIdx.x & 31;
+    const float k2 = kLog2e / a.sigma;
+    const float reach = kSoftCutoff * a.sigma + 0.01f, reach2 = reach * reach;
+    const int n_units = (int)a.ctl[3];
+    for (;;) {  // a warp per unit
+        int u = 0;
+        if (lane == 0) u = (int)atomicAdd(&a.ctl[4], 1u);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (u >= n_units) return;
+        const int2 un = a.units[u];
+        const int c = un.x, g = un.y / kBwdMaxSeg, seg = un.y % kBwdMaxSeg;
+        const short4 win = a.gwin[(size_t)c * a.ngroups + g];
+        const int bw = win.z - win.x + 1, nb = bw * (win.w - win.y + 1), ns = bwd_segments(nb);
+        const int per = (nb + ns - 1) / ns, q1 = min(nb, (seg + 1) * per);
+        const int t = g * 32 + lane;
+        const size_t ti = (size_t)c * a.NTp + t;
+        const float4 box = a.box[ti];
+        const bool drawn = box.x < INFINITY;
+        TriRec r;
+        if (drawn) {
+            r = load_rec(a, ti);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) r.x[k] = r.y[k] = 1e5f, r.tx[k] = r.ty[k] = r.L[k] = 0.0f;
+            r.orient = 0.0f;
+        }
+        EdgeSums tot{};
+        bool any = false;
+        for (int q = seg * per; q < q1; ++q) {
+            const int by = win.y + q / bw, bx = win.x + q % bw;
+            const bool near = drawn && box_near(box, bx, by, reach2);
+            if (!__any_sync(0xffffffffu, near)) continue;
+            const float wl = a.wp[(((size_t)c * a.nby + by) * a.nbx + bx) * kBlkPx + lane];
+            const unsigned nz = __ballot_sync(0xffffffffu, wl != 0.0f);
+            if (!nz) continue;
+            any = true;
+            BlockEdges e = block_edges(r, bx, by, k2);
+            if (!near) {  // out of reach of this block (or not drawn): far outside
+#pragma unroll
+                for (int k = 0; k < 3; ++k) e.b[k] = -1e4f, e.tx[k] = e.ty[k] = 0.0f;
+            }
+            EdgeSums s{};
+            for (int py = 0; py < kBlkH; ++py) {
+                const unsigned row = (nz >> (kBlkW * py)) & ((1u << kBlkW) - 1u);
+                if (row) {
+#pragma unroll
+                    for (int px = 0; px < kBlkW; ++px)
+                        if (row >> px & 1u)
+                            bwd_pixel(e, e.a, e.b, px, __shfl_sync(0xffffffffu, wl, kBlkW * py + px), s);
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    e.a[k] += e.ty[k];
+                    e.b[k] += e.tx[k];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                tot.U0[k] += s.U0[k];
+                tot.U1[k] += s.U1[k];
+                tot.Wb[k] += s.Wb[k];
+                tot.Wt[k] += s.Wt[k];
+            }
+        }
+        if (!any || !drawn) continue;
+        float gx[3] = {0.0f, 0.0f, 0.0f}, gy[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int k1 = k == 2 ? 0 : k + 1;
-            const float dx = q[k1].x - q[k].x, dy = q[k1].y - q[k].y;
-            const float L2 = fmaf(dx, dx, dy * dy);
-            S.ex[k][slot] = dx;
-            S.ey[k][slot] = dy;
-            S.il2[k][slot] = 1.0f / L2;
-            S.il[k][slot] = rsqrtf(L2);
+            const float iL = r.L[k] > 0.0f ? 1.0f / (r.L[k] * k2) : 0.0f;
+            const float b1 = tot.Wt[k] * iL, b0 = tot.Wb[k] - b1;
+            gx[k] += r.tx[k] * tot.U0[k] - r.ty[k] * b0;
+            gy[k] += r.ty[k] * tot.U0[k] + r.tx[k] * b0;
+            gx[k1] += r.tx[k] * tot.U1[k] - r.ty[k] * b1;
+            gy[k1] += r.ty[k] * tot.U1[k] + r.tx[k] * b1;
         }
-        S.win[slot] = w;
-    }
-    __syncthreads();
-}
-
-// Does chunk k of candidate c have a window reaching the tile?
-__device__ __forceinline__ bool chunk_reaches(const SoftArgs &a, int c, int k, int tx0, int ty0)
-{
-    const int4 b = a.cbox[(size_t)c * a.nchunk + k];
-    return b.x <= b.z && b.x <= tx0 + kTile - 1 && b.z >= tx0 && b.y <= ty0 + kTile - 1 && b.w >= ty0;
-}
-
-__global__ void __launch_bounds__(kSoftThreads) k_soft_tile(SoftArgs a)
-{
-    const int c = blockIdx.y;
-    const int tile = blockIdx.x;
-    const int tx0 = (tile % a.ntx) * kTile, ty0 = (tile / a.ntx) * kTile;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ SoftTriSmem S;
-    __shared__ float wpx[kTile * kTile];
-    __shared__ float red[8];
-    // this thread's pixel in the forward pass
-    const int j = tx0 + (tid & (kTile - 1)), i = ty0 + tid / kTile;
-    const float px = (float)j, py = (float)i, inv_s = 1.0f / a.sigma, cut = -kSoftCutoff * a.sigma;
-    float acc = 0.0f;
-    // is the tile within reach of any instrument?
-    bool near = false;
-    for (int b = 0; b < a.nI; ++b) {
-        const int4 ib = a.ibox[(size_t)c * a.nI + b];
-        near |= ib.x <= ib.z && ib.x <= tx0 + kTile - 1 && ib.z >= tx0 && ib.y <= ty0 + kTile - 1 && ib.w >= ty0;
-    }
-    if (near) {
-        for (int k = 0; k < a.nchunk; ++k) {
-            if (!chunk_reaches(a, c, k, tx0, ty0)) continue;  // the same decision in every thread
-            stage_chunk(a, c, k * kChunk, tx0, ty0, S);
-            const int n = S.n;
-            for (int e = 0; e < n; ++e) {
-                const short4 w = S.win[e];
-                if (j < w.x || j > w.z || i < w.y || i > w.w) continue;
-                int kind, kf;
-                const float d = soft_distance(S, e, px, py, kind, kf);
-                if (d >= cut) acc += softplusf(d * inv_s);
-            }
-            __syncthreads();
-        }
-    }
-    // squared error of the tile's pixels; per-pixel factor of the backward
-    float l = 0.0f, wp = 0.0f;
-    if (i < a.H && j < a.W) {
-        const float Sv = 1.0f - __expf(-acc);
-        const float Mv = (float)((a.mask[(size_t)i * a.Wq + (j >> 5)] >> (j & 31)) & 1u);
-        const float e = Sv - Mv;
-        l = e * e;
-        wp = 2.0f * e * (1.0f - Sv) * inv_s;
-    }
-    wpx[tid] = wp;
-    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (lane == 0) red[warp] = l;
-    __syncthreads();
-    if (tid == 0) {  // the tile's share, summed over the tiles in a fixed order by k_soft_reduce
-        double sum = 0.0;
-        for (int w = 0; w < 8; ++w) sum += (double)red[w];
-        a.lpart[(size_t)c * a.ntx * a.nty + tile] = sum;
-    }
-    if (!a.grad || !near) return;
-    // pass 2: the same pairs again, one warp per staged triangle, lanes over
-    // two rows of 16 pixels at a time
-    const int cj = tx0 + (lane & (kTile - 1)), rsub = lane / kTile;
-    const float cpx = (float)cj;
-    for (int k = 0; k < a.nchunk; ++k) {
-        if (!chunk_reaches(a, c, k, tx0, ty0)) continue;
-        stage_chunk(a, c, k * kChunk, tx0, ty0, S);
-        const int n = S.n;
-        for (int e = warp; e < n; e += 8) {
-            const short4 w = S.win[e];
-            float g[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            const bool colin = cj >= w.x && cj <= w.z && cj < a.W;
-            const int ia = max((int)w.y, ty0), ib = min((int)w.w, min(ty0 + kTile - 1, a.H - 1));
-            for (int i2 = ia + rsub; i2 <= ib; i2 += 2) {
-                if (!colin) break;
-                int kind, kf;
-                const float cpy = (float)i2;
-                const float d = soft_distance(S, e, cpx, cpy, kind, kf);
-                if (d < cut) continue;
-                const float gd = wpx[(i2 - ty0) * kTile + (cj - tx0)] * sigmoidf_(d * inv_s);
-                const int k1 = kf == 2 ? 0 : kf + 1;
-                const float x0 = S.x[kf][e], y0 = S.y[kf][e], dx = S.ex[kf][e], dy = S.ey[kf][e];
-                if (kind == 0) {
-                    // d = E / L (inside, or outside at the segment interior: d = -|E|/L = E/L there)
-                    const float E = fmaf(dx, cpy - y0, -dy * (cpx - x0));
-                    const float il = S.il[kf][e], il2 = S.il2[kf][e];
-                    const float h = E * il;
-                    float sg = 1.0f;
-                    if (d < 0.0f && E > 0.0f) sg = -1.0f;  // outside on the inner side of the line
-                    const float x1 = x0 + dx, y1 = y0 + dy;
-                    // d(E/L) = dE / L - (E / L^2) dL, dL = (-dx, -dy, dx, dy) / L
-                    g[2 * kf] += gd * sg * ((y1 - cpy) * il + h * dx * il2);
-                    g[2 * kf + 1] += gd * sg * ((cpx - x1) * il + h * dy * il2);
-                    g[2 * k1] += gd * sg * ((cpy - y0) * il - h * dx * il2);
-                    g[2 * k1 + 1] += gd * sg * (-(cpx - x0) * il - h * dy * il2);
-                } else {
-                    // d = -|p - v|: dd/dv = (p - v) / |p - v|
-                    const int kv = kind == 1 ? kf : k1;
-                    const float rx = cpx - S.x[kv][e], ry = cpy - S.y[kv][e];
-                    const float rl = rsqrtf(fmaxf(fmaf(rx, rx, ry * ry), 1e-30f));
-                    g[2 * kv] += gd * rx * rl;
-                    g[2 * kv + 1] += gd * ry * rl;
-                }
-            }
+        const int b = t >= a.T;
+        const int4 tri = a.tris[t - b * a.T];
+        const int id[3] = {tri.x, r.orient > 0.0f ? tri.y : tri.z, r.orient > 0.0f ? tri.z : tri.y};
 #pragma unroll
-            for (int q = 0; q < 6; ++q)
-                for (int o = 16; o; o >>= 1) g[q] += __shfl_xor_sync(0xffffffffu, g[q], o);
-            if (lane < 3) {  // fixed point: the sums do not depend on the order of the additions
-                unsigned long long *gp = reinterpret_cast<unsigned long long *>(a.gv + S.vid[lane][e]);
-                atomicAdd(gp, (unsigned long long)to_fixed(g[2 * lane], kGvScale));
-                atomicAdd(gp + 1, (unsigned long long)to_fixed(g[2 * lane + 1], kGvScale));
-            }
+        for (int k = 0; k < 3; ++k) {  // fixed point: the sums do not depend on the order of the additions
+            unsigned long long *gp =
+                reinterpret_cast<unsigned long long *>(a.gv + ((size_t)c * a.nI + b) * a.V + id[k]);
+            const long long vx = to_fixed(gx[k], kGvScale), vy = to_fixed(gy[k], kGvScale);
+            if (vx) atomicAdd(gp, (unsigned long long)vx);
+            if (vy) atomicAdd(gp + 1, (unsigned long long)vy);
         }
-        __syncthreads();
     }
 }
 
 // Per (candidate, instrument): dL/dX of every vertex, G_f = sum over the
-// frame's vertices of dL/dX [v; 1]^T, then dL/dtheta_k = sum_f <G_f, dT_f/dtheta_k>.
-// Block (c, 0) also sums the candidate's tile losses in a fixed order.  Every
-// sum is order-independent (fixed order, or exact fixed-point integers), so
-// a call's results do not vary from run to run.
+// frame's vertices of dL/dX [v; 1]^T; the candidate's last block contracts
+// dL/dtheta_k = sum_f <G_f, dT_f/dtheta_k>.  The sums are fixed-point integers,
+// so a call's results do not vary from run to run.  A warp takes 256
+// consecutive vertices (mostly of one frame: a link's vertices are
+// contiguous), eight per lane.
+constexpr int kRedVerts = 8;
+
 __global__ void __launch_bounds__(kSoftThreads) k_soft_reduce(SoftArgs a)
 {
-    const int c = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    __shared__ unsigned long long G[kMaxFrames * 12];  // fixed point, units of 2^-24
-    __shared__ double red[kSoftThreads];
-    if (b == 0) {
-        const int nt = a.ntx * a.nty;
-        double acc = 0.0;
-        for (int t = tid; t < nt; t += blockDim.x) acc += a.lpart[(size_t)c * nt + t];
-        red[tid] = acc;
-        __syncthreads();
-        for (int o = kSoftThreads / 2; o; o >>= 1) {
-            if (tid < o) red[tid] += red[tid + o];
-            __syncthreads();
-        }
-        if (tid == 0) a.loss[c] = (float)red[0];
-    }
-    if (!a.grad) return;
-    for (int e = tid; e < a.nF * 12; e += blockDim.x) G[e] = 0ull;
-    __syncthreads();
-    const size_t base = ((size_t)c * a.nI + b) * a.V;
-    // each thread sums its vertices' terms in registers while their frame stays
-    // the same (a link's vertices are contiguous), then adds them to G: the
-    // integer sums are exact, so grouping them changes nothing
-    long long acc[12];
+    const int c = blockIdx.y / a.nI, b = blockIdx.y % a.nI, tid = threadIdx.x, lane = tid & 31;
+    __shared__ int s_last;
+    const size_t cb = (size_t)c * a.nI + b;
+    const float *Tf = a.Tf + cb * a.nF * 12;
+    unsigned long long *G = a.G + cb * a.nF * 24;
+    long long acc[24];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = 0;
+    for (int k = 0; k < 24; ++k) acc[k] = 0;
     int fcur = -1;
     auto flush = [&]() {
         if (fcur < 0) return;
 #pragma unroll
-        for (int k = 0; k < 12; ++k)
-            if (acc[k]) atomicAdd(G + fcur * 12 + k, (unsigned long long)acc[k]);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = 0;
+        for (int k = 0; k < 24; ++k) {
+            if (acc[k]) atomicAdd(G + fcur * 24 + k, (unsigned long long)acc[k]);
+            acc[k] = 0;
+        }
     };
-    for (int v = tid; v < a.V; v += blockDim.x) {
-        const float4 s = a.sv[base + v];
-        const longlong2 q = a.gv[base + v];
-        if (s.w != 0.0f || (q.x == 0 && q.y == 0)) continue;
-        const float gx = (float)((double)q.x * (1.0 / kGvScale)), gy = (float)((double)q.y * (1.0 / kGvScale));
-        const float iz = 1.0f / s.z;
-        const float gX = gx * a.fx * iz, gY = gy * a.fy * iz, gZ = -(gx * s.x + gy * s.y) * iz;
+    auto add = [&](int k, float x) {  // the whole units and the rest, both exact
+        const float q = x * kGScale, h = rintf(q);
+        acc[2 * k] += __float2ll_rn(h);
+        acc[2 * k + 1] += __float2ll_rn((q - h) * kRestScale);
+    };
+    const int v0 = ((int)blockIdx.x * kSoftThreads + (tid & ~31)) * kRedVerts + lane;
+#pragma unroll
+    for (int q = 0; q < kRedVerts; ++q) {
+        const int v = v0 + 32 * q;
+        if (v >= a.V) break;
+        const longlong2 gq = a.gv[cb * a.V + v];
+        if (gq.x == 0 && gq.y == 0) continue;
         const float4 p = a.verts[v];
         const int f = (int)p.w;
+        const float4 s = soft_project(a, Tf + 12 * f, p);
+        const float gx = __ll2float_rn(gq.x) * (1.0f / kGvScale), gy = __ll2float_rn(gq.y) * (1.0f / kGvScale);
+        const float iz = 1.0f / s.z;
+        const float gX = gx * a.fx * iz, gY = gy * a.fy * iz, gZ = -(gx * s.x + gy * s.y) * iz;
         if (f != fcur) {
             flush();
             fcur = f;
@@ -646,24 +917,47 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_reduce(SoftArgs a)
         const float vh[4] = {p.x, p.y, p.z, 1.0f};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            acc[k] += to_fixed(gX * vh[k], kGScale);
-            acc[4 + k] += to_fixed(gY * vh[k], kGScale);
-            acc[8 + k] += to_fixed(gZ * vh[k], kGScale);
+            add(k, gX * vh[k]);
+            add(4 + k, gY * vh[k]);
+            add(8 + k, gZ * vh[k]);
         }
     }
-    flush();
+    // one frame in the whole warp: one addition per entry instead of 32
+    const int fw = __reduce_max_sync(0xffffffffu, fcur);
+    if (__all_sync(0xffffffffu, fcur == fw || fcur < 0)) {
+        if (fw >= 0) {
+#pragma unroll
+            for (int k = 0; k < 24; ++k)
+                for (int o = 16; o; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+            if (lane == 0) {
+                fcur = fw;
+                flush();
+            }
+        }
+    } else {
+        flush();
+    }
     __syncthreads();
-    if (tid < 9) {
-        float acc = 0.0f;
-        for (int f = 0; f < a.nF; ++f) {
-            const float *dT = a.dT + ((((size_t)c * a.nI + b) * a.nF + f) * 9 + tid) * 12;
-            for (int e = 0; e < 12; ++e)
-                acc = fmaf((float)((double)(long long)G[f * 12 + e] * (1.0 / kGScale)), dT[e], acc);
-        }
-        a.grad[(size_t)c * a.d + 9 * b + tid] = acc;
+    if (tid == 0) {
+        __threadfence();
+        s_last = atomicAdd(a.rdone + c, 1u) == gridDim.x * a.nI - 1;
     }
+    __syncthreads();
+    if (!s_last || tid >= 9 * a.nI) return;
+    __threadfence();
+    const int bb = tid / 9, k = tid - 9 * bb;
+    const size_t cbb = (size_t)c * a.nI + bb;
+    float sum = 0.0f;
+    for (int f = 0; f < a.nF; ++f)
+#pragma unroll
+        for (int e = 0; e < 12; ++e) {
+            const unsigned long long *g = a.G + ((cbb * a.nF + f) * 12 + e) * 2;
+            const float gv = fmaf(__ll2float_rn((long long)__ldcg(g + 1)), 1.0f / kRestScale,
+                                  __ll2float_rn((long long)__ldcg(g)));
+            sum = fmaf(gv * (1.0f / kGScale), a.dT[((cbb * a.nF + f) * 9 + k) * 12 + e], sum);
+        }
+    a.grad[(size_t)c * a.d + 9 * bb + k] = sum;
 }
-
 
 // Adam on the refined candidates, in the optimiser's normalised units
 // (x = params / scales): m, v, bias correction (Kingma & Ba, 2015).
@@ -743,17 +1037,19 @@ using namespace trk;
 
 namespace {
 
+// Scratch of one tracker: one allocation, laid out for `cap` candidates.
 struct SoftScratch {
     int cap = 0;
-    float4 *sv = nullptr;
-    longlong2 *gv = nullptr;
-    float *dT = nullptr;
-    short4 *box = nullptr;
-    int4 *ibox = nullptr;
-    int4 *cbox = nullptr;
-    double *lpart = nullptr;
-    int lpart_cap = 0;
+    bool grad = false;         // laid out with the backward's arrays
+    int fwd_grid = 0, bwd_grid = 0;
+    void *mem = nullptr;
+    SoftArgs a{};              // the arrays
 };
+
+// A call on more candidates than this takes them in slices: the scratch stays
+// below about two gigabytes (the records and the per-pixel factors of a
+// 640x512, 20k-triangle candidate are about 3.5 MB).
+constexpr size_t kSoftBudget = (size_t)2 << 30;
 
 struct RefineBuf {
     int cap = 0;
@@ -767,33 +1063,91 @@ trk_status soft_fail(trk_status st, const char *why)
     return st;
 }
 
-trk_status soft_scratch(trk_tracker *t, int lam, SoftScratch **out)
+// Lays the arrays out from `base` (NULL: only counts) and returns the bytes.
+size_t soft_layout(SoftArgs &a, int lam, bool grad, char *base)
+{
+    size_t off = 0;
+    auto take = [&](auto *&p, size_t n) {
+        p = base ? reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + off) : nullptr;
+        off += (n * sizeof(*p) + 255) & ~(size_t)255;
+    };
+    const size_t L = (size_t)lam, nb = (size_t)a.nbx * a.nby, nt = L * a.NTp, fr = L * a.nI * a.nF;
+    take(a.rec, 4 * nt);
+    take(a.box, nt);
+    take(a.gwin, L * a.ngroups);
+    take(a.active, L * a.nby * a.wpr);
+    take(a.items, L * nb);
+    take(a.ctl, 8);
+    take(a.rdone, L);
+    take(a.lsum, L);
+    take(a.Tf, fr * 12);
+    take(a.dT, fr * 9 * 12);
+    if (grad) {
+        take(a.units, L * a.ngroups * kBwdMaxSeg);
+        take(a.wp, L * nb * kBlkPx);
+        take(a.gv, L * a.nI * a.V);
+        take(a.G, fr * 24);
+    }
+    return off;
+}
+
+void soft_shape(SoftArgs &a, const trk_tracker *t)
+{
+    a.ch = t->ch;
+    a.nF = t->ch.n_frames;
+    a.nI = t->ch.n_inst;
+    a.V = t->V;
+    a.T = t->T;
+    a.d = t->d;
+    a.W = t->cam.W;
+    a.H = t->cam.H;
+    a.Wq = t->cam.Wq;
+    a.nbx = (a.W + kBlkW - 1) / kBlkW;
+    a.nby = (a.H + kBlkH - 1) / kBlkH;
+    a.wpr = (a.nbx + 31) / 32;
+    a.ngroups = (int)(((long long)a.nI * a.T + 31) / 32);
+    a.NTp = 32 * a.ngroups;
+}
+
+// The largest slice of a call on lam candidates (at least one).
+int soft_slice(const trk_tracker *t, int lam, bool grad)
+{
+    SoftArgs a{};
+    soft_shape(a, t);
+    const size_t per = soft_layout(a, 1, grad, nullptr);
+    return (int)std::max<size_t>(1, std::min<size_t>((size_t)lam, kSoftBudget / std::max<size_t>(per, 1)));
+}
+
+trk_status soft_scratch(trk_tracker *t, int lam, bool grad, SoftScratch **out)
 {
     SoftScratch *s = static_cast<SoftScratch *>(t->soft);
-    if (s && s->cap >= lam) {
+    if (s && s->cap >= lam && (s->grad || !grad)) {
         *out = s;
         return TRK_OK;
     }
+    if (s) {  // grow: keep what either kind of call needs
+        lam = std::max(lam, s->cap);
+        grad |= s->grad;
+    }
     soft_free(t);
     s = new SoftScratch();
-    const int nI = t->ch.n_inst;
-    const size_t nv = (size_t)lam * nI * t->V;
+    t->soft = s;
+    soft_shape(s->a, t);
+    const size_t bytes = soft_layout(s->a, lam, grad, nullptr);
     cudaError_t e;
-    if ((e = cudaMalloc(&s->sv, sizeof(float4) * nv)) != cudaSuccess ||
-        (e = cudaMalloc(&s->gv, sizeof(longlong2) * nv)) != cudaSuccess ||
-        (e = cudaMalloc(&s->dT, sizeof(float) * (size_t)lam * nI * t->ch.n_frames * 9 * 12)) != cudaSuccess ||
-        (e = cudaMalloc(&s->box, sizeof(short4) * (size_t)lam * nI * t->T)) != cudaSuccess ||
-        (e = cudaMalloc(&s->ibox, sizeof(int4) * (size_t)lam * nI)) != cudaSuccess ||
-        (e = cudaMalloc(&s->cbox, sizeof(int4) * (size_t)lam * ((nI * t->T + kChunk - 1) / kChunk))) != cudaSuccess ||
-        (e = cudaMalloc(&s->lpart, sizeof(double) * lam * (size_t)((t->cam.W + kTile - 1) / kTile) *
-                                       ((t->cam.H + kTile - 1) / kTile))) != cudaSuccess) {
-        t->soft = s;
+    int fwd = 0, bwd = 0, sms = 0;
+    if ((e = cudaMalloc(&s->mem, bytes)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, t->device)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fwd, k_soft_fwd, 32 * kFwdWarps, 0)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bwd, k_soft_bwd, 128, 0)) != cudaSuccess) {
         soft_free(t);
         return soft_fail(e == cudaErrorMemoryAllocation ? TRK_ENOMEM : TRK_ECUDA, cudaGetErrorString(e));
     }
+    soft_layout(s->a, lam, grad, static_cast<char *>(s->mem));
     s->cap = lam;
-    s->lpart_cap = lam;
-    t->soft = s;
+    s->grad = grad;
+    s->fwd_grid = std::max(1, fwd) * sms;
+    s->bwd_grid = std::max(1, bwd) * sms;
     *out = s;
     return TRK_OK;
 }
@@ -802,17 +1156,11 @@ trk_status soft_launch(trk_tracker *t, const float *params, int lam, const uint3
                        float *grad, cudaStream_t st)
 {
     if (lam == 0) return TRK_OK;
+    const int slice = soft_slice(t, lam, grad != nullptr);
     SoftScratch *s = nullptr;
-    trk_status r = soft_scratch(t, lam, &s);
+    trk_status r = soft_scratch(t, slice, grad != nullptr, &s);
     if (r != TRK_OK) return r;
-    SoftArgs a{};
-    a.ch = t->ch;
-    a.nF = t->ch.n_frames;
-    a.nI = t->ch.n_inst;
-    a.V = t->V;
-    a.T = t->T;
-    a.d = t->d;
-    a.lam = lam;
+    SoftArgs a = s->a;
     a.fx = (float)t->cam.fx;
     a.fy = (float)t->cam.fy;
     a.cx = (float)(t->cam.cx256 / 256.0);
@@ -820,29 +1168,27 @@ trk_status soft_launch(trk_tracker *t, const float *params, int lam, const uint3
     a.z_near = (float)t->cam.z_near;
     a.guard = (float)t->cam.guard;
     a.sigma = sigma;
-    a.W = t->cam.W;
-    a.H = t->cam.H;
-    a.Wq = t->cam.Wq;
-    a.ntx = (a.W + kTile - 1) / kTile;
-    a.nty = (a.H + kTile - 1) / kTile;
     a.verts = t->verts;
     a.tris = t->tris;
-    a.params = params;
     a.mask = mask;
-    a.sv = s->sv;
-    a.gv = s->gv;
-    a.dT = s->dT;
-    a.box = s->box;
-    a.ibox = s->ibox;
-    a.lpart = s->lpart;
-    a.cbox = s->cbox;
-    a.nchunk = (a.nI * a.T + kChunk - 1) / kChunk;
-    a.loss = loss;
-    a.grad = grad;
-    k_soft_project<<<dim3(lam, a.nI), kSoftThreads, 0, st>>>(a);
-    k_soft_tribox<<<dim3(a.nchunk, lam), kChunk, 0, st>>>(a);
-    k_soft_tile<<<dim3(a.ntx * a.nty, lam), kSoftThreads, 0, st>>>(a);
-    k_soft_reduce<<<dim3(lam, a.nI), kSoftThreads, 0, st>>>(a);
+    for (int c0 = 0; c0 < lam; c0 += slice) {
+        a.lam = std::min(slice, lam - c0);
+        a.params = params + (size_t)c0 * a.d;
+        a.loss = loss + c0;
+        a.grad = grad ? grad + (size_t)c0 * a.d : nullptr;
+        k_soft_fk<<<dim3(a.lam, a.nI), kSoftThreads, 0, st>>>(a);
+        if (a.ngroups) {
+            const int gpb = kSoftThreads / 32;
+            k_soft_tris<<<dim3((a.ngroups + gpb - 1) / gpb, a.lam), kSoftThreads, a.nI * a.nF * 12 * sizeof(float),
+                          st>>>(a);
+        }
+        k_soft_fwd<<<s->fwd_grid, 32 * kFwdWarps, 0, st>>>(a);
+        if (grad) {
+            if (a.ngroups) k_soft_bwd<<<s->bwd_grid, 128, 0, st>>>(a);
+            const int vpb = kSoftThreads * kRedVerts;
+            k_soft_reduce<<<dim3(std::max(1, (a.V + vpb - 1) / vpb), a.lam * a.nI), kSoftThreads, 0, st>>>(a);
+        }
+    }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TRK_OK : soft_fail(TRK_ECUDA, cudaGetErrorString(e));
 }
@@ -853,13 +1199,7 @@ void trk::soft_free(trk_tracker *t)
 {
     SoftScratch *s = static_cast<SoftScratch *>(t->soft);
     if (!s) return;
-    cudaFree(s->sv);
-    cudaFree(s->gv);
-    cudaFree(s->dT);
-    cudaFree(s->box);
-    cudaFree(s->ibox);
-    cudaFree(s->cbox);
-    cudaFree(s->lpart);
+    cudaFree(s->mem);
     delete s;
     t->soft = nullptr;
 }

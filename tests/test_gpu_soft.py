@@ -161,3 +161,48 @@ def test_soft_results_repeat_bit_for_bit(api):
         pose, picked = es.refine(Mp, top_k=8, steps=5, lr=0.05)
         poses.append((pose.cpu().numpy().copy(), picked))
     assert np.array_equal(poses[0][0], poses[1][0]) and poses[0][1] == poses[1][1]
+
+
+# Image sizes around the 8x4-pixel blocks of the pair kernels, triangle counts
+# around the groups of 32, one and two instruments, sigma on both sides of 1.
+# Tolerances: coordinates are rounded to about 3e-5 px in FP32, which moves an
+# exponential's argument by 3e-5 / sigma; the bounds are those of the tests
+# above (1e-4, 1e-3) at sigma >= 1 and twice them at sigma = 0.5.
+@pytest.mark.parametrize("W,H,mesh,n_inst,sigma,lam", [
+    (8, 4, "c1", 1, 1.0, 1), (9, 5, "c1", 1, 1.0, 2), (31, 33, "800", 2, 0.5, 3), (64, 64, "800", 1, 4.0, 2),
+    (257, 67, "c1", 1, 1.0, 2), (100, 3, "900", 1, 0.5, 5),
+])
+def test_soft_block_edges_and_remainders(api, W, H, mesh, n_inst, sigma, lam):
+    f = 1.25 * max(W, H)
+    sc, tr, M, Mp, P = _case(api, mesh, "c1", n_inst, wl.Intrinsics(f, f, W / 2, H / 2, W, H), 91, lam)
+    P[-1, 3:6] = [0.0, 0.0, -50.0]  # behind the camera: nothing drawn for this instrument
+    loss, g = tr.soft_eval(torch.from_numpy(P).cuda(), Mp, sigma=sigma, grad=True)
+    assert torch.equal(loss, tr.soft_eval(torch.from_numpy(P).cuda(), Mp, sigma=sigma))
+    loss, g = loss.cpu().numpy(), g.cpu().numpy()
+    s = wl.default_scales(sc.d)
+    k = 1.0 if sigma >= 1.0 else 2.0
+    for c in range(lam):
+        L, gref = soft.soft_grad(sc, P[c].astype(np.float64), M, sigma)
+        assert loss[c] == pytest.approx(L, rel=k * 1e-4, abs=1e-6), c
+        if np.linalg.norm(gref * s) > 0:
+            assert _rel(g[c], gref, s) < k * 1e-3, (c, g[c], gref)
+        else:
+            assert not g[c].any()
+
+
+def test_soft_results_do_not_depend_on_the_population(api):
+    """A population larger than one slice of the scratch (1280x1024, two
+    instruments of 40k triangles: about 170 candidates) gives, candidate by
+    candidate, the bits of a call on that candidate alone."""
+    sc = wl.make_scene("40000", "c2", n_instruments=2, K=wl.Intrinsics(1600.0, 1600.0, 640.0, 512.0, 1280, 1024))
+    rng = np.random.default_rng(95)
+    gt = np.concatenate([wl.sample_state(rng, sc.K) for _ in range(2)])
+    tr = api.Tracker(sc, lambda_max=1)
+    M = api.unpack_mask(tr.render(torch.from_numpy(gt.astype(np.float32)).cuda()), 1280)
+    Mp = tr.pack_mask(M)
+    P = torch.from_numpy(wl.population_around(rng, gt, 190)).cuda()
+    loss, g = tr.soft_eval(P, Mp, grad=True)
+    for c in (0, 95, 169, 170, 171, 189):
+        l1, g1 = tr.soft_eval(P[c:c + 1].contiguous(), Mp, grad=True)
+        assert torch.equal(l1.view(torch.int32), loss[c:c + 1].view(torch.int32)), c
+        assert torch.equal(g1.view(torch.int32), g[c:c + 1].view(torch.int32)), c
