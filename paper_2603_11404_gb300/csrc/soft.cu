@@ -18,13 +18,14 @@
 //                   state tangents carried along (forward mode); clears the
 //                   candidate's accumulators
 //   k_soft_tris     a warp per group of 32 triangles: projection, edge
-//                   records, boxes; marks the 8x4-pixel blocks that the group
-//                   can reach and lists each marked block once
+//                   records, boxes; counts the groups that can reach each
+//                   8x4-pixel block
+//   k_soft_list     the blocks within reach, heavy ones first
 //   k_soft_fwd      per listed block: the product over the triangles, the
 //                   block's squared error and, for a gradient, the factor
 //                   2 (S - M) (1 - S) / sigma of its pixels
-//   k_soft_bwd      per (group, part of its window): dL/d(u, v) of the
-//                   group's triangles, added to the vertices
+//   k_soft_bwd      per pair of listed blocks: dL/d(u, v) of the triangles in
+//                   reach over the blocks' pixels, added to the vertices
 //   k_soft_reduce   dL/dX per vertex, reduced per kinematic frame to a 3x4
 //                   matrix G_f, contracted with the tangents dT_f/dtheta_k
 //
@@ -47,9 +48,9 @@ constexpr float kSoftCutoff = 14.0f;   // in units of sigma
 constexpr int kBlkW = 8, kBlkH = 4;    // pixel block of the pair kernels: one pixel per lane at its ends
 constexpr int kBlkPx = kBlkW * kBlkH;
 constexpr int kSoftThreads = 256;
-constexpr int kFwdWarps = 4;           // most warps that share a block of the forward
-constexpr int kBwdSeg = 64;            // blocks of a group's window per backward unit ...
-constexpr int kBwdMaxSeg = 16;         // ... and at most this many units per group
+constexpr int kFwdWarps = 4;           // warps that share a heavy block of the forward
+constexpr int kBwdWarps = 4;           // and of the backward
+constexpr int kHeavy = 48;             // groups within reach that make a block heavy
 // With 1 + Q = prod (1 + exp): Q above kOne makes 1 - S < 2^-25, S is 1 in FP32
 // and the pixel's gradient factor 0, whatever the remaining triangles add.  The
 // forward stops early only at the larger kSaturated, so that a product formed
@@ -260,8 +261,9 @@ struct SoftArgs {
     int nF, nI, V, T, d, lam;
     float fx, fy, cx, cy, z_near, guard, sigma;
     int W, H, Wq;
-    int nbx, nby, wpr;        // pixel blocks per row and column, bitmap words per block row
+    int nbx, nby;             // pixel blocks per row and column
     int ngroups, NTp;         // groups of 32 triangles (over all instruments), triangles padded to whole groups
+    int nsup;                 // runs of 32 groups
     const float4 *verts;
     const int4 *tris;
     const float *params;      // [lam * d]
@@ -271,11 +273,12 @@ struct SoftArgs {
     float4 *rec;              // [4][lam * NTp] edge records (struct TriRec)
     float4 *box;              // [lam * NTp] centre and half extents of the triangle's bounding box
     short4 *gwin;             // [lam * ngroups] blocks that the group can reach: bx0, by0, bx1, by1 (bx0 > bx1: none)
-    uint32_t *active;         // [lam * nby * wpr] bitmap of the listed blocks
-    int2 *items;              // [lam * nbx * nby] listed blocks: candidate, by << 16 | bx
-    int2 *units;              // [lam * ngroups * kBwdMaxSeg] backward units: candidate, group * kBwdMaxSeg + part
+    int4 *swin;               // [lam * nsup] the same for runs of 32 groups
+    int *count;               // [lam * nby * nbx] groups that can reach each block
+    int2 *fwd, *bwd;          // [lam * nby * nbx], [lam * (nby + 1) / 2 * nbx] listed blocks and pairs of blocks
+                              // (candidate, by << 16 | bx): many groups from the front, the others from the back
     float *wp;                // [lam * nbx * nby * kBlkPx] 2 (S - M) (1 - S) / sigma of the listed blocks' pixels
-    unsigned *ctl;            // [5] blocks listed, forward ticket, forward exits, units listed, backward ticket
+    unsigned *ctl;            // [kCtl] list lengths, tickets, forward exits
     unsigned *rdone;          // [lam] finished blocks of k_soft_reduce
     longlong2 *gv;            // [lam * nI * V]: dL/du, dL/dv in fixed point (units of 2^-36)
     unsigned long long *G;    // [lam * nI * nF * 12][2] fixed point, units of 2^-24 and of 2^-56
@@ -283,6 +286,8 @@ struct SoftArgs {
     float *loss;              // [lam]
     float *grad;              // [lam * d] or NULL
 };
+
+enum { kFwdHeavy, kFwdLight, kBwdHeavy, kBwdLight, kTicket, kFwdExit = kTicket + 4, kCtl };
 
 // Edge record of a drawable triangle, positively oriented, in image pixels: the
 // corners, the edges' unit directions and lengths, and
@@ -331,10 +336,12 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fk(SoftArgs a)
         }
     } else {
         const int t = tid - 32, nt = kSoftThreads - 32;
-        if (c == 0 && b == 0 && t < 5) a.ctl[t] = 0u;
+        if (c == 0 && b == 0 && t < kCtl) a.ctl[t] = 0u;
         if (b == 0) {
-            uint32_t *act = a.active + (size_t)c * a.nby * a.wpr;
-            for (int i = t; i < a.nby * a.wpr; i += nt) act[i] = 0u;
+            int *cnt = a.count + (size_t)c * a.nby * a.nbx;
+            for (int i = t; i < a.nby * a.nbx; i += nt) cnt[i] = 0;
+            for (int i = t; i < a.nsup; i += nt)
+                a.swin[(size_t)c * a.nsup + i] = make_int4(INT_MAX, INT_MAX, INT_MIN, INT_MIN);
             int m = 0;
             for (int i = t; i < a.H * a.Wq; i += nt) m += __popc(a.mask[i]);
             m = __reduce_add_sync(0xffffffffu, m);
@@ -365,8 +372,6 @@ __device__ __forceinline__ float4 soft_project(const SoftArgs &a, const float *M
     }
     return o;
 }
-
-__device__ __forceinline__ int bwd_segments(int blocks) { return min(kBwdMaxSeg, (blocks + kBwdSeg - 1) / kBwdSeg); }
 
 // A warp per group of 32 triangles.  Every lane projects its triangle's three
 // corners itself: cheaper than a pass of its own over the vertices and a gather.
@@ -437,29 +442,86 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_tris(SoftArgs a)
     }
     if (lane == 0) a.gwin[(size_t)c * a.ngroups + g] = win;
     if (win.x > win.z) return;
-    // list the blocks of the window that no group has listed yet
-    const int w0 = win.x >> 5, nw = (win.z >> 5) - w0 + 1, rows = win.w - win.y + 1;
-    for (int e = lane; e < rows * nw; e += 32) {
-        const int by = win.y + e / nw, w = w0 + e % nw;
-        uint32_t need = 0xffffffffu;
-        if (w == w0) need &= 0xffffffffu << (win.x & 31);
-        if (w == (win.z >> 5)) need &= 0xffffffffu >> (31 - (win.z & 31));
-        uint32_t *word = a.active + ((size_t)c * a.nby + by) * a.wpr + w;
-        need &= ~__ldcg(word);
-        if (!need) continue;
-        uint32_t neu = need & ~atomicOr(word, need);
-        if (!neu) continue;
-        unsigned at = atomicAdd(&a.ctl[0], (unsigned)__popc(neu));
-        for (; neu; neu &= neu - 1) a.items[at++] = make_int2(c, by << 16 | (w * 32 + __ffs(neu) - 1));
+    if (lane < 4) {
+        int *sw = reinterpret_cast<int *>(a.swin + (size_t)c * a.nsup + (g >> 5)) + lane;
+        if (lane < 2) atomicMin(sw, lane ? win.y : win.x);
+        else atomicMax(sw, lane == 3 ? win.w : win.z);
     }
-    if (a.grad) {
-        const int ns = bwd_segments(rows * (win.z - win.x + 1));
+    const int bw = win.z - win.x + 1, nb = bw * (win.w - win.y + 1);
+    int *cnt = a.count + ((size_t)c * a.nby + win.y) * a.nbx + win.x;
+    for (int e = lane; e < nb; e += 32) atomicAdd(cnt + (e / bw) * a.nbx + e % bw, 1);
+}
+
+// The work lists: a thread per pair of blocks (a block and the one below).
+__device__ __forceinline__ void append(const SoftArgs &a, bool on, bool heavy, int2 v, int base, int2 *list, int cap)
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const bool take = on && heavy == (h == 0);
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (!m) continue;
+        const int lane = threadIdx.x & 31;
         unsigned at = 0;
-        if (lane == 0) at = atomicAdd(&a.ctl[3], (unsigned)ns);
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (lane < ns) a.units[at + lane] = make_int2(c, g * kBwdMaxSeg + lane);
+        if (lane == __ffs(m) - 1) at = atomicAdd(&a.ctl[base + h], (unsigned)__popc(m));
+        at = __shfl_sync(0xffffffffu, at, __ffs(m) - 1) + __popc(m & ((1u << lane) - 1u));
+        if (take) list[h == 0 ? at : cap - 1 - at] = v;
     }
 }
+
+__global__ void __launch_bounds__(kSoftThreads) k_soft_list(SoftArgs a)
+{
+    const int c = blockIdx.y, i = blockIdx.x * kSoftThreads + threadIdx.x, nby2 = (a.nby + 1) / 2;
+    const int by = 2 * (i / a.nbx), bx = i % a.nbx;
+    const bool in = i < nby2 * a.nbx;
+    const int *cnt = a.count + ((size_t)c * a.nby + by) * a.nbx + bx;
+    const int n0 = in ? cnt[0] : 0, n1 = in && by + 1 < a.nby ? cnt[a.nbx] : 0;
+    const int2 v0 = make_int2(c, by << 16 | bx), v1 = make_int2(c, (by + 1) << 16 | bx);
+    const int cap = a.lam * a.nby * a.nbx;
+    append(a, n0 > 0, n0 >= kHeavy, v0, kFwdHeavy, a.fwd, cap);
+    append(a, n1 > 0, n1 >= kHeavy, v1, kFwdHeavy, a.fwd, cap);
+    if (a.grad) append(a, n0 + n1 > 0, max(n0, n1) >= kHeavy, v0, kBwdHeavy, a.bwd, a.lam * nby2 * a.nbx);
+}
+
+// The entries of a kernel's list: the heavy ones are taken by the whole block
+// (a ticket through shared memory), then the light ones by each warp for
+// itself.  The next ticket is drawn while the entry before it is worked on.
+struct Work {
+    bool heavy = true;
+    int c = 0, bx = 0, by = 0;
+    int ticket = 0, n_heavy, n_light;  // the ticket: thread 0's, later each warp's lane 0's
+
+    __device__ __forceinline__ Work(const SoftArgs &a, int base) : n_heavy((int)a.ctl[base]), n_light((int)a.ctl[base + 1])
+    {
+        if (threadIdx.x == 0) ticket = (int)atomicAdd(&a.ctl[kTicket + base], 1u);
+    }
+
+    __device__ __forceinline__ void take(int2 v) { c = v.x, bx = v.y & 0xffff, by = v.y >> 16; }
+
+    __device__ __forceinline__ bool next(const SoftArgs &a, int base, const int2 *list, int cap, int *s_it)
+    {
+        const int lane = threadIdx.x & 31;
+        if (heavy) {
+            __syncthreads();  // the previous entry's shared memory is free
+            if (threadIdx.x == 0) {
+                *s_it = ticket;
+                if (ticket < n_heavy) ticket = (int)atomicAdd(&a.ctl[kTicket + base], 1u);
+            }
+            __syncthreads();
+            const int i = *s_it;
+            if (i < n_heavy) {
+                take(list[i]);
+                return true;
+            }
+            heavy = false;
+            if (lane == 0) ticket = (int)atomicAdd(&a.ctl[kTicket + base + 1], 1u);
+        }
+        const int i = __shfl_sync(0xffffffffu, ticket, 0);
+        if (i >= n_light) return false;
+        if (lane == 0) ticket = (int)atomicAdd(&a.ctl[kTicket + base + 1], 1u);
+        take(list[cap - 1 - i]);
+        return true;
+    }
+};
 
 __device__ __forceinline__ float min3(float a, float b, float c)
 {
@@ -467,16 +529,16 @@ __device__ __forceinline__ float min3(float a, float b, float c)
     asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-__device__ __forceinline__ float max3(float a, float b, float c)
-{
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
 __device__ __forceinline__ float ex2(float x)
 {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float sqrt_(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 __device__ __forceinline__ float rsq(float x)
@@ -497,75 +559,171 @@ __device__ __forceinline__ float with_sign(float x, float s)
     return __uint_as_float(__float_as_uint(x) | (__float_as_uint(s) & 0x80000000u));
 }
 
-// Does the triangle's bounding box come within the cutoff of block (bx, by)?
-__device__ __forceinline__ bool box_near(float4 b, int bx, int by, float reach2)
-{
-    const float x = (float)(bx * kBlkW) + 0.5f * (kBlkW - 1), y = (float)(by * kBlkH) + 0.5f * (kBlkH - 1);
-    const float dx = fmaxf(fabsf(b.x - x) - (b.z + 0.5f * (kBlkW - 1)), 0.0f);
-    const float dy = fmaxf(fabsf(b.y - y) - (b.w + 0.5f * (kBlkH - 1)), 0.0f);
-    return fmaf(dx, dx, dy * dy) <= reach2;
-}
+// The triangles that come within the cutoff of `kRows` rows of pixels from block
+// (bx, by) down, collected into batches of 32 by one warp.  Runs of 32 groups,
+// then groups (of those the ones whose number is `warp` modulo nw), then
+// triangles are tested against the block, one per lane; the next group's boxes
+// and the next batch's records are on their way while the last are used.
+template <int kRows>
+struct Collector {
+    const int4 *sw;    // the candidate's windows of runs and groups, boxes and records
+    const short4 *gw;
+    const float4 *box, *rec;
+    size_t stride;
+    int *qu;           // the warp's queue (64 entries)
+    int bx, by, s0 = 0, sb = 0, gb = 0, qn = 0, nsup, ngroups;
+    unsigned sup = 0, hits = 0, mine;
+    float reach2;
+    float4 pre;        // box of the next group's triangle
 
-// The edges of a triangle seen from a block: coordinates of the block's first
-// pixel along (a) and across (b, positive inside) each edge and the steps to
-// the next pixel, all in units of sigma / log2(e), so that 2^distance is the
-// sigmoid's exponential.
-struct BlockEdges {
-    float a[3], b[3], tx[3], ty[3], L[3];
+    __device__ __forceinline__ Collector(const SoftArgs &a, int c, int bx_, int by_, int warp, int nw, int *queue)
+        : sw(a.swin + (size_t)c * a.nsup), gw(a.gwin + (size_t)c * a.ngroups), box(a.box + (size_t)c * a.NTp),
+          rec(a.rec + (size_t)c * a.NTp), stride((size_t)a.lam * a.NTp), qu(queue), bx(bx_), by(by_), nsup(a.nsup),
+          ngroups(a.ngroups), mine(nw == 1 ? 0xffffffffu : 0x11111111u << warp)
+    {
+        static_assert(kFwdWarps == 4 && kBwdWarps == 4, "`mine` takes every fourth group");
+        const float reach = kSoftCutoff * a.sigma + 0.01f;
+        reach2 = reach * reach;
+    }
+
+    __device__ __forceinline__ bool near(float4 b) const
+    {
+        const float x = (float)(bx * kBlkW) + 0.5f * (kBlkW - 1), y = (float)(by * kBlkH) + 0.5f * (kRows - 1);
+        const float dx = fmaxf(fabsf(b.x - x) - (b.z + 0.5f * (kBlkW - 1)), 0.0f);
+        const float dy = fmaxf(fabsf(b.y - y) - (b.w + 0.5f * (kRows - 1)), 0.0f);
+        return fmaf(dx, dx, dy * dy) <= reach2;
+    }
+
+    __device__ __forceinline__ bool in(int x0, int y0, int x1, int y1) const
+    {
+        return x0 <= bx && bx <= x1 && y0 <= by + (kRows - 1) / kBlkH && by <= y1;
+    }
+
+    // The next batch: the lane's triangle (numbered within the candidate) or
+    // -1; false when no triangle is left.
+    __device__ __forceinline__ bool next(int lane, int &t)
+    {
+        while (qn < 32) {
+            if (!hits) {
+                if (!sup) {
+                    if (s0 >= nsup) break;
+                    sb = s0;
+                    bool h = false;
+                    if (sb + lane < nsup) {
+                        const int4 w = sw[sb + lane];
+                        h = in(w.x, w.y, w.z, w.w);
+                    }
+                    sup = __ballot_sync(0xffffffffu, h);
+                    s0 += 32;
+                    continue;
+                }
+                gb = (sb + __ffs(sup) - 1) * 32;
+                sup &= sup - 1;
+                bool h = false;
+                if (gb + lane < ngroups) {
+                    const short4 w = gw[gb + lane];
+                    h = in(w.x, w.y, w.z, w.w);
+                }
+                hits = __ballot_sync(0xffffffffu, h) & mine;
+                if (hits) pre = box[(gb + __ffs(hits) - 1) * 32 + lane];
+                continue;
+            }
+            const int tt = (gb + __ffs(hits) - 1) * 32 + lane;
+            const float4 b = pre;
+            hits &= hits - 1;
+            if (hits) pre = box[(gb + __ffs(hits) - 1) * 32 + lane];
+            const bool h = near(b);
+            const unsigned m = __ballot_sync(0xffffffffu, h);
+            if (h) qu[qn + __popc(m & ((1u << lane) - 1u))] = tt;
+            qn += __popc(m);
+        }
+        if (qn == 0) return false;
+        __syncwarp();
+        const int n = min(qn, 32);  // the last (up to) 32 of the queue
+        qn -= n;
+        t = lane < n ? qu[qn + lane] : -1;
+        __syncwarp();
+        if (t >= 0)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) asm volatile("prefetch.global.L1 [%0];" ::"l"(rec + q * stride + t));
+        return true;
+    }
 };
 
-__device__ __forceinline__ BlockEdges block_edges(const TriRec &r, int bx, int by, float k)
+// The edges of a triangle seen from a block, in units of the cutoff (14 sigma):
+// the coordinates of the row's first pixel along each edge from its middle (a)
+// and across it (b, positive inside), the edge's direction and half its length.
+// In these units a point's distance beyond an edge's end, |a| - h clamped to
+// [0, 1], is one saturating addition: what is clamped at 1 is out of reach.
+// (FP32 additions and FMAs issue every cycle, minima, selections and logic
+// every second one, packed FP32 pairs take two cycles: a version on pairs of
+// pixels was no faster.)
+struct BlockEdges {
+    float a[3], b[3], tx[3], ty[3], h[3];
+
+    __device__ __forceinline__ void down()  // to the next row of pixels
+    {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            a[k] += ty[k];
+            b[k] += tx[k];
+        }
+    }
+};
+
+__device__ __forceinline__ BlockEdges block_edges(const TriRec &r, bool drawn, int bx, int by, float unit)
 {
     const float X = (float)(bx * kBlkW), Y = (float)(by * kBlkH);
     BlockEdges e;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const float rx = X - r.x[q], ry = Y - r.y[q];
-        e.tx[q] = r.tx[q] * k;
-        e.ty[q] = r.ty[q] * k;
-        e.L[q] = r.L[q] * k;
-        e.a[q] = fmaf(rx, e.tx[q], ry * e.ty[q]);
-        e.b[q] = fmaf(ry, e.tx[q], -rx * e.ty[q]);
+        e.tx[q] = drawn ? r.tx[q] * unit : 0.0f;
+        e.ty[q] = drawn ? r.ty[q] * unit : 0.0f;
+        e.h[q] = 0.5f * r.L[q] * unit;
+        e.a[q] = fmaf(rx, e.tx[q], ry * e.ty[q]) - e.h[q];
+        e.b[q] = drawn ? fmaf(ry, e.tx[q], -rx * e.ty[q]) : -10.0f;  // no triangle: out of reach
     }
     return e;
 }
 
-// log2-scaled cutoff and unit of the distances
-constexpr float kLog2e = 1.44269504089f;
-constexpr float kCutLog2 = -kSoftCutoff * kLog2e;
+constexpr float kExpScale = kSoftCutoff * 1.44269504089f;  // exp(d / sigma) = 2^(kExpScale d / cutoff)
 
 // The product over one batch of triangles (one per lane) into the lane's 32
 // running products Q (1 + Q = product of 1 + exp(d / sigma)).  Per pixel: the
 // point's coordinates (a, b) in the three edge frames, the squared distance
-// b^2 + max(a - L, -a, 0)^2 to each edge, its minimum, the sign from the
-// smallest b (inside: every b >= 0, and there the nearest edge's line is
-// nearest at the edge), and one exponential.
+// b^2 + max(|a| - h, 0)^2 to each edge, its minimum, the sign from the smallest
+// b (inside: every b >= 0, and there the nearest edge's line is nearest at the
+// edge), and one exponential.
 __device__ __forceinline__ void fwd_batch(BlockEdges &e, float (&Q)[kBlkPx])
 {
 #pragma unroll
     for (int py = 0; py < kBlkH; ++py) {
+        // stage by stage over a row, so that eight pixels are in flight
+        float d[kBlkW], sg[kBlkW];
 #pragma unroll
         for (int px = 0; px < kBlkW; ++px) {
-            float d2[3], bb[3];
+            float d2[3], b[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const float av = fmaf((float)px, e.tx[k], e.a[k]);
-                bb[k] = fmaf(-(float)px, e.ty[k], e.b[k]);
-                const float o = max3(av - e.L[k], -av, 0.0f);
-                d2[k] = fmaf(o, o, bb[k] * bb[k]);
+                const float a = fmaf((float)px, e.tx[k], e.a[k]);
+                b[k] = fmaf(-(float)px, e.ty[k], e.b[k]);
+                const float o = __saturatef(fabsf(a) - e.h[k]);
+                d2[k] = fmaf(o, o, b[k] * b[k]);
             }
-            const float m2 = fmaxf(min3(d2[0], d2[1], d2[2]), 1e-30f);
-            const float dist = fminf(m2 * rsq(m2), 64.0f);  // 2^64 saturates the pixel; no infinity enters the product
-            const float x = with_sign(dist, min3(bb[0], bb[1], bb[2]));
-            const float p = ex2(x);
-            float &q = Q[py * kBlkW + px];
-            if (x >= kCutLog2) q = fmaf(q, p, q + p);
+            d[px] = min3(d2[0], d2[1], d2[2]);
+            sg[px] = min3(b[0], b[1], b[2]);
         }
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            e.a[k] += e.ty[k];
-            e.b[k] += e.tx[k];
+        for (int px = 0; px < kBlkW; ++px) d[px] = with_sign(sqrt_(d[px]), sg[px]);
+#pragma unroll
+        for (int px = 0; px < kBlkW; ++px) sg[px] = ex2(d[px] * kExpScale);
+#pragma unroll
+        for (int px = 0; px < kBlkW; ++px) {
+            float &q = Q[py * kBlkW + px];
+            if (d[px] > -1.0f) q = fmaf(q, sg[px], q + sg[px]);  // q > 0: an infinite term makes q infinite, never NaN
         }
+        e.down();
     }
 }
 
@@ -596,129 +754,94 @@ __device__ __forceinline__ float combine_lanes(const float (&Q)[kBlkPx], int lan
     return v[0];
 }
 
-// Bound by instruction issue (67-82 % of the cycles; about 30 instructions per
-// 32 pairs).  640x512, 20k triangles, 64 candidates: 1.9 ms, where a pixel per
-// thread with the triangles in shared memory (four 16-byte reads, a branchy
-// distance of about 180 instructions and a log1p per pair) took 12 ms.
-// Persistent blocks over the listed pixel blocks.  The warps of a block share
-// the triangles of its pixel block group by group (group g belongs to warp
-// g mod warps); each warp collects the triangles that come near into full
-// batches of 32.  Every kCheck batches a warp looks whether the pixels are
-// saturated (see kSaturated) by its own products and the last ones the other
-// warps left in shared memory: those only grow, so a decision made on them
-// holds, and the results do not depend on when it is made.
-__global__ void __launch_bounds__(32 * kFwdWarps) k_soft_fwd(SoftArgs a)
+// Persistent blocks over the listed pixel blocks.  A light block of pixels is
+// one warp's (no barrier, at most one batch that is not full); a heavy one (a
+// shaft seen end-on puts thousands of triangles within its reach) is shared by
+// the block's warps, every fourth group to a warp.  Bound by issue (72 % of the
+// cycles; half of the instructions evaluate pairs, a third collect them).
+// 640x512, 20k triangles, 64 candidates (two scenes): 0.52 and 1.54 ms; with
+// every block shared by four warps 0.92 and 1.93 ms, with one warp each 0.56
+// and 1.44 ms -- but then 8 candidates, where the heaviest blocks decide, take
+// 1.52 instead of 1.03 ms for a loss and a gradient.  (A pixel per thread with
+// the triangles in shared memory, about 180 instructions per pair: 12 ms.)
+// Every kCheck batches a warp looks whether the pixels are saturated (see
+// kSaturated) by its own products and the last ones the other warps left in
+// shared memory: those only grow, so a decision made on them holds, and the
+// results do not depend on when it is made.
+__global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
 {
     constexpr int kCheck = 6;
     __shared__ int queue[kFwdWarps][64];
     __shared__ float part[kFwdWarps][kBlkPx];
     __shared__ int s_it;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const float k2 = kLog2e / a.sigma, inv_s = 1.0f / a.sigma;
-    const float reach = kSoftCutoff * a.sigma + 0.01f, reach2 = reach * reach;
-    const int n_items = (int)a.ctl[0];
-    int *qu = queue[warp];
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_it = (int)atomicAdd(&a.ctl[1], 1u);
-        part[warp][lane] = 0.0f;
-        __syncthreads();
-        if (s_it >= n_items) break;
-        const int2 it = a.items[s_it];
-        const int c = it.x, bx = it.y & 0xffff, by = it.y >> 16;
-        const short4 *gw = a.gwin + (size_t)c * a.ngroups;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float unit = 1.0f / (kSoftCutoff * a.sigma), inv_s = 1.0f / a.sigma;
+    Work w(a, kFwdHeavy);
+    while (w.next(a, kFwdHeavy, a.fwd, a.lam * a.nby * a.nbx, &s_it)) {
+        const int c = w.c;
         const size_t tb = (size_t)c * a.NTp;
-        const int j = bx * kBlkW + (lane & (kBlkW - 1)), i = by * kBlkH + lane / kBlkW;
+        const int j = w.bx * kBlkW + (lane & (kBlkW - 1)), i = w.by * kBlkH + lane / kBlkW;
         const bool on = j < a.W && i < a.H;
+        if (w.heavy) {
+            part[warp][lane] = 0.0f;
+            __syncthreads();
+        }
         float Q[kBlkPx];
 #pragma unroll
-        for (int p = 0; p < kBlkPx; ++p) Q[p] = 0.0f;
-        int qn = 0, g0 = warp, batches = 0;
-        unsigned hits = 0;
-        int gb = 0;
-        for (;;) {
-            while (qn < 32) {
-                if (!hits) {
-                    if (g0 >= a.ngroups) break;
-                    gb = g0;
-                    const int g = gb + lane * nw;
-                    bool h = false;
-                    if (g < a.ngroups) {
-                        const short4 w = gw[g];
-                        h = w.x <= bx && bx <= w.z && w.y <= by && by <= w.w;
-                    }
-                    hits = __ballot_sync(0xffffffffu, h);
-                    g0 += 32 * nw;
-                    continue;
-                }
-                const int g = gb + (__ffs(hits) - 1) * nw;
-                hits &= hits - 1;
-                const int t = g * 32 + lane;
-                const bool h = box_near(a.box[tb + t], bx, by, reach2);
-                const unsigned m = __ballot_sync(0xffffffffu, h);
-                if (h) qu[qn + __popc(m & ((1u << lane) - 1u))] = t;
-                qn += __popc(m);
-            }
-            if (qn == 0) break;
-            __syncwarp();
-            // the last (up to) 32 of the queue, one per lane
-            const int n = min(qn, 32);
-            qn -= n;
-            BlockEdges e;
-            if (lane < n) {
-                e = block_edges(load_rec(a, tb + qu[qn + lane]), bx, by, k2);
-            } else {  // no triangle: far outside
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    e.a[k] = 0.0f;
-                    e.b[k] = -1e4f;
-                    e.tx[k] = e.ty[k] = e.L[k] = 0.0f;
-                }
-            }
-            __syncwarp();
+        for (int p = 0; p < kBlkPx; ++p) Q[p] = 1e-30f;  // nothing beside the smallest term (8e-7), and not zero
+        Collector<kBlkH> col(a, c, w.bx, w.by, warp, w.heavy ? kFwdWarps : 1, queue[warp]);
+        int t, batches = 0;
+        bool more = col.next(lane, t);
+        while (more) {
+            BlockEdges e = block_edges(load_rec(a, tb + max(t, 0)), t >= 0, w.bx, w.by, unit);
+            more = col.next(lane, t);
             fwd_batch(e, Q);
             if (++batches % kCheck == 0) {
                 float q = combine_lanes(Q, lane);
-                part[warp][lane] = q;
-                volatile float(*pv)[kBlkPx] = part;
-                for (int w = 0; w < nw; ++w)
-                    if (w != warp) {
-                        const float o = pv[w][lane];
-                        q = fmaf(q, o, q + o);
+                if (w.heavy) {
+                    part[warp][lane] = q;
+                    volatile float(*pv)[kBlkPx] = part;
+#pragma unroll
+                    for (int o = 1; o < kFwdWarps; ++o) {
+                        const float r = pv[(warp + o) % kFwdWarps][lane];
+                        q = fmaf(q, r, q + r);
                     }
+                }
                 if (__all_sync(0xffffffffu, !on || q >= kSaturated)) break;
             }
         }
-        part[warp][lane] = combine_lanes(Q, lane);
-        __syncthreads();
-        if (warp == 0) {
-            float q = part[0][lane];
-            for (int w = 1; w < nw; ++w) {
-                const float o = part[w][lane];
-                q = fmaf(q, o, q + o);
+        float q = combine_lanes(Q, lane);
+        if (w.heavy) {
+            part[warp][lane] = q;
+            __syncthreads();
+            if (warp) continue;
+            for (int o = 1; o < kFwdWarps; ++o) {
+                const float r = part[o][lane];
+                q = fmaf(q, r, q + r);
             }
-            float l = 0.0f, wpx = 0.0f;
-            const bool mv = on && ((a.mask[(size_t)i * a.Wq + (j >> 5)] >> (j & 31)) & 1u);
-            if (on) {
-                const bool sat = q >= kOne;
-                const float om = sat ? 0.0f : __frcp_rn(1.0f + q);  // 1 - S
-                const float S = sat ? 1.0f : q * om;
-                const float e = mv ? -om : S;
-                l = e * e;
-                wpx = 2.0f * e * om * inv_s;
-            }
-            if (a.grad) a.wp[(((size_t)c * a.nby + by) * a.nbx + bx) * kBlkPx + lane] = wpx;
-            const int m = __popc(__ballot_sync(0xffffffffu, mv));
-            for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-            if (lane == 0)  // squared error minus the mask pixels counted in advance: exact sums, in any order
-                atomicAdd(a.lsum + c, (unsigned long long)__double2ll_rn((double)l * kLossScale) -
-                                          ((unsigned long long)m << 32));
         }
+        float l = 0.0f, wpx = 0.0f;
+        const bool mv = on && ((a.mask[(size_t)i * a.Wq + (j >> 5)] >> (j & 31)) & 1u);
+        if (on) {
+            const bool sat = q >= kOne;
+            const float om = sat ? 0.0f : __frcp_rn(1.0f + q);  // 1 - S
+            const float S = sat ? 1.0f : q * om;
+            const float e = mv ? -om : S;
+            l = e * e;
+            wpx = 2.0f * e * om * inv_s;
+        }
+        if (a.grad) a.wp[(((size_t)c * a.nby + w.by) * a.nbx + w.bx) * kBlkPx + lane] = wpx;
+        const int m = __popc(__ballot_sync(0xffffffffu, mv));
+        for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0)  // squared error minus the mask pixels counted in advance: exact sums, in any order
+            atomicAdd(a.lsum + c, (unsigned long long)__double2ll_rn((double)l * kLossScale) -
+                                      ((unsigned long long)m << 32));
     }
     // the last block to run out of work writes the losses
+    __syncthreads();
     if (tid == 0) {
         __threadfence();
-        s_it = atomicAdd(&a.ctl[2], 1u) == gridDim.x - 1;
+        s_it = atomicAdd(&a.ctl[kFwdExit], 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (s_it) {
@@ -728,139 +851,141 @@ __global__ void __launch_bounds__(32 * kFwdWarps) k_soft_fwd(SoftArgs a)
     }
 }
 
-// dL/d(u, v) of a group's triangles over a part of the group's window, one
-// triangle per lane.  With c the closest boundary point, at parameter t of edge
-// k, the signed distance d changes with c by -(p - c) / d, and c follows the
-// edge's ends by 1 - t and t.  The sums are kept in the edges' frames: Wb and
-// Wt for the part across the edge (all of it, and weighted by the position
-// along the edge), U0 and U1 for the part along it (only beyond an end).
-// Bound by instruction issue (82 %): 5.6 ms at 640x512, 20k triangles, 64
-// candidates (a warp per triangle and tile with its lanes on the pixels, six
-// values reduced over the warp for each: 24 ms, the forward again included).
+// dL/d(u, v) of the triangles over two blocks of pixels, one triangle per lane.
+// With c the closest boundary point, at parameter t of edge k, the signed
+// distance d changes with c by -(p - c) / d, and c follows the edge's ends by
+// 1 - t and t.  The sums are kept in the edges' frames: the parts along the
+// edge (U: only beyond an end) and across it (W), all of them and weighted by
+// the position of c on the edge (from its middle).
+// The blocks are the forward's, two at a time (half the atomic additions for a
+// few more idle lanes); light and heavy ones as there.  Bound by issue: 1.03
+// and 2.53 ms for the forward's scenes above.  With the groups walking the whole
+// of their windows, one set of additions per triangle, 18-21 % of the lanes
+// had a pair within reach (here 60 %): 5.6 ms for the second scene.
 struct EdgeSums {
-    float U0[3], U1[3], Wb[3], Wt[3];
+    float U[3], Ut[3], W[3], Wt[3];
 };
 
-__device__ __forceinline__ void bwd_pixel(const BlockEdges &e, const float (&ar)[3], const float (&br)[3], int px,
-                                          float w, EdgeSums &s)
+__device__ __forceinline__ void bwd_pixel(const BlockEdges &e, int px, float w, EdgeSums &s)
 {
-    float d2[3], bb[3], lo[3], hi[3], av[3];
+    float d2[3], b[3], o[3], f[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        av[k] = fmaf((float)px, e.tx[k], ar[k]);
-        bb[k] = fmaf(-(float)px, e.ty[k], br[k]);
-        lo[k] = fminf(av[k], 0.0f);
-        hi[k] = fmaxf(av[k] - e.L[k], 0.0f);
-        d2[k] = fmaf(bb[k], bb[k], fmaf(lo[k], lo[k], hi[k] * hi[k]));
+        const float a = fmaf((float)px, e.tx[k], e.a[k]);
+        b[k] = fmaf(-(float)px, e.ty[k], e.b[k]);
+        const float over = __saturatef(fabsf(a) - e.h[k]);
+        d2[k] = fmaf(over, over, fmaf(b[k], b[k], 1e-30f));  // never zero
+        o[k] = with_sign(over, a);
+        f[k] = a - o[k];
     }
-    const float m2 = min3(d2[0], d2[1], d2[2]);
-    const bool k0 = d2[0] == m2, k1 = !k0 && d2[1] == m2;
-    const float m2c = fmaxf(m2, 1e-30f), ir = rsq(m2c);
-    const float mb = min3(bb[0], bb[1], bb[2]);
-    const float x = with_sign(m2c * ir, mb);
-    const float sg = rcp_(1.0f + ex2(-x));
+    const float m = min3(d2[0], d2[1], d2[2]);
+    const float ir = with_sign(rsq(m), min3(b[0], b[1], b[2]));
+    const float d = m * ir;
+    const float sg = rcp_(1.0f + ex2(d * -kExpScale));
     // outside: d = -|p - c|, the sum grows along p - c; inside the other way
-    float g = __uint_as_float(__float_as_uint(w * sg * ir) ^ (~__float_as_uint(mb) & 0x80000000u));
-    g = x >= kCutLog2 ? g : 0.0f;
-    const float gk[3] = {k0 ? g : 0.0f, k1 ? g : 0.0f, (k0 || k1) ? 0.0f : g};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        s.U0[k] = fmaf(gk[k], lo[k], s.U0[k]);
-        s.U1[k] = fmaf(gk[k], hi[k], s.U1[k]);
-        const float h = gk[k] * bb[k];
-        s.Wb[k] += h;
-        s.Wt[k] = fmaf(h, av[k] - lo[k] - hi[k], s.Wt[k]);
-    }
+    const float v = w * sg * -ir;
+    // the nearest edge (the first of equal ones) takes it, none beyond the cutoff
+    asm("{\n\t"
+        ".reg .pred in, p0, r, p1, p2;\n\t"
+        ".reg .f32 u, x;\n\t"
+        "setp.gt.f32 in, %12, 0fBF800000;\n\t"
+        "setp.eq.and.f32 p0|r, %13, %16, in;\n\t"
+        "setp.eq.and.f32 p1|p2, %14, %16, r;\n\t"
+        "@p0 mul.f32 u, %17, %18;\n\t"
+        "@p0 mul.f32 x, %17, %19;\n\t"
+        "@p0 add.f32 %0, %0, u;\n\t"
+        "@p0 fma.rn.f32 %3, u, %20, %3;\n\t"
+        "@p0 add.f32 %6, %6, x;\n\t"
+        "@p0 fma.rn.f32 %9, x, %20, %9;\n\t"
+        "@p1 mul.f32 u, %17, %21;\n\t"
+        "@p1 mul.f32 x, %17, %22;\n\t"
+        "@p1 add.f32 %1, %1, u;\n\t"
+        "@p1 fma.rn.f32 %4, u, %23, %4;\n\t"
+        "@p1 add.f32 %7, %7, x;\n\t"
+        "@p1 fma.rn.f32 %10, x, %23, %10;\n\t"
+        "@p2 mul.f32 u, %17, %24;\n\t"
+        "@p2 mul.f32 x, %17, %25;\n\t"
+        "@p2 add.f32 %2, %2, u;\n\t"
+        "@p2 fma.rn.f32 %5, u, %26, %5;\n\t"
+        "@p2 add.f32 %8, %8, x;\n\t"
+        "@p2 fma.rn.f32 %11, x, %26, %11;\n\t"
+        "}"
+        : "+f"(s.U[0]), "+f"(s.U[1]), "+f"(s.U[2]), "+f"(s.Ut[0]), "+f"(s.Ut[1]), "+f"(s.Ut[2]), "+f"(s.W[0]),
+          "+f"(s.W[1]), "+f"(s.W[2]), "+f"(s.Wt[0]), "+f"(s.Wt[1]), "+f"(s.Wt[2])
+        : "f"(d), "f"(d2[0]), "f"(d2[1]), "f"(d2[2]), "f"(m), "f"(v), "f"(o[0]), "f"(b[0]), "f"(f[0]), "f"(o[1]),
+          "f"(b[1]), "f"(f[1]), "f"(o[2]), "f"(b[2]), "f"(f[2]));
 }
 
-__global__ void __launch_bounds__(128) k_soft_bwd(SoftArgs a)
+constexpr int kBwdRows = 2 * kBlkH;  // the backward takes a block and the one below
+
+__global__ void __launch_bounds__(32 * kBwdWarps, 5) k_soft_bwd(SoftArgs a)
 {
-    const int lane = threadIdx.x & 31;
-    const float k2 = kLog2e / a.sigma;
-    const float reach = kSoftCutoff * a.sigma + 0.01f, reach2 = reach * reach;
-    const int n_units = (int)a.ctl[3];
-    for (;;) {  // a warp per unit
-        int u = 0;
-        if (lane == 0) u = (int)atomicAdd(&a.ctl[4], 1u);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= n_units) return;
-        const int2 un = a.units[u];
-        const int c = un.x, g = un.y / kBwdMaxSeg, seg = un.y % kBwdMaxSeg;
-        const short4 win = a.gwin[(size_t)c * a.ngroups + g];
-        const int bw = win.z - win.x + 1, nb = bw * (win.w - win.y + 1), ns = bwd_segments(nb);
-        const int per = (nb + ns - 1) / ns, q1 = min(nb, (seg + 1) * per);
-        const int t = g * 32 + lane;
-        const size_t ti = (size_t)c * a.NTp + t;
-        const float4 box = a.box[ti];
-        const bool drawn = box.x < INFINITY;
-        TriRec r;
-        if (drawn) {
-            r = load_rec(a, ti);
-        } else {
+    __shared__ int queue[kBwdWarps][64];
+    __shared__ float s_w[kBwdWarps][kBwdRows * kBlkW];
+    __shared__ int s_it;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float unit = 1.0f / (kSoftCutoff * a.sigma);
+    Work w(a, kBwdHeavy);
+    while (w.next(a, kBwdHeavy, a.bwd, a.lam * ((a.nby + 1) / 2) * a.nbx, &s_it)) {
+        const int c = w.c;
+        float *sw = s_w[warp];  // the pixels' factors, a copy for every warp
+        unsigned nzh[2];
+        const size_t blk = ((size_t)c * a.nby + w.by) * a.nbx + w.bx;
+        __syncwarp();
 #pragma unroll
-            for (int k = 0; k < 3; ++k) r.x[k] = r.y[k] = 1e5f, r.tx[k] = r.ty[k] = r.L[k] = 0.0f;
-            r.orient = 0.0f;
+        for (int h = 0; h < 2; ++h) {
+            const size_t q = blk + (size_t)h * a.nbx;
+            const float v = w.by + h < a.nby && a.count[q] > 0 ? a.wp[q * kBlkPx + lane] : 0.0f;
+            sw[h * kBlkPx + lane] = v;
+            nzh[h] = __ballot_sync(0xffffffffu, v != 0.0f);
         }
-        EdgeSums tot{};
-        bool any = false;
-        for (int q = seg * per; q < q1; ++q) {
-            const int by = win.y + q / bw, bx = win.x + q % bw;
-            const bool near = drawn && box_near(box, bx, by, reach2);
-            if (!__any_sync(0xffffffffu, near)) continue;
-            const float wl = a.wp[(((size_t)c * a.nby + by) * a.nbx + bx) * kBlkPx + lane];
-            const unsigned nz = __ballot_sync(0xffffffffu, wl != 0.0f);
-            if (!nz) continue;
-            any = true;
-            BlockEdges e = block_edges(r, bx, by, k2);
-            if (!near) {  // out of reach of this block (or not drawn): far outside
-#pragma unroll
-                for (int k = 0; k < 3; ++k) e.b[k] = -1e4f, e.tx[k] = e.ty[k] = 0.0f;
-            }
+        const unsigned long long nz = (unsigned long long)nzh[1] << 32 | nzh[0];
+        if (!nz) continue;
+        __syncwarp();
+        const size_t tb = (size_t)c * a.NTp;
+        Collector<kBwdRows> col(a, c, w.bx, w.by, warp, w.heavy ? kBwdWarps : 1, queue[warp]);
+        int tn;
+        bool more = col.next(lane, tn);
+        while (more) {
+            const int t = tn;
+            const TriRec r = load_rec(a, tb + max(t, 0));
+            more = col.next(lane, tn);
+            BlockEdges e = block_edges(r, t >= 0, w.bx, w.by, unit);
             EdgeSums s{};
-            for (int py = 0; py < kBlkH; ++py) {
-                const unsigned row = (nz >> (kBlkW * py)) & ((1u << kBlkW) - 1u);
+            for (int py = 0; py < kBwdRows; ++py) {
+                const unsigned row = (unsigned)(nz >> (kBlkW * py)) & ((1u << kBlkW) - 1u);
                 if (row) {
 #pragma unroll
                     for (int px = 0; px < kBlkW; ++px)
-                        if (row >> px & 1u)
-                            bwd_pixel(e, e.a, e.b, px, __shfl_sync(0xffffffffu, wl, kBlkW * py + px), s);
+                        if (row >> px & 1u) bwd_pixel(e, px, sw[kBlkW * py + px], s);
                 }
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    e.a[k] += e.ty[k];
-                    e.b[k] += e.tx[k];
-                }
+                e.down();
             }
+            if (t < 0) continue;
+            float gx[3] = {0.0f, 0.0f, 0.0f}, gy[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                tot.U0[k] += s.U0[k];
-                tot.U1[k] += s.U1[k];
-                tot.Wb[k] += s.Wb[k];
-                tot.Wt[k] += s.Wt[k];
+                const int k1 = k == 2 ? 0 : k + 1;
+                const float h = 0.5f * r.L[k] * unit, i2h = h > 0.0f ? 0.5f / h : 0.0f;
+                // the ends' shares: t = (f + h) / 2h, and what is left
+                const float u1 = fmaf(h, s.U[k], s.Ut[k]) * i2h, u0 = s.U[k] - u1;
+                const float w1 = fmaf(h, s.W[k], s.Wt[k]) * i2h, w0 = s.W[k] - w1;
+                gx[k] += r.tx[k] * u0 - r.ty[k] * w0;
+                gy[k] += r.ty[k] * u0 + r.tx[k] * w0;
+                gx[k1] += r.tx[k] * u1 - r.ty[k] * w1;
+                gy[k1] += r.ty[k] * u1 + r.tx[k] * w1;
             }
-        }
-        if (!any || !drawn) continue;
-        float gx[3] = {0.0f, 0.0f, 0.0f}, gy[3] = {0.0f, 0.0f, 0.0f};
+            const int b = t >= a.T;
+            const int4 tri = a.tris[t - b * a.T];
+            const int id[3] = {tri.x, r.orient > 0.0f ? tri.y : tri.z, r.orient > 0.0f ? tri.z : tri.y};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int k1 = k == 2 ? 0 : k + 1;
-            const float iL = r.L[k] > 0.0f ? 1.0f / (r.L[k] * k2) : 0.0f;
-            const float b1 = tot.Wt[k] * iL, b0 = tot.Wb[k] - b1;
-            gx[k] += r.tx[k] * tot.U0[k] - r.ty[k] * b0;
-            gy[k] += r.ty[k] * tot.U0[k] + r.tx[k] * b0;
-            gx[k1] += r.tx[k] * tot.U1[k] - r.ty[k] * b1;
-            gy[k1] += r.ty[k] * tot.U1[k] + r.tx[k] * b1;
-        }
-        const int b = t >= a.T;
-        const int4 tri = a.tris[t - b * a.T];
-        const int id[3] = {tri.x, r.orient > 0.0f ? tri.y : tri.z, r.orient > 0.0f ? tri.z : tri.y};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {  // fixed point: the sums do not depend on the order of the additions
-            unsigned long long *gp =
-                reinterpret_cast<unsigned long long *>(a.gv + ((size_t)c * a.nI + b) * a.V + id[k]);
-            const long long vx = to_fixed(gx[k], kGvScale), vy = to_fixed(gy[k], kGvScale);
-            if (vx) atomicAdd(gp, (unsigned long long)vx);
-            if (vy) atomicAdd(gp + 1, (unsigned long long)vy);
+            for (int k = 0; k < 3; ++k) {  // fixed point: the sums do not depend on the order of the additions
+                unsigned long long *gp =
+                    reinterpret_cast<unsigned long long *>(a.gv + ((size_t)c * a.nI + b) * a.V + id[k]);
+                const long long vx = to_fixed(gx[k], kGvScale), vy = to_fixed(gy[k], kGvScale);
+                if (vx) atomicAdd(gp, (unsigned long long)vx);
+                if (vy) atomicAdd(gp + 1, (unsigned long long)vy);
+            }
         }
     }
 }
@@ -868,10 +993,10 @@ __global__ void __launch_bounds__(128) k_soft_bwd(SoftArgs a)
 // Per (candidate, instrument): dL/dX of every vertex, G_f = sum over the
 // frame's vertices of dL/dX [v; 1]^T; the candidate's last block contracts
 // dL/dtheta_k = sum_f <G_f, dT_f/dtheta_k>.  The sums are fixed-point integers,
-// so a call's results do not vary from run to run.  A warp takes 256
-// consecutive vertices (mostly of one frame: a link's vertices are
-// contiguous), eight per lane.
-constexpr int kRedVerts = 8;
+// so a call's results do not vary from run to run.  A warp takes 64
+// consecutive vertices (mostly of one frame: a link's vertices are contiguous),
+// two per lane.
+constexpr int kRedVerts = 2;
 
 __global__ void __launch_bounds__(kSoftThreads) k_soft_reduce(SoftArgs a)
 {
@@ -1075,15 +1200,16 @@ size_t soft_layout(SoftArgs &a, int lam, bool grad, char *base)
     take(a.rec, 4 * nt);
     take(a.box, nt);
     take(a.gwin, L * a.ngroups);
-    take(a.active, L * a.nby * a.wpr);
-    take(a.items, L * nb);
-    take(a.ctl, 8);
+    take(a.swin, L * a.nsup);
+    take(a.count, L * nb);
+    take(a.fwd, L * nb);
+    take(a.ctl, kCtl);
     take(a.rdone, L);
     take(a.lsum, L);
     take(a.Tf, fr * 12);
     take(a.dT, fr * 9 * 12);
     if (grad) {
-        take(a.units, L * a.ngroups * kBwdMaxSeg);
+        take(a.bwd, L * ((a.nby + 1) / 2) * a.nbx);
         take(a.wp, L * nb * kBlkPx);
         take(a.gv, L * a.nI * a.V);
         take(a.G, fr * 24);
@@ -1104,9 +1230,9 @@ void soft_shape(SoftArgs &a, const trk_tracker *t)
     a.Wq = t->cam.Wq;
     a.nbx = (a.W + kBlkW - 1) / kBlkW;
     a.nby = (a.H + kBlkH - 1) / kBlkH;
-    a.wpr = (a.nbx + 31) / 32;
     a.ngroups = (int)(((long long)a.nI * a.T + 31) / 32);
     a.NTp = 32 * a.ngroups;
+    a.nsup = (a.ngroups + 31) / 32;
 }
 
 // The largest slice of a call on lam candidates (at least one).
@@ -1139,7 +1265,7 @@ trk_status soft_scratch(trk_tracker *t, int lam, bool grad, SoftScratch **out)
     if ((e = cudaMalloc(&s->mem, bytes)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, t->device)) != cudaSuccess ||
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fwd, k_soft_fwd, 32 * kFwdWarps, 0)) != cudaSuccess ||
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bwd, k_soft_bwd, 128, 0)) != cudaSuccess) {
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bwd, k_soft_bwd, 32 * kBwdWarps, 0)) != cudaSuccess) {
         soft_free(t);
         return soft_fail(e == cudaErrorMemoryAllocation ? TRK_ENOMEM : TRK_ECUDA, cudaGetErrorString(e));
     }
@@ -1182,9 +1308,11 @@ trk_status soft_launch(trk_tracker *t, const float *params, int lam, const uint3
             k_soft_tris<<<dim3((a.ngroups + gpb - 1) / gpb, a.lam), kSoftThreads, a.nI * a.nF * 12 * sizeof(float),
                           st>>>(a);
         }
+        const int pairs = (a.nby + 1) / 2 * a.nbx;
+        k_soft_list<<<dim3((pairs + kSoftThreads - 1) / kSoftThreads, a.lam), kSoftThreads, 0, st>>>(a);
         k_soft_fwd<<<s->fwd_grid, 32 * kFwdWarps, 0, st>>>(a);
         if (grad) {
-            if (a.ngroups) k_soft_bwd<<<s->bwd_grid, 128, 0, st>>>(a);
+            if (a.ngroups) k_soft_bwd<<<s->bwd_grid, 32 * kBwdWarps, 0, st>>>(a);
             const int vpb = kSoftThreads * kRedVerts;
             k_soft_reduce<<<dim3(std::max(1, (a.V + vpb - 1) / vpb), a.lam * a.nI), kSoftThreads, 0, st>>>(a);
         }
