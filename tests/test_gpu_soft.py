@@ -206,3 +206,21 @@ def test_soft_results_do_not_depend_on_the_population(api):
         l1, g1 = tr.soft_eval(P[c:c + 1].contiguous(), Mp, grad=True)
         assert torch.equal(l1.view(torch.int32), loss[c:c + 1].view(torch.int32)), c
         assert torch.equal(g1.view(torch.int32), g[c:c + 1].view(torch.int32)), c
+
+
+def test_autograd_forms_give_the_same_bits(api):
+    """The op with the gradient taken along in the forward, the op that
+    evaluates it in the backward, no_grad and a non-contiguous input."""
+    sc, tr, M, Mp, P = _case(api, "c1", "c1", 1, None, 43, 5)
+    wide = torch.from_numpy(np.repeat(P, 2, axis=1)).cuda()
+    w = torch.arange(1, 6, dtype=torch.float32, device="cuda")
+    l0, g0 = tr.soft_eval(torch.from_numpy(P).cuda(), Mp, grad=True)
+    for x in (torch.from_numpy(P).cuda().requires_grad_(True), wide.requires_grad_(True)):
+        y = x if x.shape[1] == 9 else x[:, ::2]
+        for L in (api.soft_silhouette_loss(y, tr, Mp), api.SoftSilhouetteLoss.apply(y, tr, Mp)):
+            assert torch.equal(L, l0)
+            (g,) = torch.autograd.grad(L, y, w, retain_graph=True)
+            assert torch.equal(g, w[:, None] * g0)
+            assert torch.equal(torch.autograd.grad(L, y, w)[0], g)
+    with torch.no_grad():
+        assert torch.equal(api.soft_silhouette_loss(torch.from_numpy(P).cuda().requires_grad_(True), tr, Mp), l0)
