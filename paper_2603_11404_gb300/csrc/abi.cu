@@ -9,6 +9,8 @@
 #include <algorithm>
 #include <new>
 #include <string>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 #include "internal.cuh"
@@ -72,6 +74,71 @@ static void binned_free(BinDev &b)
     b = BinDev{};
 }
 
+// The mesh's directed edges by their first end: entries start[u] .. start[u + 1]
+// hold (second end << 32 | triangle) in increasing order.
+struct EdgeLists {
+    std::vector<int> start;
+    std::vector<uint64_t> e;
+
+    // corners renamed by id (NULL: as they are)
+    EdgeLists(const std::vector<int4> &tris, long long T, long long V, const int *id)
+        : start((size_t)V + 1, 0), e((size_t)(3 * T))
+    {
+        auto corner = [&](int t, int k) {
+            const int4 &r = tris[t];
+            const int c = k == 0 ? r.x : (k == 1 ? r.y : r.z);
+            return id ? id[c] : c;
+        };
+        for (int t = 0; t < (int)T; ++t)
+            for (int k = 0; k < 3; ++k) ++start[corner(t, k) + 1];
+        for (size_t u = 0; u + 1 < start.size(); ++u) start[u + 1] += start[u];
+        std::vector<int> at(start.begin(), start.end() - 1);
+        for (int t = 0; t < (int)T; ++t)
+            for (int k = 0; k < 3; ++k)
+                e[at[corner(t, k)]++] = (uint64_t)(uint32_t)corner(t, (k + 1) % 3) << 32 | (uint32_t)t;
+        for (size_t u = 0; u + 1 < start.size(); ++u) std::sort(e.begin() + start[u], e.begin() + start[u + 1]);
+    }
+
+    // the entries of edges u -> v
+    std::pair<const uint64_t *, const uint64_t *> find(int u, int v) const
+    {
+        const uint64_t *lo = e.data() + start[u], *hi = e.data() + start[u + 1];
+        lo = std::lower_bound(lo, hi, (uint64_t)(uint32_t)v << 32);
+        const uint64_t *end = lo;
+        while (end < hi && (uint32_t)(*end >> 32) == (uint32_t)v) ++end;
+        return {lo, end};
+    }
+
+    // is every edge traversed equally often in both directions?
+    bool cancel() const
+    {
+        for (int u = 0; u + 1 < (int)start.size(); ++u)
+            for (int i = start[u], j; i < start[u + 1]; i = j) {
+                const int v = (int)(e[i] >> 32);
+                for (j = i; j < start[u + 1] && (int)(e[j] >> 32) == v; ++j) {
+                }
+                const auto r = find(v, u);
+                if (r.second - r.first != j - i) return false;
+            }
+        return true;
+    }
+};
+
+// A closed surface, also one whose faces carry vertices of their own: corners
+// at one place of one frame project to the same point, so they count as one.
+static bool mesh_closed(const EdgeLists &edges, const std::vector<float4> &verts, const std::vector<int4> &tris,
+                        long long V, long long T)
+{
+    if (edges.cancel()) return true;
+    std::vector<int> order((size_t)V), id((size_t)V);
+    for (int i = 0; i < (int)V; ++i) order[i] = i;
+    auto key = [&](int i) { return std::make_tuple(verts[i].w, verts[i].x, verts[i].y, verts[i].z); };
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
+    for (size_t i = 0; i < order.size(); ++i)
+        id[order[i]] = i && key(order[i]) == key(order[i - 1]) ? id[order[i - 1]] : order[i];
+    return EdgeLists(tris, T, V, id.data()).cancel();
+}
+
 // The mesh as primitives for the fitness kernel: triangles that share an edge
 // with opposite directions (a consistently wound pair) become one record
 // (a, b, c, d) for the triangles (a, b, c) and (a, c, d); the rest stay single
@@ -80,23 +147,8 @@ static void binned_free(BinDev &b)
 // the mesh's order (neighbouring records draw neighbouring pixels).  Whether a
 // pair is drawn as one quadrilateral is decided per candidate on the device
 // (convexity of the projected corners); the union of pixels is the same.
-static std::vector<int4> pair_triangles(const std::vector<int4> &tris, long long T)
+static std::vector<int4> pair_triangles(const std::vector<int4> &tris, long long T, const EdgeLists &edges)
 {
-    struct DirEdge {
-        int u, v, t;
-    };
-    std::vector<DirEdge> edges;
-    edges.reserve((size_t)(3 * T));
-    for (int t = 0; t < (int)T; ++t) {
-        const int4 &r = tris[t];
-        edges.push_back({r.x, r.y, t});
-        edges.push_back({r.y, r.z, t});
-        edges.push_back({r.z, r.x, t});
-    }
-    auto key_less = [](const DirEdge &a, const DirEdge &b) {
-        return a.u != b.u ? a.u < b.u : (a.v != b.v ? a.v < b.v : a.t < b.t);
-    };
-    std::sort(edges.begin(), edges.end(), key_less);
     std::vector<char> taken((size_t)std::max<long long>(T, 1), 0);
     std::vector<int4> prims;
     prims.reserve((size_t)T);
@@ -108,9 +160,9 @@ static std::vector<int4> pair_triangles(const std::vector<int4> &tris, long long
         for (int k = 0; k < 3; ++k) {
             const int u = c[k], v = c[(k + 1) % 3];
             // triangles holding the reverse edge v -> u
-            auto it = std::lower_bound(edges.begin(), edges.end(), DirEdge{v, u, 0}, key_less);
-            for (; it != edges.end() && it->u == v && it->v == u; ++it) {
-                const int o = it->t;
+            const auto rev = edges.find(v, u);
+            for (const uint64_t *it = rev.first; it != rev.second; ++it) {
+                const int o = (int)(uint32_t)*it;
                 if (taken[o] || (best >= 0 && o >= best)) continue;
                 const int4 &r = tris[o];
                 const int w = r.x + r.y + r.z - u - v;  // the other triangle's third corner
@@ -329,7 +381,9 @@ trk_status tracker_create(const trk_link_mesh *meshes, int32_t n_meshes, const t
         vb += m.n_verts;
         tb += m.n_tris;
     }
-    std::vector<int4> hp = pair_triangles(ht, T);
+    const EdgeLists edges(ht, T, std::max<long long>(V, 1), nullptr);
+    t->closed = mesh_closed(edges, hv, ht, V, T);
+    std::vector<int4> hp = pair_triangles(ht, T, edges);
     // draw order: the reverse of the mesh's.  Instrument meshes list the links
     // from the shaft to the jaws and the shaft from its far end, so the tip
     // (the largest primitives on screen) is drawn first and the small far end

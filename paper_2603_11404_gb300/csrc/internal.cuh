@@ -73,7 +73,9 @@ struct __align__(16) EvalArgs {
     // and (a, c, d) sharing the edge a-c, (a, b, c, -1) a single triangle; NULL
     // in the index-checked launch, which draws tris[]
     const int4 *prims;
-    int P, pad_p;
+    // closed: every edge of the mesh is traversed equally often in both
+    // directions, so its front faces alone cover the silhouette (see draw_prims)
+    int P, closed;
     const float *params;   // [lam * d]
     int d, lam;
     const uint32_t *mask;  // packed [H * Wq]
@@ -240,6 +242,7 @@ struct trk_tracker {
     int4 *tris = nullptr;
     int4 *prims = nullptr;     // the mesh as quadrilateral pairs and single triangles (EvalArgs::prims)
     int P = 0;
+    bool closed = false;       // EvalArgs::closed
     int2 *snap = nullptr;       // scratch [lambda_max * n_inst * V]
     int raster = 0;             // TRK_RASTER_CLUSTER or TRK_RASTER_BINNED (resolved at create)
     trk::BinDev bin{};          // binned pipeline scratch (raster == TRK_RASTER_BINNED)
@@ -265,6 +268,7 @@ inline void apply_mesh(trk::EvalArgs &a, const trk_tracker *t)
     a.T = t->T;
     a.prims = t->prims;
     a.P = t->P;
+    a.closed = t->closed ? 1 : 0;
 }
 
 // The tracker's keypoint term into a launch's arguments.

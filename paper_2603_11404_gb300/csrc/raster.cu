@@ -34,6 +34,7 @@ namespace cg = cooperative_groups;
 
 namespace trk {
 
+constexpr int kAccWords = 12;  // counters behind the deferred list (see eval_candidate)
 
 // Projected keypoints of given states (synthetic detections, diagnostics):
 // one warp per state composes its frames and writes (u, v) of both keypoints
@@ -120,11 +121,11 @@ __device__ __forceinline__ bool small_box(int spanx, int spany) { return spanx <
 // a whole warp through the CTA's list (entry `ent`).  Returns 1 when the
 // triangle is culled for a flagged vertex.
 template <bool kInlineFallback>
-__device__ __forceinline__ int draw_one_tri(int2 v0, int2 v1, int2 v2, int ent, const EvalArgs &a, uint32_t *bm,
-                                            int *big, int *sacc)
+__device__ __forceinline__ int draw_one_tri(int2 v0, int2 v1, int2 v2, int ent, const EvalArgs &a, int cull,
+                                            uint32_t *bm, int *big, int *sacc)
 {
     TriSetup t;
-    const int st = tri_setup(v0, v1, v2, a.cam.W, a.cam.H, a.cull, t);
+    const int st = tri_setup(v0, v1, v2, a.cam.W, a.cam.H, cull, t);
     if (st == 1) {
         if (small_box(t.spanx, t.spany)) {
             raster_small(t, bm, a.cam.Wq);
@@ -164,14 +165,14 @@ __device__ __forceinline__ void gather_prim(const EvalArgs &a, const int2 *snapc
 // pass, anything else as its triangles; large ones are deferred to a whole
 // warp.  Returns the number of its triangles culled for a flagged vertex.
 template <bool kInlineFallback>
-__device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int t, int d, int2 v0, int2 v1, int2 v2, int2 v3,
+__device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int cull, int t, int d, int2 v0, int2 v1, int2 v2, int2 v3,
                                               uint32_t *bm, int *big, int *sacc)
 {
     const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
     int st = 3, culled = 0;
     if (d >= 0) {
         QuadSetup q;
-        st = quad_setup(v0, v1, v2, v3, W, H, a.cull, q);
+        st = quad_setup(v0, v1, v2, v3, W, H, cull, q);
         if (st == 1) {
             if (small_box(q.spanx, q.spany)) {
                 raster_quad_small(q, bm, Wq);
@@ -181,8 +182,8 @@ __device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int t, int d, i
                     big[slot] = 4 * t;
                 } else if constexpr (kInlineFallback) {
                     TriSetup ts;
-                    if (tri_setup(v0, v1, v2, W, H, a.cull, ts) == 1) raster_serial(ts, bm, Wq);
-                    if (tri_setup(v0, v2, v3, W, H, a.cull, ts) == 1) raster_serial(ts, bm, Wq);
+                    if (tri_setup(v0, v1, v2, W, H, cull, ts) == 1) raster_serial(ts, bm, Wq);
+                    if (tri_setup(v0, v2, v3, W, H, cull, ts) == 1) raster_serial(ts, bm, Wq);
                 } else {
                     sacc[6] = 1;
                 }
@@ -190,8 +191,8 @@ __device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int t, int d, i
         }
     }
     if (st == 3) {
-        culled += draw_one_tri<kInlineFallback>(v0, v1, v2, 4 * t + 1, a, bm, big, sacc);
-        if (d >= 0) culled += draw_one_tri<kInlineFallback>(v0, v2, v3, 4 * t + 2, a, bm, big, sacc);
+        culled += draw_one_tri<kInlineFallback>(v0, v1, v2, 4 * t + 1, a, cull, bm, big, sacc);
+        if (d >= 0) culled += draw_one_tri<kInlineFallback>(v0, v2, v3, 4 * t + 2, a, cull, bm, big, sacc);
     }
     return culled;
 }
@@ -199,7 +200,7 @@ __device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int t, int d, i
 // One deferred entry drawn by the whole warp into this CTA's bitmap: the
 // triangles of primitive ent / 4 (part 0 both, 1 the first, 2 the second), a
 // pixel per lane with int64 edge functions.
-__device__ __forceinline__ void draw_deferred(const EvalArgs &a, const int2 *snapc0, int ent, uint32_t *bm, int lane)
+__device__ __forceinline__ void draw_deferred(const EvalArgs &a, int cull, const int2 *snapc0, int ent, uint32_t *bm, int lane)
 {
     const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
     const int t = ent >> 2, part = ent & 3;
@@ -208,8 +209,8 @@ __device__ __forceinline__ void draw_deferred(const EvalArgs &a, const int2 *sna
     const int2 *sv = snapc0 + b * a.V;
     const int2 u0 = __ldcg(sv + p.x), u1 = __ldcg(sv + p.y), u2 = __ldcg(sv + p.z);
     TriSetup ts;
-    if (part != 2 && tri_setup(u0, u1, u2, W, H, a.cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
-    if (part != 1 && tri_setup(u0, u2, __ldcg(sv + p.w), W, H, a.cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
+    if (part != 2 && tri_setup(u0, u1, u2, W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
+    if (part != 1 && tri_setup(u0, u2, __ldcg(sv + p.w), W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
 }
 
 // Phase 2 over the tracker's primitive list (quadrilateral pairs and single
@@ -220,11 +221,11 @@ __device__ __forceinline__ void draw_deferred(const EvalArgs &a, const int2 *sna
 // 4 * primitive + part: part 0 the whole quadrilateral (its two triangles), 1
 // its first triangle (a, b, c), 2 its second (a, c, d); they are drawn after
 // the cluster barrier that follows, shared out over the whole cluster (in
-// eval_candidate).  Returns this thread's count of triangles culled for a
-// flagged vertex.
+// eval_candidate).  `cull` leaves out back faces.  Returns this thread's count
+// of triangles culled for a flagged vertex.
 template <bool kInlineFallback>
-__device__ __forceinline__ int draw_prims(const EvalArgs &a, cg::cluster_group &cluster, const int2 *snapc0, uint32_t *bm,
-                                          int *big, int *sacc, int lane, int warp, int nwarp)
+__device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::cluster_group &cluster, const int2 *snapc0,
+                                          uint32_t *bm, int *big, int *sacc, int lane, int warp, int nwarp)
 {
     const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
     const int NP = a.ch.n_inst * a.P, V = a.V, P = a.P;
@@ -239,7 +240,7 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, cg::cluster_group &
             const int4 p = load_prim(a, t);
             int2 v0, v1, v2, v3 = make_int2(0, 0);
             gather_prim(a, snapc0, t, p, v0, v1, v2, v3);
-            culled += draw_prim_lane<kInlineFallback>(a, t, p.w, v0, v1, v2, v3, bm, big, sacc);
+            culled += draw_prim_lane<kInlineFallback>(a, cull, t, p.w, v0, v1, v2, v3, bm, big, sacc);
         }
         cur = __shfl_sync(0xffffffffu, tk, 0);
     }
@@ -260,16 +261,16 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, cg::cluster_group &
                 if (p.w >= 0) {
                     const int2 u3 = __ldcg(sv + p.w);
                     QuadSetup q;
-                    st = quad_setup(u0, u1, u2, u3, W, H, a.cull, q);
+                    st = quad_setup(u0, u1, u2, u3, W, H, cull, q);
                     if (st == 1) l1 = l2 = !small_box(q.spanx, q.spany);
                     if (st == 3) {
                         TriSetup ts;
-                        l2 = tri_setup(u0, u2, u3, W, H, a.cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
+                        l2 = tri_setup(u0, u2, u3, W, H, cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
                     }
                 }
                 if (st == 3) {
                     TriSetup ts;
-                    l1 = tri_setup(u0, u1, u2, W, H, a.cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
+                    l1 = tri_setup(u0, u1, u2, W, H, cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
                 }
             }
             for (int part = 1; part <= 2; ++part)
@@ -282,7 +283,7 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, cg::cluster_group &
                     const int2 u1 = __ldcg(sv + (part == 1 ? p.y : p.z));
                     const int2 u2 = __ldcg(sv + (part == 1 ? p.z : p.w));
                     TriSetup ts;
-                    if (tri_setup(u0, u1, u2, W, H, a.cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
+                    if (tri_setup(u0, u1, u2, W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
                 }
         }
     }
@@ -323,7 +324,7 @@ __device__ __forceinline__ int draw_tris(const EvalArgs &a, cg::cluster_group &c
             b2 = t2 >= a.T;
             tri2 = load_tri<kChecked>(a, t2);
         }
-        if (t0 < NT) culled += draw_one_tri<kInlineFallback>(v0, v1, v2, t0, a, bm, big, sacc);
+        if (t0 < NT) culled += draw_one_tri<kInlineFallback>(v0, v1, v2, t0, a, a.cull, bm, big, sacc);
         cur = nx1;
         t0 = t1;
         v0 = w0;
@@ -390,8 +391,8 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     uint32_t *bm = reinterpret_cast<uint32_t *>(scr + nI * kComposeScratch);  // [H*Wq]
     float *sM = reinterpret_cast<float *>(bm + ((nwords + 3) & ~3));          // [nI*nF*24]
     int *big = reinterpret_cast<int *>(sM + nI * nF * 24);                    // [kBigListCap]
-    // [8]: s I m culled, big-list count, chunk ticket counter, big-list
-    // overflow, deferred-entry ticket counter
+    // [kAccWords]: s I m culled, big-list count, chunk ticket counter, big-list
+    // overflow, deferred-entry ticket counter, a vertex of this CTA is flagged
     int *sacc = big + kBigListCap;
     __shared__ int red[4][32];
     __shared__ float s_par[kMaxD];
@@ -403,7 +404,7 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
         uint4 *bm4 = reinterpret_cast<uint4 *>(bm);
         for (int w = tid - c0; w >= 0 && w < (nwords + 3) >> 2; w += nthr - c0) bm4[w] = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (tid < 8) sacc[tid] = 0;
+    if (tid < kAccWords) sacc[tid] = 0;
     // everything above touches only this CTA's shared memory; from here on the
     // launch reads what the previous generation wrote
     if (dependent_launch) griddep_wait();
@@ -462,6 +463,7 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
             if (a.snap_dbg) a.snap_dbg[(size_t)c * NV + idx1] = o1;
             if (a.uv_dbg) a.uv_dbg[(size_t)c * NV + idx1] = uv1;
         }
+        if (o0.x == kSnapFlag || (has1 && o1.x == kSnapFlag)) sacc[8] = 1;
     }
     cluster.sync();  // arrive.release / wait.acquire: the snapped vertices are visible cluster-wide
 
@@ -470,7 +472,16 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     //      shared memory, so the cluster finishes together whatever they cost;
     //      the bitmaps are OR-ed in phase 3, so which CTA draws a primitive does
     //      not change the result ----
-    int culled = kQuads ? draw_prims<kInlineFallback>(a, cluster, snapc, bm, big, sacc, lane, warp, nwarp)
+    // A closed mesh without a flagged vertex is drawn by its front faces
+    // alone: the edges of its triangles cancel in pairs, so the triangles that
+    // cover a pixel centre (see the quadrilateral rule: no centre lies on an
+    // edge) have as many positive as negative orientations among them -- a
+    // pixel that any triangle covers, some front face covers.  A flagged
+    // vertex drops triangles and opens the surface.
+    int cull = a.cull;
+    if (kQuads && a.closed)
+        cull |= !__any_sync(0xffffffffu, lane < K && *cluster.map_shared_rank(&sacc[8], lane < K ? lane : 0) != 0);
+    int culled = kQuads ? draw_prims<kInlineFallback>(a, cull, cluster, snapc, bm, big, sacc, lane, warp, nwarp)
                         : draw_tris<kInlineFallback, kChecked>(a, cluster, snapc, bm, big, sacc, lane, warp, nwarp);
     cluster.sync();
     if (kQuads) {
@@ -492,7 +503,7 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
                 const int r = __popc(__ballot_sync(0xffffffffu, lane < K && incl <= e));
                 const int start = __shfl_sync(0xffffffffu, incl - cnt, r);
                 const int ent = cluster.map_shared_rank(big, r)[e - start];
-                draw_deferred(a, snapc, ent, bm, lane);
+                draw_deferred(a, cull, snapc, ent, bm, lane);
             }
             cluster.sync();  // every deferred primitive drawn before the bitmaps are read
         }
@@ -708,7 +719,7 @@ size_t eval_smem_bytes(const EvalArgs &a)
 {
     size_t nwords = (size_t)a.cam.H * a.cam.Wq;
     return (size_t)a.ch.n_inst * kComposeScratch * sizeof(float2) + ((nwords + 3) & ~(size_t)3) * 4 +
-           (size_t)a.ch.n_inst * a.ch.n_frames * 24 * 4 + (size_t)kBigListCap * 4 + 8 * 4;
+           (size_t)a.ch.n_inst * a.ch.n_frames * 24 * 4 + (size_t)kBigListCap * 4 + kAccWords * 4;
 }
 
 int eval_max_threads() { return 1024; }

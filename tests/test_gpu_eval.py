@@ -480,3 +480,47 @@ def test_large_quads_deferred_over_the_cluster(api):
     for cull in (False, True):
         for cluster, threads in ((1, 64), (8, 256)):
             _check_population(api, sc, st, M, cull=cull, cluster=cluster, threads=threads)
+
+
+def _variant_scene(kind):
+    """A 101x77 scene on which the front-face rule applies or must not apply:
+    the closed instrument, the same with a vertex of its own per corner (closed
+    once corners at one place count as one), with one face missing, with half of
+    its faces wound the other way, and a single reversed triangle."""
+    K = wl.Intrinsics(150.0, 150.0, 50.0, 38.5, 101, 77)
+    if kind == "one":
+        sc = tiny_scene(101, 77, 100.0, [[-5, -5, 0], [6, -4, 1], [0, 7, -1]], [[0, 2, 1]])
+        return sc
+    sc = wl.make_scene("800", "c1", K=K)
+    meshes = []
+    for k, m in enumerate(sc.meshes):
+        v, t = m.verts, m.tris
+        if kind == "split":
+            v, t = v[t.reshape(-1)], np.arange(t.size, dtype=np.int32).reshape(-1, 3)
+        elif kind == "open" and k == 0:
+            t = np.delete(t, 40, axis=0)
+        elif kind == "wound" and k == 0:
+            t = t.copy()
+            t[::2] = t[::2, ::-1]
+        meshes.append(wl.LinkMesh(m.frame, np.ascontiguousarray(v), np.ascontiguousarray(t)))
+    sc.meshes[:] = meshes
+    return sc
+
+
+@pytest.mark.parametrize("kind", ["closed", "split", "open", "wound", "one"])
+@pytest.mark.parametrize("cull", [False, True])
+@pytest.mark.parametrize("cluster", [1, 0])
+def test_front_face_rule_and_its_exceptions(api, kind, cull, cluster):
+    """Candidates in view, close enough for the deferred list, and with a part
+    behind the camera (flagged vertices: every face is drawn)."""
+    sc = _variant_scene(kind)
+    rng = np.random.default_rng(61)
+    gt = wl.sample_state(rng, sc.K)
+    P = wl.population_around(rng, gt, 9, sigma_rad=0.3, sigma_mm=6.0)
+    P[3:5, 5] = 18.0   # close to the camera
+    P[5:7, 5] = 4.0    # partly behind it
+    P[6, :3] = [0.3, 0.2, 0.1]
+    M = random_mask(rng, 77, 101)
+    counts, _, _ = _check_population(api, sc, P, M, cull=cull, cluster=cluster, fk_tol=1e-3)
+    if kind == "closed":
+        assert (counts[:, 3] > 0).any() and (counts[:, 3] == 0).any() and counts[:, 0].max() > 50
