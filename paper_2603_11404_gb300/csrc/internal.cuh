@@ -105,7 +105,8 @@ struct __align__(16) EvalArgs {
     const float *kp_obs;
     BinDev bin;            // binned pipeline scratch (unused by the cluster-bitmap kernel)
     unsigned *err;         // the tracker's device error word (TRK_DEVERR_*), or NULL
-    int pad_err[2];
+    int qcap;              // entries per warp of the cluster-bitmap kernel's drawing queue
+    int pad_err;
 };
 
 struct LaunchCfg {
@@ -196,6 +197,7 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
 cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_clusters);
 cudaError_t launch_pack_mask(const uint8_t *mask, uint32_t *packed, int W, int H, int Wq, cudaStream_t s);
 size_t eval_smem_bytes(const EvalArgs &a);
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam);
 cudaError_t prepare_eval(size_t smem);
 void set_last_error(const char *msg);  // the text tracker_last_error() returns
 int eval_max_threads();
@@ -269,6 +271,7 @@ inline void apply_mesh(trk::EvalArgs &a, const trk_tracker *t)
     a.prims = t->prims;
     a.P = t->P;
     a.closed = t->closed ? 1 : 0;
+    a.qcap = trk::eval_queue_cap(t->ch, t->cam);
 }
 
 // The tracker's keypoint term into a launch's arguments.

@@ -34,6 +34,16 @@ namespace cg = cooperative_groups;
 
 namespace trk {
 
+// Front of the dynamic shared memory: the composition's scratch and, once the
+// frames are composed, the warps' drawing queues (at most 8 warps).
+constexpr int kQueueEntryBytes = 40;  // an entry of draw_rows' table; a queued primitive takes 32
+
+__host__ __device__ inline size_t front_smem_bytes(int n_inst, int qcap)
+{
+    const size_t scr = (size_t)n_inst * kComposeScratch * sizeof(float2), q = (size_t)8 * qcap * kQueueEntryBytes;
+    return scr > q ? scr : q;
+}
+
 constexpr int kAccWords = 12;  // counters behind the deferred list (see eval_candidate)
 
 // Projected keypoints of given states (synthetic detections, diagnostics):
@@ -161,40 +171,29 @@ __device__ __forceinline__ void gather_prim(const EvalArgs &a, const int2 *snapc
     if (p.w >= 0) v3 = __ldcg(sv + p.w);
 }
 
-// One primitive of phase 2 drawn by this lane: a convex quadrilateral in one
-// pass, anything else as its triangles; large ones are deferred to a whole
-// warp.  Returns the number of its triangles culled for a flagged vertex.
+// A large entry waits for a whole warp, unless none of its triangles is to be
+// drawn.  If the list is full: the plain launch redraws every large primitive
+// after the loop (raster code here would make its loop spill); the batched
+// launch, compiled with more registers, draws its triangles in this lane.
 template <bool kInlineFallback>
-__device__ __forceinline__ int draw_prim_lane(const EvalArgs &a, int cull, int t, int d, int2 v0, int2 v1, int2 v2, int2 v3,
-                                              uint32_t *bm, int *big, int *sacc)
+__device__ __forceinline__ void defer_large(int t, const PrimEntry &e, const EvalArgs &a, int cull, uint32_t *bm, int *big,
+                                            int *sacc)
 {
-    const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
-    int st = 3, culled = 0;
-    if (d >= 0) {
-        QuadSetup q;
-        st = quad_setup(v0, v1, v2, v3, W, H, cull, q);
-        if (st == 1) {
-            if (small_box(q.spanx, q.spany)) {
-                raster_quad_small(q, bm, Wq);
-            } else {
-                const int slot = atomicAdd(&sacc[4], 1);
-                if (slot < kBigListCap) {
-                    big[slot] = 4 * t;
-                } else if constexpr (kInlineFallback) {
-                    TriSetup ts;
-                    if (tri_setup(v0, v1, v2, W, H, cull, ts) == 1) raster_serial(ts, bm, Wq);
-                    if (tri_setup(v0, v2, v3, W, H, cull, ts) == 1) raster_serial(ts, bm, Wq);
-                } else {
-                    sacc[6] = 1;
-                }
-            }
-        }
+    const int W = a.cam.W, H = a.cam.H;
+    const bool pair = e.c3.x != kSnapFlag;
+    TriSetup ts;
+    const bool d1 = tri_setup(e.c0, e.c1, e.c2, W, H, cull, ts) == 1;
+    const bool d2 = pair && tri_setup(e.c0, e.c2, e.c3, W, H, cull, ts) == 1;
+    if (!d1 && !d2) return;
+    const int slot = atomicAdd(&sacc[4], 1);
+    if (slot < kBigListCap) {
+        big[slot] = 4 * t + e.part;
+    } else if constexpr (kInlineFallback) {
+        if (d1 && tri_setup(e.c0, e.c1, e.c2, W, H, cull, ts) == 1) raster_serial(ts, bm, a.cam.Wq);
+        if (d2 && tri_setup(e.c0, e.c2, e.c3, W, H, cull, ts) == 1) raster_serial(ts, bm, a.cam.Wq);
+    } else {
+        sacc[6] = 1;
     }
-    if (st == 3) {
-        culled += draw_one_tri<kInlineFallback>(v0, v1, v2, 4 * t + 1, a, cull, bm, big, sacc);
-        if (d >= 0) culled += draw_one_tri<kInlineFallback>(v0, v2, v3, 4 * t + 2, a, cull, bm, big, sacc);
-    }
-    return culled;
 }
 
 // One deferred entry drawn by the whole warp into this CTA's bitmap: the
@@ -216,33 +215,71 @@ __device__ __forceinline__ void draw_deferred(const EvalArgs &a, int cull, const
 // Phase 2 over the tracker's primitive list (quadrilateral pairs and single
 // triangles, prims[] of EvalArgs).  A warp takes a chunk of 32 primitives
 // (one per lane) from the cluster's counter and takes the next chunk's ticket
-// while it draws: a warp holds at most one chunk beyond the one it draws, so
-// the warps of a cluster run out of work together.  Deferred-list entries are
-// 4 * primitive + part: part 0 the whole quadrilateral (its two triangles), 1
-// its first triangle (a, b, c), 2 its second (a, c, d); they are drawn after
-// the cluster barrier that follows, shared out over the whole cluster (in
-// eval_candidate).  `cull` leaves out back faces.  Returns this thread's count
-// of triangles culled for a flagged vertex.
+// while it sets the current one up: a warp holds at most one chunk beyond the
+// one it works on, so the warps of a cluster run out of work together.
+// Set-up and drawing are apart: of the 32 primitives of a chunk five to ten are
+// front faces with a pixel centre in their box (640x512, 20k triangles).  The
+// warp queues those (EvalArgs::qcap entries in shared memory) and takes a full
+// queue at a time through the convexity test, the edge set-up and the drawing.
+// Deferred-list entries are 4 * primitive + part: part 0 the whole
+// quadrilateral (its two triangles), 1 its first triangle (a, b, c), 2 its
+// second (a, c, d); they are drawn after the cluster barrier that follows,
+// shared out over the whole cluster (in eval_candidate).  `cull` leaves out
+// back faces.  Returns this thread's count of triangles culled for a flagged
+// vertex.
 template <bool kInlineFallback>
 __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::cluster_group &cluster, const int2 *snapc0,
-                                          uint32_t *bm, int *big, int *sacc, int lane, int warp, int nwarp)
+                                          uint32_t *bm, int *big, int *sacc, int4 *queue, int lane, int warp, int nwarp)
 {
     const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
-    const int NP = a.ch.n_inst * a.P, V = a.V, P = a.P;
+    const int NP = a.ch.n_inst * a.P, V = a.V, P = a.P, cap = a.qcap;
     int culled = 0;
     int *ctr = cluster.map_shared_rank(&sacc[5], 0);
-    int cur = chunk_ticket(ctr, lane);
-    while (cur * 32 < NP) {  // tickets of one warp increase: once past the end, done
-        int tk = 0;
-        if (lane == 0) tk = atomicAdd(ctr, 1);  // the next chunk, read after drawing this one
-        const int t = cur * 32 + lane;
-        if (t < NP) {
-            const int4 p = load_prim(a, t);
-            int2 v0, v1, v2, v3 = make_int2(0, 0);
-            gather_prim(a, snapc0, t, p, v0, v1, v2, v3);
-            culled += draw_prim_lane<kInlineFallback>(a, cull, t, p.w, v0, v1, v2, v3, bm, big, sacc);
+    int cur = chunk_ticket(ctr, lane), qn = 0;
+    for (;;) {
+        PrimEntry e;
+        bool live = false;
+        const bool last = cur * 32 >= NP;  // tickets of one warp increase: once past the end, done
+        if (!last) {
+            int tk = 0;
+            if (lane == 0) tk = atomicAdd(ctr, 1);  // the next chunk, read after this one's set-up
+            const int t = cur * 32 + lane;
+            if (t < NP) {
+                const int4 p = load_prim(a, t);
+                int2 v0, v1, v2, v3 = make_int2(0, 0);
+                gather_prim(a, snapc0, t, p, v0, v1, v2, v3);
+                if (make_entry(v0, v1, v2, v3, p.w >= 0, culled, e)) {
+                    const int size = entry_size(e, W, H);
+                    live = size == 1 && !(cull && back_small(e));
+                    if (size == 2) defer_large<kInlineFallback>(t, e, a, cull, bm, big, sacc);
+                }
+            }
+            cur = __shfl_sync(0xffffffffu, tk, 0);
         }
-        cur = __shfl_sync(0xffffffffu, tk, 0);
+        const unsigned m = __ballot_sync(0xffffffffu, live);
+        int pos = qn + __popc(m & ((1u << lane) - 1u));
+        qn += __popc(m);
+        for (;;) {  // enter what fits, draw the queue when it is full
+            if (live && pos < cap) {
+                queue[pos] = make_int4(e.c0.x, e.c0.y, e.c1.x, e.c1.y);
+                queue[cap + pos] = make_int4(e.c2.x, e.c2.y, e.c3.x, e.c3.y);
+                live = false;
+            }
+            if (qn < cap && !(last && qn > 0)) break;
+            __syncwarp();
+            const bool on = lane < min(qn, cap);
+            int4 p = make_int4(0, 0, 0, 0), q = p;
+            if (on) {
+                p = queue[lane];
+                q = queue[cap + lane];
+            }
+            __syncwarp();  // the queue's memory becomes the row table
+            draw_rows(on, make_int2(p.x, p.y), make_int2(p.z, p.w), make_int2(q.x, q.y), make_int2(q.z, q.w), W, H, cull,
+                      bm, Wq, queue, cap, lane);
+            qn = max(qn - cap, 0);
+            pos -= cap;
+        }
+        if (last) break;
     }
     __syncthreads();
     if (!kInlineFallback && sacc[6]) {
@@ -253,24 +290,14 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::clust
             const int tt = base + lane;
             bool l1 = false, l2 = false;
             if (tt < NP) {
-                const int b = tt >= P;
-                const int4 p = a.prims[tt - b * P];
-                const int2 *sv = snapc0 + b * V;
-                const int2 u0 = __ldcg(sv + p.x), u1 = __ldcg(sv + p.y), u2 = __ldcg(sv + p.z);
-                int st = 3;
-                if (p.w >= 0) {
-                    const int2 u3 = __ldcg(sv + p.w);
-                    QuadSetup q;
-                    st = quad_setup(u0, u1, u2, u3, W, H, cull, q);
-                    if (st == 1) l1 = l2 = !small_box(q.spanx, q.spany);
-                    if (st == 3) {
-                        TriSetup ts;
-                        l2 = tri_setup(u0, u2, u3, W, H, cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
-                    }
-                }
-                if (st == 3) {
-                    TriSetup ts;
-                    l1 = tri_setup(u0, u1, u2, W, H, cull, ts) == 1 && !small_box(ts.spanx, ts.spany);
+                const int4 p = load_prim(a, tt);
+                int2 u0, u1, u2, u3 = make_int2(0, 0);
+                gather_prim(a, snapc0, tt, p, u0, u1, u2, u3);
+                PrimEntry e;
+                int dummy = 0;
+                if (make_entry(u0, u1, u2, u3, p.w >= 0, dummy, e) && entry_size(e, W, H) == 2) {
+                    l1 = e.part != 2;
+                    l2 = e.part != 1;
                 }
             }
             for (int part = 1; part <= 2; ++part)
@@ -388,7 +415,8 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
 
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *scr = reinterpret_cast<float2 *>(smem);                           // [nI*kComposeScratch]
-    uint32_t *bm = reinterpret_cast<uint32_t *>(scr + nI * kComposeScratch);  // [H*Wq]
+    int4 *queues = reinterpret_cast<int4 *>(smem);                            // [nwarp][qcap entries]: phase 2, over scr
+    uint32_t *bm = reinterpret_cast<uint32_t *>(smem + front_smem_bytes(nI, a.qcap));  // [H*Wq]
     float *sM = reinterpret_cast<float *>(bm + ((nwords + 3) & ~3));          // [nI*nF*24]
     int *big = reinterpret_cast<int *>(sM + nI * nF * 24);                    // [kBigListCap]
     // [kAccWords]: s I m culled, big-list count, chunk ticket counter, big-list
@@ -430,40 +458,21 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     }
     __syncthreads();
 
-    // ---- phase 1: project and snap this CTA's share of the vertices, two in flight ----
-    const int gtid = rank * nthr + tid, gstride = K * nthr;
+    // ---- phase 1: project and snap this CTA's share of the vertices ----
     int2 *snapc = a.snap + (size_t)c * nI * a.V;
     const int NV = nI * a.V;
-    for (int idx0 = gtid; idx0 < NV; idx0 += 2 * gstride) {
-        const int idx1 = idx0 + gstride;
-        const bool has1 = idx1 < NV;
-        int b0 = idx0 >= a.V, b1 = has1 ? (idx1 >= a.V) : b0;  // instrument (at most 2): no division
-        float4 p0 = a.verts[idx0 - b0 * a.V];
-        float4 p1 = has1 ? a.verts[idx1 - b1 * a.V] : p0;
-        float2 uv0, uv1;
-        int2 o0, o1;
-        const int f0 = (int)p0.w, f1 = (int)p1.w;
-        if (kChecked && !((unsigned)f0 < (unsigned)nF && (float)f0 == p0.w)) {  // a frame index out of range: flagged
-            o0 = make_int2(kSnapFlag, kSnapFlag);
-            uv0 = make_float2(0.0f, 0.0f);
-        } else {
-            o0 = project_vertex(p0, sM + (b0 * nF + f0) * 24, a.cam, uv0);
-        }
-        if (kChecked && !((unsigned)f1 < (unsigned)nF && (float)f1 == p1.w)) {
-            o1 = make_int2(kSnapFlag, kSnapFlag);
-            uv1 = make_float2(0.0f, 0.0f);
-        } else {
-            o1 = project_vertex(p1, sM + (b1 * nF + f1) * 24, a.cam, uv1);
-        }
-        snapc[idx0] = o0;
-        if (a.snap_dbg) a.snap_dbg[(size_t)c * NV + idx0] = o0;
-        if (a.uv_dbg) a.uv_dbg[(size_t)c * NV + idx0] = uv0;
-        if (has1) {
-            snapc[idx1] = o1;
-            if (a.snap_dbg) a.snap_dbg[(size_t)c * NV + idx1] = o1;
-            if (a.uv_dbg) a.uv_dbg[(size_t)c * NV + idx1] = uv1;
-        }
-        if (o0.x == kSnapFlag || (has1 && o1.x == kSnapFlag)) sacc[8] = 1;
+    for (int idx = rank * nthr + tid; idx < NV; idx += K * nthr) {
+        const int b = idx >= a.V;  // instrument (at most 2): no division
+        const float4 p = a.verts[idx - b * a.V];
+        float2 uv = make_float2(0.0f, 0.0f);
+        int2 o = make_int2(kSnapFlag, kSnapFlag);
+        const int f = (int)p.w;
+        if (!kChecked || ((unsigned)f < (unsigned)nF && (float)f == p.w))  // else: a frame index out of range
+            o = project_vertex(p, sM + (b * nF + f) * 24, a.cam, uv);
+        snapc[idx] = o;
+        if (a.snap_dbg) a.snap_dbg[(size_t)c * NV + idx] = o;
+        if (a.uv_dbg) a.uv_dbg[(size_t)c * NV + idx] = uv;
+        if (o.x == kSnapFlag) sacc[8] = 1;
     }
     cluster.sync();  // arrive.release / wait.acquire: the snapped vertices are visible cluster-wide
 
@@ -481,7 +490,8 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     int cull = a.cull;
     if (kQuads && a.closed)
         cull |= !__any_sync(0xffffffffu, lane < K && *cluster.map_shared_rank(&sacc[8], lane < K ? lane : 0) != 0);
-    int culled = kQuads ? draw_prims<kInlineFallback>(a, cull, cluster, snapc, bm, big, sacc, lane, warp, nwarp)
+    int culled = kQuads ? draw_prims<kInlineFallback>(a, cull, cluster, snapc, bm, big, sacc, queues + a.qcap * kQueueEntryBytes / 16 * warp, lane,
+                                                       warp, nwarp)
                         : draw_tris<kInlineFallback, kChecked>(a, cluster, snapc, bm, big, sacc, lane, warp, nwarp);
     cluster.sync();
     if (kQuads) {
@@ -718,8 +728,18 @@ size_t tell_smem_bytes() { return sizeof(TellSmem); }
 size_t eval_smem_bytes(const EvalArgs &a)
 {
     size_t nwords = (size_t)a.cam.H * a.cam.Wq;
-    return (size_t)a.ch.n_inst * kComposeScratch * sizeof(float2) + ((nwords + 3) & ~(size_t)3) * 4 +
+    return front_smem_bytes(a.ch.n_inst, eval_queue_cap(a.ch, a.cam)) + ((nwords + 3) & ~(size_t)3) * 4 +
            (size_t)a.ch.n_inst * a.ch.n_frames * 24 * 4 + (size_t)kBigListCap * 4 + kAccWords * 4;
+}
+
+// Entries per warp of the drawing queue: one per lane, or what the composition
+// scratch has room for when the image's bitmap leaves no more.
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam)
+{
+    const size_t nwords = (size_t)cam.H * cam.Wq;
+    const size_t rest = ((nwords + 3) & ~(size_t)3) * 4 + (size_t)ch.n_inst * ch.n_frames * 24 * 4 +
+                        (size_t)kBigListCap * 4 + kAccWords * 4;
+    return front_smem_bytes(ch.n_inst, 32) + rest <= 227 * 1024 ? 32 : 8;
 }
 
 int eval_max_threads() { return 1024; }

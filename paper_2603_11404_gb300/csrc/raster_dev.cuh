@@ -198,7 +198,18 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
     e = __fmaf_rn(a, b, -p);
 }
 
-// (hi + lo) . (x, y, z, 1)
+// hi + lo renormalised, |hi| >= |lo| (Dekker's FastTwoSum)
+__device__ __forceinline__ DF fast_two_sum(float hi, float lo)
+{
+    DF r;
+    r.hi = __fadd_rn(hi, lo);
+    r.lo = __fsub_rn(lo, __fsub_rn(r.hi, hi));
+    return r;
+}
+
+// (hi + lo) . (x, y, z, 1).  The sum of the rounding errors is below the sum
+// itself unless the row cancels to nothing, and then what FastTwoSum loses is
+// below the errors' own rounding.
 __device__ __forceinline__ DF df_affine(const float *h, const float *l, float x, float y, float z)
 {
     float p0, e0, p1, e1, p2, e2, s, t0, t1, t2;
@@ -211,35 +222,39 @@ __device__ __forceinline__ DF df_affine(const float *h, const float *l, float x,
     float err = __fadd_rn(__fadd_rn(t0, t1), __fadd_rn(t2, e0));
     err = __fadd_rn(err, __fadd_rn(e1, e2));
     err = __fadd_rn(err, __fmaf_rn(l[0], x, __fmaf_rn(l[1], y, __fmaf_rn(l[2], z, l[3]))));
-    DF r;
-    two_sum(s, err, r.hi, r.lo);
-    return r;
+    return fast_two_sum(s, err);
 }
 
-// a / b given rb = 1/b.hi (approximate): one correction step from the exact residual.
+// a / b given rb = 1/b.hi (approximate): one correction step from the residual
+// (a.hi - q1 b.hi is exact: q1 is the quotient to within a few ulp).
 __device__ __forceinline__ DF df_div(DF a, DF b, float rb)
 {
-    float q1 = __fmul_rn(a.hi, rb);
-    float p, e;
-    two_prod(q1, b.hi, p, e);
-    float r = __fsub_rn(__fsub_rn(a.hi, p), e);
-    r = __fadd_rn(r, __fsub_rn(a.lo, __fmul_rn(q1, b.lo)));
-    float q2 = __fmul_rn(r, rb);
-    DF o;
-    two_sum(q1, q2, o.hi, o.lo);
-    return o;
+    const float q1 = __fmul_rn(a.hi, rb);
+    const float r = __fadd_rn(__fmaf_rn(-q1, b.hi, a.hi), __fmaf_rn(-q1, b.lo, a.lo));
+    return fast_two_sum(q1, __fmul_rn(r, rb));
 }
 
-// Round-half-even of 256 (hi + lo), exact for |256 hi| < 2^22 (the guard band).
+// Round-half-even of 256 (hi + lo), exact for |256 hi| <= 2^22 (the guard band):
+// adding 1.5 2^23 rounds to an integer and leaves it in the low mantissa bits.
 __device__ __forceinline__ int snap256(DF u)
 {
-    float a = __fmul_rn(u.hi, 256.0f);
-    float b = __fmul_rn(u.lo, 256.0f);
-    float n = rintf(a);
-    float d = __fsub_rn(a, n);
-    if (d == 0.5f && b > 0.0f) n = __fadd_rn(n, 1.0f);
-    else if (d == -0.5f && b < 0.0f) n = __fsub_rn(n, 1.0f);
-    return (int)n;
+    const float magic = 12582912.0f;  // 1.5 * 2^23
+    const float a = __fmul_rn(u.hi, 256.0f);
+    const float t = __fadd_rn(a, magic);
+    int n = __float_as_int(t) - __float_as_int(magic);
+    const float d = __fsub_rn(a, __fsub_rn(t, magic));
+    if (fabsf(d) == 0.5f) {  // a tie of the high part: the low part decides
+        if (d > 0.0f && u.lo > 0.0f) ++n;
+        if (d < 0.0f && u.lo < 0.0f) --n;
+    }
+    return n;
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 // ----------------------------------------------------------------------------
@@ -445,53 +460,185 @@ __device__ __forceinline__ int quad_setup(int2 a, int2 b, int2 c, int2 d, int W,
     return 1;
 }
 
-// One thread, four int32 incremental edge functions (edge k from corner k to
-// corner k+1, the top-left bias as in raster_small_at).  The same bounds as the
-// triangle form: spanx < 32 px, spany < 64 px.
-__device__ __forceinline__ void raster_quad_small(const QuadSetup &q, uint32_t *bm, int Wq)
+// ----------------------------------------------------------------------------
+// Small primitives (corners spanning less than 32 px across and 64 px down, so
+// that int32 edge functions are exact over the box and its corner, and a row
+// fits one 64-bit window) drawn a row per lane.
+// ----------------------------------------------------------------------------
+
+// A primitive's corners (c3.x == kSnapFlag: a triangle); part: which of its
+// record's triangles it stands for (0 both, 1 the first, 2 the second).
+struct PrimEntry {
+    int2 c0, c1, c2, c3;
+    int part;
+};
+
+// The entry of a record's snapped corners: triangles with a flagged corner are
+// left out (and counted).  False: nothing left.
+__device__ __forceinline__ bool make_entry(int2 v0, int2 v1, int2 v2, int2 v3, bool pair, int &culled, PrimEntry &e)
 {
-    int r[4], cs[4], rs[4];
-    const int Px = 256 * q.j0, Py = 256 * q.i0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int k1 = (k + 1) & 3;
-        const int dx = q.x[k1] - q.x[k], dy = q.y[k1] - q.y[k];
-        const int bias = (dy < 0 || (dy == 0 && dx > 0)) ? 0 : 1;
-        r[k] = dx * (Py - q.y[k]) - dy * (Px - q.x[k]) - bias;
-        cs[k] = dy * 256;
-        rs[k] = dx * 256;
+    const bool f = v0.x == kSnapFlag || v2.x == kSnapFlag;
+    const bool fa = f || v1.x == kSnapFlag, fb = pair && (f || v3.x == kSnapFlag);
+    culled += fa + fb;
+    e.c0 = v0;
+    e.c1 = v1;
+    e.c2 = v2;
+    e.c3 = v3;
+    e.part = pair ? 0 : 1;
+    if (!pair || fb) {
+        e.c3.x = kSnapFlag;
+        e.part = 1;
+        return !fa;
     }
-    const int jb = q.j0 & ~31;
-    const int off = q.j0 - jb;
-    const int nb = q.j1 - q.j0 + 1;  // 1..32
-    const bool one_word = off + nb <= 32;
-    uint32_t *row = bm + (size_t)q.i0 * Wq + (jb >> 5);
-    for (int i = q.i0; i <= q.i1; ++i) {
-        int a0 = r[0], a1 = r[1], a2 = r[2], a3 = r[3];
-        uint32_t bits = 0u;
-#pragma unroll 4
-        for (int n = 0; n < nb; ++n) {
-            bits = __funnelshift_l((uint32_t)(~(a0 | a1 | a2 | a3)), bits, 1);  // (bits << 1) | covered
-            a0 -= cs[0];
-            a1 -= cs[1];
-            a2 -= cs[2];
-            a3 -= cs[3];
+    if (fa) {
+        e.c1 = v2;
+        e.c2 = v3;
+        e.c3.x = kSnapFlag;
+        e.part = 2;
+    }
+    return true;
+}
+
+// Pixel box of an entry, clipped to the image.  Returns 0: no pixel centre in
+// it, 1: small, 2: large.
+__device__ __forceinline__ int entry_size(const PrimEntry &e, int W, int H)
+{
+    const int2 c3 = e.c3.x == kSnapFlag ? e.c2 : e.c3;
+    const int xmn = min(min(e.c0.x, e.c1.x), min(e.c2.x, c3.x)), xmx = max(max(e.c0.x, e.c1.x), max(e.c2.x, c3.x));
+    const int ymn = min(min(e.c0.y, e.c1.y), min(e.c2.y, c3.y)), ymx = max(max(e.c0.y, e.c1.y), max(e.c2.y, c3.y));
+    if (max(0, (xmn + 255) >> 8) > min(W - 1, xmx >> 8) || max(0, (ymn + 255) >> 8) > min(H - 1, ymx >> 8)) return 0;
+    return xmx - xmn < 32 * 256 && ymx - ymn < 64 * 256 ? 1 : 2;
+}
+
+__device__ __forceinline__ int orient_small(int2 p, int2 q, int2 r)
+{
+    return (q.x - p.x) * (r.y - p.y) - (r.x - p.x) * (q.y - p.y);
+}
+
+// No triangle of a small entry faces the camera (negative orientation).
+__device__ __forceinline__ bool back_small(const PrimEntry &e)
+{
+    return orient_small(e.c0, e.c1, e.c2) >= 0 && (e.c3.x == kSnapFlag || orient_small(e.c0, e.c2, e.c3) >= 0);
+}
+
+// A warp draws the small primitives that its lanes hold (`live`), a row of
+// pixels per lane: rows, not primitives, are shared out, so the lanes work alike
+// whatever the primitives' sizes.  A pair of triangles is drawn as one convex
+// quadrilateral where it is one, else as its triangles, one after the other;
+// `cull` leaves out the back faces.  tab: the warp's table of n entries, n at
+// least the number of live lanes: the polygons' edge functions at the first
+// pixel of their box (int4 [n]), edge vectors (int4 [n], dx and dy in 16 bits),
+// first task, columns and place in the bitmap (int2 [n]).
+__device__ __forceinline__ void draw_rows(bool live, int2 c0, int2 c1, int2 c2, int2 c3, int W, int H, int cull,
+                                          uint32_t *bm, int Wq, int4 *tab, int n, int lane)
+{
+    int4 *tab_r = tab, *tab_d = tab + n;
+    int2 *tab_m = reinterpret_cast<int2 *>(tab + 2 * n);
+    bool tri = c3.x == kSnapFlag, two = false;
+    const int2 mid = c2, end = c3;
+    int A = 0;
+    if (live) {
+        A = orient_small(c0, c1, c2);
+        if (!tri) {
+            const int A2 = orient_small(c0, c2, c3);
+            const int Da = orient_small(c1, c3, c0), Dc = orient_small(c1, c3, c2);
+            // same non-zero orientation, and c0, c2 strictly on opposite sides of c1-c3
+            if (!(((A > 0 && A2 > 0) || (A < 0 && A2 < 0)) && ((Da > 0 && Dc < 0) || (Da < 0 && Dc > 0)))) tri = two = true;
         }
-        if (bits) {
-            const uint32_t rb = __brev(bits) >> (32 - nb);  // pixel j0 at bit 0
-            if (one_word) {
-                atomicOr(row, rb << off);
-            } else {
-                const uint32_t lo = rb << off, hi = rb >> (32 - off);
-                if (lo) atomicOr(row, lo);
-                if (hi) atomicOr(row + 1, hi);
+    }
+    for (;;) {
+        bool on = live && A != 0 && !(cull && A > 0);
+        int4 r, d;
+        int2 m;
+        int rows = 0;
+        if (on) {
+            if (A < 0) {  // positive orientation
+                const int2 t = c1;
+                c1 = tri ? c2 : c3;
+                (tri ? c2 : c3) = t;
+            }
+            if (tri) c3 = c2;
+            const int j0 = max(0, (min(min(c0.x, c1.x), min(c2.x, c3.x)) + 255) >> 8);
+            const int j1 = min(W - 1, max(max(c0.x, c1.x), max(c2.x, c3.x)) >> 8);
+            const int i0 = max(0, (min(min(c0.y, c1.y), min(c2.y, c3.y)) + 255) >> 8);
+            const int i1 = min(H - 1, max(max(c0.y, c1.y), max(c2.y, c3.y)) >> 8);
+            on = j0 <= j1 && i0 <= i1;
+            rows = on ? i1 - i0 + 1 : 0;
+            const int Px = 256 * j0, Py = 256 * i0;
+            auto edge = [&](int2 p, int2 q, int &rv, int &dv) {
+                const int dx = q.x - p.x, dy = q.y - p.y;
+                const int bias = (dy < 0 || (dy == 0 && dx > 0)) ? 0 : 1;
+                rv = dx * (Py - p.y) - dy * (Px - p.x) - bias;
+                dv = (int)((unsigned)dx << 16 | ((unsigned)dy & 0xffffu));
+            };
+            edge(c0, c1, r.x, d.x);
+            edge(c1, c2, r.y, d.y);
+            edge(c2, c3, r.z, d.z);
+            edge(c3, c0, r.w, d.w);
+            if (tri) r.z = 0;  // the edge from c2 to c2: no constraint (its steps are 0)
+            m.x = (j1 - j0) << 16 | (j0 & 31) << 24;
+            m.y = i0 * Wq + (j0 >> 5);
+        }
+        int incl = rows;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31), first = incl - rows;
+        const unsigned lm = __ballot_sync(0xffffffffu, on);
+        if (on) {
+            const int slot = __popc(lm & ((1u << lane) - 1u));
+            m.x |= first;
+            tab_r[slot] = r;
+            tab_d[slot] = d;
+            tab_m[slot] = m;
+        }
+        __syncwarp();
+        for (int base = 0; base < total; base += 32) {
+            // the polygon of task base + lane: those that start before this
+            // window, then one more at each start within it
+            const int rel = first - base;
+            const unsigned starts = __reduce_or_sync(0xffffffffu, on && rel >= 0 && rel < 32 ? 1u << rel : 0u);
+            const int before = __popc(__ballot_sync(0xffffffffu, on && rel < 0));
+            const int t = base + lane;
+            if (t < total) {
+                const int slot = before - 1 + __popc(starts & (0xffffffffu >> (31 - lane)));
+                const int4 rv = tab_r[slot], dv = tab_d[slot];
+                const int2 mv = tab_m[slot];
+                const int row = t - (mv.x & 0xffff), nb = (mv.x >> 16 & 31) + 1, off = mv.x >> 24;
+                const int cs0 = (int)((unsigned)dv.x << 16) >> 8, cs1 = (int)((unsigned)dv.y << 16) >> 8;  // 256 dy
+                const int cs2 = (int)((unsigned)dv.z << 16) >> 8, cs3 = (int)((unsigned)dv.w << 16) >> 8;
+                int a0 = rv.x + row * 256 * (dv.x >> 16), a1 = rv.y + row * 256 * (dv.y >> 16);
+                int a2 = rv.z + row * 256 * (dv.z >> 16), a3 = rv.w + row * 256 * (dv.w >> 16);
+                uint32_t bits = 0u;
+#pragma unroll 4
+                for (int q = 0; q < nb; ++q) {
+                    bits = __funnelshift_l((uint32_t)(~(a0 | a1 | a2 | a3)), bits, 1);  // (bits << 1) | covered
+                    a0 -= cs0;
+                    a1 -= cs1;
+                    a2 -= cs2;
+                    a3 -= cs3;
+                }
+                if (bits) {
+                    const uint32_t rb = __brev(bits) >> (32 - nb);  // pixel j0 at bit 0
+                    uint32_t *w = bm + mv.y + row * Wq;
+                    const uint32_t lo = rb << off, hi = off ? rb >> (32 - off) : 0u;
+                    if (lo) atomicOr(w, lo);
+                    if (hi) atomicOr(w + 1, hi);
+                }
             }
         }
-        r[0] += rs[0];
-        r[1] += rs[1];
-        r[2] += rs[2];
-        r[3] += rs[3];
-        row += Wq;
+        __syncwarp();
+        if (!__any_sync(0xffffffffu, two)) break;
+        live = two;  // the second triangles
+        two = false;
+        tri = true;
+        if (live) {
+            c1 = mid;
+            c2 = end;
+            A = orient_small(c0, c1, c2);
+        }
     }
 }
 
@@ -507,7 +654,7 @@ __device__ __forceinline__ int2 project_vertex(float4 p, const float *Mh, const 
     int2 o = make_int2(kSnapFlag, kSnapFlag);
     uv = make_float2(0.f, 0.f);
     if (Z.hi >= (float)cam.z_near) {
-        float rz = __frcp_rn(Z.hi);
+        const float rz = rcp_approx(Z.hi);
         DF u = df_div(X, Z, rz), w = df_div(Y, Z, rz);
         uv = make_float2(__fadd_rn(u.hi, u.lo), __fadd_rn(w.hi, w.lo));
         const float guard = (float)cam.guard;
