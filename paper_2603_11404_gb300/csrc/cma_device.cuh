@@ -116,15 +116,22 @@ __device__ __forceinline__ void cma_sample_warp(const CmaConst &k, const CmaStat
 // Shared memory of one update; the selected steps are staged in shared memory
 // when mu * d <= kYselCap (populations up to lam = 128 at d = 18, 256 at d = 9).
 constexpr int kYselCap = 64 * kMaxD;
-struct TellSmem {
-    float sl[TRK_MAX_LAMBDA];
-    int order[TRK_MAX_LAMBDA];
+struct alignas(16) TellSmem {
+    union {
+        struct {
+            float sl[TRK_MAX_LAMBDA];
+            int order[TRK_MAX_LAMBDA];
+        };
+        double wy[kYselCap];  // the staged steps times their weights, once they are ranked
+    };
     double yw[kMaxD], pc[kMaxD], sq[kMaxD], isq[kMaxD];
     double part[8][kMaxD];
     double C[kMaxD * kMaxD], A[kMaxD * kMaxD], A2[kMaxD * kMaxD], V[kMaxD * kMaxD], V2[kMaxD * kMaxD];
     double B[kMaxD * kMaxD], ysel[kYselCap], w[TRK_MAX_LAMBDA / 2];
     float Af[kMaxD * kMaxD], Vf[kMaxD * kMaxD], Vf2[kMaxD * kMaxD];
     double n2, hs;
+    int best;        // the population's best candidate and its loss
+    float best_loss;
 };
 
 // C (d x d, FP64, row-major) -> out = X^T C X for square X, FP64.
@@ -353,8 +360,9 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
                                               const float *loss, TellSmem &S, int tid, int nt, bool do_sqrt)
 {
     const int d = DC ? DC : k.d, lam = k.lam, dd = d * d, mu = k.mu;
-    for (int i = tid; i < lam; i += nt) {
-        float v = loss[i];
+    const int lam4 = (lam + 3) & ~3;  // padded with losses that rank behind every candidate
+    for (int i = tid; i < lam4; i += nt) {
+        float v = i < lam ? loss[i] : INFINITY;
         S.sl[i] = isnan(v) ? INFINITY : v;
     }
     for (int e = tid; e < dd; e += nt) {
@@ -375,11 +383,19 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
                 if (q < d) yi[q] = y[(size_t)i * d + q];
         float li = S.sl[i];
         int r = 0;
-        for (int j = 0; j < lam; ++j) {
-            float lj = S.sl[j];
-            r += (lj < li) || (lj == li && j < i);
+#pragma unroll 4
+        for (int j = 0; j < lam4; j += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(S.sl + j);
+            r += (v.x < li) || (v.x == li && j < i);
+            r += (v.y < li) || (v.y == li && j + 1 < i);
+            r += (v.z < li) || (v.z == li && j + 2 < i);
+            r += (v.w < li) || (v.w == li && j + 3 < i);
         }
         S.order[r] = i;
+        if (r == 0) {
+            S.best = i;
+            S.best_loss = li;
+        }
         if (staged && r < mu)
 #pragma unroll
             for (int q = 0; q < kMaxD; ++q)
@@ -387,12 +403,12 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
     }
     __syncthreads();
     if (tid >= nt - 32) {  // the frame's best so far, on the last warp (the mean's partial sums start on the first)
-        const int lane = tid - (nt - 32), b = S.order[0];
+        const int lane = tid - (nt - 32), b = S.best;
         const float prev = st->best_loss;
         __syncwarp();
-        if (S.sl[b] < prev) {
+        if (S.best_loss < prev) {
             for (int i = lane; i < d; i += 32) st->best_x[i] = params[(size_t)b * d + i];
-            if (lane == 0) st->best_loss = S.sl[b];
+            if (lane == 0) st->best_loss = S.best_loss;
         }
     }
 #define YSEL(r, i) (staged ? S.ysel[(r) * d + (i)] : y[(size_t)S.order[r] * d + (i)])
@@ -405,6 +421,8 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
         for (int r = part * chunk; r < r1; ++r) acc = __fma_rn(S.w[r], YSEL(r, i), acc);
         S.part[part][i] = acc;
     }
+    if (staged)  // from the threads at the block's other end; over sl and order, which a staged update is done with
+        for (int e = nt - 1 - tid; e < mu * d; e += nt) S.wy[e] = S.w[e / d] * S.ysel[e];
     __syncthreads();
     // The mean, the evolution paths and h_sigma in warp 0 (lanes = coordinates,
     // d <= 32, shuffles instead of block barriers) while the other warps form
@@ -414,7 +432,8 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
     const double sigma = st->sigma, cs = k.c_sigma, cc = k.c_c;
     const double c1 = k.c_1, cmu = k.c_mu;
     double *part4[4] = {S.A, S.A2, S.V, S.V2};
-    const int nup = d * (d + 1) / 2;  // entries (i, j), j >= i
+    const int bd = DC == 18 && k.block == 9 ? 9 : d;  // rows of a diagonal block
+    const int bup = bd * (bd + 1) / 2, nup = d / bd * bup;  // its entries (i, j), j >= i
     const bool split = nt > 32;  // warp 0 takes the paths, the rest the rank-mu sums
     if (tid < 32) {
         const int lane = tid;
@@ -468,14 +487,20 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
         for (int e = split ? tid - 32 : tid; e < 4 * nup; e += split ? nt - 32 : nt) {
             const int pr = e / nup;
             int u = e - pr * nup, i = 0;
-            while (u >= d - i) {  // row i holds d - i entries of the upper triangle
-                u -= d - i;
+            const int first = u >= bup ? bd : 0;  // the block's first row
+            if (first) u -= bup;
+            while (u >= bd - i) {  // its row i holds bd - i entries of the upper triangle
+                u -= bd - i;
                 ++i;
             }
+            i += first;
             const int j = i + u, ij = i * d + j;
             double rmu = 0.0;
-            int r1 = min(mu, (pr + 1) * rchunk);
-            for (int r = pr * rchunk; r < r1; ++r) rmu = __fma_rn(S.w[r] * YSEL(r, i), YSEL(r, j), rmu);
+            const int r1 = min(mu, (pr + 1) * rchunk);
+            if (staged)
+                for (int r = pr * rchunk; r < r1; ++r) rmu = __fma_rn(S.wy[r * d + i], S.ysel[r * d + j], rmu);
+            else
+                for (int r = pr * rchunk; r < r1; ++r) rmu = __fma_rn(S.w[r] * YSEL(r, i), YSEL(r, j), rmu);
             part4[pr][ij] = rmu;
         }
     }
@@ -540,29 +565,136 @@ __device__ __forceinline__ void cma_tell_impl(const CmaConst &k, CmaState *st, c
 // (d = 9: four fit) or S.A, S.V, S.V2, S.B (d = 18), T in S.A2.
 constexpr int kNsMaxSteps = 64;
 
-template <int DC>
-__device__ __forceinline__ double ns_dot(const double *L, const double *R, int i, int j)
+// Entry (i, j) of L R over the columns q0 .. q0 + B - 1 of L (a diagonal block,
+// or all of them); the three chains take every third column.
+template <int DC, int B>
+__device__ __forceinline__ double ns_dot(const double *L, const double *R, int i, int j, int q0)
 {
     constexpr int d = DC;
+    static_assert(B == DC || B % 3 == 0, "a block starts on the first chain");
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;  // three chains: FP64 latency, not throughput, bounds this
 #pragma unroll
-    for (int q = 0; q < d; q += 3) {
-        a0 = __fma_rn(L[i * d + q], R[q * d + j], a0);
-        if (q + 1 < d) a1 = __fma_rn(L[i * d + q + 1], R[(q + 1) * d + j], a1);
-        if (q + 2 < d) a2 = __fma_rn(L[i * d + q + 2], R[(q + 2) * d + j], a2);
+    for (int q = 0; q < B; q += 3) {
+        a0 = __fma_rn(L[i * d + q0 + q], R[(q0 + q) * d + j], a0);
+        if (q + 1 < B) a1 = __fma_rn(L[i * d + q0 + q + 1], R[(q0 + q + 1) * d + j], a1);
+        if (q + 2 < B) a2 = __fma_rn(L[i * d + q0 + q + 2], R[(q0 + q + 2) * d + j], a2);
     }
     return __dadd_rn(__dadd_rn(a0, a1), a2);
+}
+
+// |x| < 1e-8 (false for NaN), by the bit patterns: no FP64 instruction.
+__device__ __forceinline__ bool below_1em8(double x)
+{
+    return (__double_as_longlong(x) & 0x7fffffffffffffffLL) < __double_as_longlong(1e-8);
+}
+
+// The iteration over diagonal blocks of B rows (B = DC: the whole matrix), from
+// the scale exponent e2.  The entries outside the blocks are zero throughout
+// and are neither formed nor read; those inside get the bits of the whole
+// products (a term 0 * 0 leaves an FMA chain as it is, and a block starts on
+// the first of the three chains).
+template <int DC, int B>
+__device__ __forceinline__ bool newton_schulz_blocks(CmaState *st, TellSmem &S, int tid, int nt, int e2, bool do_sigma,
+                                                     const CmaConst &k, double sigma)
+{
+    constexpr int d = DC, dd = d * d, bb = B * B, ne = DC / B * bb;
+    constexpr bool kPacked = 4 * dd <= kMaxD * kMaxD;
+    static_assert(DC > 0 && dd <= kMaxD * kMaxD && DC % B == 0, "d x d iterates");
+    double *Y = S.A, *Z = kPacked ? S.A + dd : S.V, *Y2 = kPacked ? S.A + 2 * dd : S.V2,
+           *Z2 = kPacked ? S.A + 3 * dd : S.B, *T = S.A2;
+    const double *C = S.C;
+    // entry n of the blocks: row i, column j, the block's first row q0
+    auto entry = [](int n, int &i, int &j, int &q0) {
+        q0 = B == DC ? 0 : n / bb * B;
+        const int f = B == DC ? n : n - n / bb * bb;
+        i = q0 + f / B;
+        j = q0 + f % B;
+    };
+    int i, j, q0;
+    const double ic = ldexp(1.0, -e2);
+    // the first step needs no products: Z_0 = I makes Z_0 Y_0 = Y_0 and
+    // T_0 Z_0 = T_0 exactly (bit for bit what the products would give)
+    bool open0 = false;
+    for (int n = tid; n < ne; n += nt) {
+        entry(n, i, j, q0);
+        const int e = i * d + j;
+        const double y = __dmul_rn(C[e], ic);
+        const double r = ((i == j) ? 1.0 : 0.0) - y;
+        open0 |= !below_1em8(r);
+        const double t = ((i == j) ? 1.0 : 0.0) + 0.5 * r;
+        Y[e] = y;
+        T[e] = t;
+        Z[e] = t;
+    }
+    bool done = !__syncthreads_or(open0);
+    for (int n = tid; n < ne; n += nt) {
+        entry(n, i, j, q0);
+        Y2[i * d + j] = ns_dot<DC, B>(Y, T, i, j, q0);
+    }
+    __syncthreads();
+    {
+        double *t = Y; Y = Y2; Y2 = t;
+    }
+    int steps = 1;
+    while (!done && steps < kNsMaxSteps) {
+        bool open = false;  // a residual entry at or above 1e-8 (or not a number)
+        for (int n = tid; n < ne; n += nt) {
+            entry(n, i, j, q0);
+            const double r = ((i == j) ? 1.0 : 0.0) - ns_dot<DC, B>(Z, Y, i, j, q0);  // I - Z Y
+            open |= !below_1em8(r);
+            T[i * d + j] = ((i == j) ? 1.0 : 0.0) + 0.5 * r;  // (3 I - Z Y) / 2
+        }
+        done = !__syncthreads_or(open);
+        for (int n = tid; n < 2 * ne; n += nt) {
+            const int m = n >= ne;
+            entry(n - m * ne, i, j, q0);
+            (m ? Z2 : Y2)[i * d + j] = ns_dot<DC, B>(m ? T : Y, m ? Z : T, i, j, q0);
+        }
+        __syncthreads();
+        double *t = Y; Y = Y2; Y2 = t;
+        t = Z; Z = Z2; Z2 = t;
+        ++steps;
+    }
+    if (!done) {
+        if (tid == 0) atomicOr(&st->warn, 2);
+        return false;
+    }
+    // outputs: C^(1/2) = sqrt(c) Y, C^(-1/2) = Z / sqrt(c) (sqrt(c) a power of
+    // two, times sqrt 2 for odd e), symmetrised; the
+    // step size on a thread that has no entry (FP64 exp off the critical path)
+    const double sc = ldexp((e2 & 1) ? M_SQRT2 : 1.0, e2 >> 1), isc = ldexp((e2 & 1) ? M_SQRT1_2 : 1.0, -(e2 >> 1));
+    for (int n = tid; n < ne; n += nt) {
+        entry(n, i, j, q0);
+        if (j < i) continue;
+        const double h = __dmul_rn(0.5 * __dadd_rn(Y[i * d + j], Y[j * d + i]), sc);
+        const double ih = __dmul_rn(0.5 * __dadd_rn(Z[i * d + j], Z[j * d + i]), isc);
+        st->C_half[i * d + j] = h;
+        st->C_half[j * d + i] = h;
+        st->C_half_df[i * d + j] = split_df(h);
+        st->C_half_df[j * d + i] = split_df(h);
+        st->C_inv_half[i * d + j] = ih;
+        st->C_inv_half[j * d + i] = ih;
+    }
+    if constexpr (B < DC) {
+        for (int e = tid; e < dd; e += nt) {
+            if (e / d / B == e % d / B) continue;
+            st->C_half[e] = 0.0;
+            st->C_half_df[e] = make_float2(0.0f, 0.0f);
+            st->C_inv_half[e] = 0.0;
+        }
+    }
+    if (tid == nt - 1) {
+        if (do_sigma) cma_sigma_step(k, st, S.n2, sigma);
+        st->jacobi_sweeps = -steps;
+    }
+    return true;
 }
 
 template <int DC>
 __device__ __forceinline__ bool cma_sqrt_newton_schulz(const CmaConst &k, CmaState *st, TellSmem &S, int tid,
                                                        int nt, bool do_sigma, double sigma)
 {
-    constexpr int d = DC, dd = d * d;
-    constexpr bool kPacked = 4 * dd <= kMaxD * kMaxD;
-    static_assert(DC > 0 && dd <= kMaxD * kMaxD, "d x d iterates");
-    double *Y = S.A, *Z = kPacked ? S.A + dd : S.V, *Y2 = kPacked ? S.A + 2 * dd : S.V2,
-           *Z2 = kPacked ? S.A + 3 * dd : S.B, *T = S.A2;
+    constexpr int d = DC;
     const double *C = S.C;
     if (tid < 32) {  // the scale c = 2^e, chosen in FP32 (kept in S.part[1][0])
         float tr = 0.0f, row = 0.0f;
@@ -580,73 +712,21 @@ __device__ __forceinline__ bool cma_sqrt_newton_schulz(const CmaConst &k, CmaSta
             S.part[1][0] = (m > 0.0f) ? (double)e : 0.0;
         }
     }
-    __syncthreads();
+    // d = 18: a C whose 9x9 off-diagonal blocks are zero (two instruments in
+    // block form, the usual case) takes a quarter of the FP64 instructions, and
+    // those are what the update waits for: one per warp and 64 cycles on each of
+    // the SM's four partitions.  Stand-alone update, together with the rank-mu
+    // sums over the blocks alone: 64 candidates 58.0 -> 33.4 us, 128 candidates
+    // 74.4 -> 37.5 us, 256 candidates 107 -> 56 us
+    bool full = DC != 18;
+    if constexpr (DC == 18)
+        for (int e = tid; e < d * d; e += nt)
+            full |= e / d / 9 != e % d / 9 && (__double_as_longlong(C[e]) << 1) != 0;  // not +-0
+    full = __syncthreads_or(full);
     const int e2 = (int)S.part[1][0];
-    const double ic = ldexp(1.0, -e2);
-    // the first step needs no products: Z_0 = I makes Z_0 Y_0 = Y_0 and
-    // T_0 Z_0 = T_0 exactly (bit for bit what the products would give)
-    bool open0 = false;
-    for (int e = tid; e < dd; e += nt) {
-        const int i = e / d, j = e - i * d;
-        const double y = __dmul_rn(C[e], ic);
-        const double r = ((i == j) ? 1.0 : 0.0) - y;
-        open0 |= !(fabs(r) < 1e-8);
-        const double t = ((i == j) ? 1.0 : 0.0) + 0.5 * r;
-        Y[e] = y;
-        T[e] = t;
-        Z[e] = t;
-    }
-    bool done = !__syncthreads_or(open0);
-    for (int e = tid; e < dd; e += nt) Y2[e] = ns_dot<DC>(Y, T, e / d, e - (e / d) * d);
-    __syncthreads();
-    {
-        double *t = Y; Y = Y2; Y2 = t;
-    }
-    int steps = 1;
-    while (!done && steps < kNsMaxSteps) {
-        bool open = false;  // a residual entry at or above 1e-8 (or not a number)
-        for (int e = tid; e < dd; e += nt) {
-            const int i = e / d, j = e - i * d;
-            const double r = ((i == j) ? 1.0 : 0.0) - ns_dot<DC>(Z, Y, i, j);  // I - Z Y
-            open |= !(fabs(r) < 1e-8);
-            T[e] = ((i == j) ? 1.0 : 0.0) + 0.5 * r;  // (3 I - Z Y) / 2
-        }
-        done = !__syncthreads_or(open);
-        for (int e = tid; e < 2 * dd; e += nt) {
-            const int m = e >= dd, f = e - m * dd, i = f / d, j = f - i * d;
-            if (m) Z2[f] = ns_dot<DC>(T, Z, i, j);
-            else Y2[f] = ns_dot<DC>(Y, T, i, j);
-        }
-        __syncthreads();
-        double *t = Y; Y = Y2; Y2 = t;
-        t = Z; Z = Z2; Z2 = t;
-        ++steps;
-    }
-    if (!done) {
-        if (tid == 0) atomicOr(&st->warn, 2);
-        return false;
-    }
-    // outputs: C^(1/2) = sqrt(c) Y, C^(-1/2) = Z / sqrt(c) (sqrt(c) a power of
-    // two, times sqrt 2 for odd e), symmetrised; the
-    // step size on a thread that has no entry (FP64 exp off the critical path)
-    const double sc = ldexp((e2 & 1) ? M_SQRT2 : 1.0, e2 >> 1), isc = ldexp((e2 & 1) ? M_SQRT1_2 : 1.0, -(e2 >> 1));
-    for (int e = tid; e < dd; e += nt) {
-        const int i = e / d, j = e - i * d;
-        if (j < i) continue;
-        const double h = __dmul_rn(0.5 * __dadd_rn(Y[i * d + j], Y[j * d + i]), sc);
-        const double ih = __dmul_rn(0.5 * __dadd_rn(Z[i * d + j], Z[j * d + i]), isc);
-        st->C_half[i * d + j] = h;
-        st->C_half[j * d + i] = h;
-        st->C_half_df[i * d + j] = split_df(h);
-        st->C_half_df[j * d + i] = split_df(h);
-        st->C_inv_half[i * d + j] = ih;
-        st->C_inv_half[j * d + i] = ih;
-    }
-    if (tid == nt - 1) {
-        if (do_sigma) cma_sigma_step(k, st, S.n2, sigma);
-        st->jacobi_sweeps = -steps;
-    }
-    return true;
+    if constexpr (DC == 18)
+        if (!full) return newton_schulz_blocks<18, 9>(st, S, tid, nt, e2, do_sigma, k, sigma);
+    return newton_schulz_blocks<DC, DC>(st, S, tid, nt, e2, do_sigma, k, sigma);
 }
 
 // C^(1/2) and C^(-1/2) of C (held in S.C), with the step-size update when

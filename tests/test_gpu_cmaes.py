@@ -75,6 +75,14 @@ def test_ask_tell_state_parity(api, d, lam, block):
     assert n_ulp_diff <= 3 + lam * d * 25 // 5000  # one-ulp sampling differences at rounding ties are rare
 
 
+@pytest.mark.parametrize("d,lam,block", [(18, 128, True), (18, 127, True), (18, 130, True), (18, 128, False),
+                                         (9, 255, False), (9, 257, False), (9, 5, False)])
+def test_update_at_the_edges_of_its_stages(api, d, lam, block):
+    """Populations at the staging limit (mu d = 1152) and one beyond it, and ones
+    that are no multiple of the ranking's four losses at a time."""
+    test_ask_tell_state_parity(api, d, lam, block)
+
+
 def test_square_roots_stay_exact_on_an_ill_conditioned_quadratic(api):
     """A quadratic whose curvatures span 12 decades: the covariance learns a
     condition number above 1e10 within 500 generations, where an FP32
