@@ -130,7 +130,6 @@ __device__ __forceinline__ bool small_box(int spanx, int spany) { return spanx <
 // One triangle of phase 2: drawn by this lane when small, otherwise deferred to
 // a whole warp through the CTA's list (entry `ent`).  Returns 1 when the
 // triangle is culled for a flagged vertex.
-template <bool kInlineFallback>
 __device__ __forceinline__ int draw_one_tri(int2 v0, int2 v1, int2 v2, int ent, const EvalArgs &a, int cull,
                                             uint32_t *bm, int *big, int *sacc)
 {
@@ -140,13 +139,11 @@ __device__ __forceinline__ int draw_one_tri(int2 v0, int2 v1, int2 v2, int ent, 
         if (small_box(t.spanx, t.spany)) {
             raster_small(t, bm, a.cam.Wq);
         } else {
-            // larger triangles wait for a whole warp.  If the list is full: the
-            // plain launch redraws every large primitive after the loop (raster
-            // code here would make its loop spill); the batched launch,
-            // compiled with more registers, draws the triangle in this lane
+            // larger triangles wait for a whole warp.  If the list is full,
+            // every large triangle is drawn again after the loop (raster code
+            // here would make it spill)
             const int slot = atomicAdd(&sacc[4], 1);
             if (slot < kBigListCap) big[slot] = ent;
-            else if constexpr (kInlineFallback) raster_serial(t, bm, a.cam.Wq);
             else sacc[6] = 1;
         }
     }
@@ -171,45 +168,19 @@ __device__ __forceinline__ void gather_prim(const EvalArgs &a, const int2 *snapc
     if (p.w >= 0) v3 = __ldcg(sv + p.w);
 }
 
-// A large entry waits for a whole warp, unless none of its triangles is to be
-// drawn.  If the list is full: the plain launch redraws every large primitive
-// after the loop (raster code here would make its loop spill); the batched
-// launch, compiled with more registers, draws its triangles in this lane.
-template <bool kInlineFallback>
-__device__ __forceinline__ void defer_large(int t, const PrimEntry &e, const EvalArgs &a, int cull, uint32_t *bm, int *big,
-                                            int *sacc)
+// A large entry waits for the end of the loop, unless none of its triangles is
+// to be drawn.  If the list is full, every large primitive is drawn again after
+// the loop (raster code here would make it spill).
+__device__ __forceinline__ void defer_large(int t, const PrimEntry &e, const EvalArgs &a, int cull, int *big, int *sacc)
 {
     const int W = a.cam.W, H = a.cam.H;
-    const bool pair = e.c3.x != kSnapFlag;
     TriSetup ts;
-    const bool d1 = tri_setup(e.c0, e.c1, e.c2, W, H, cull, ts) == 1;
-    const bool d2 = pair && tri_setup(e.c0, e.c2, e.c3, W, H, cull, ts) == 1;
-    if (!d1 && !d2) return;
+    if (tri_setup(e.c0, e.c1, e.c2, W, H, cull, ts) != 1 &&
+        (e.c3.x == kSnapFlag || tri_setup(e.c0, e.c2, e.c3, W, H, cull, ts) != 1))
+        return;
     const int slot = atomicAdd(&sacc[4], 1);
-    if (slot < kBigListCap) {
-        big[slot] = 4 * t + e.part;
-    } else if constexpr (kInlineFallback) {
-        if (d1 && tri_setup(e.c0, e.c1, e.c2, W, H, cull, ts) == 1) raster_serial(ts, bm, a.cam.Wq);
-        if (d2 && tri_setup(e.c0, e.c2, e.c3, W, H, cull, ts) == 1) raster_serial(ts, bm, a.cam.Wq);
-    } else {
-        sacc[6] = 1;
-    }
-}
-
-// One deferred entry drawn by the whole warp into this CTA's bitmap: the
-// triangles of primitive ent / 4 (part 0 both, 1 the first, 2 the second), a
-// pixel per lane with int64 edge functions.
-__device__ __forceinline__ void draw_deferred(const EvalArgs &a, int cull, const int2 *snapc0, int ent, uint32_t *bm, int lane)
-{
-    const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
-    const int t = ent >> 2, part = ent & 3;
-    const int b = t >= a.P;
-    const int4 p = a.prims[t - b * a.P];
-    const int2 *sv = snapc0 + b * a.V;
-    const int2 u0 = __ldcg(sv + p.x), u1 = __ldcg(sv + p.y), u2 = __ldcg(sv + p.z);
-    TriSetup ts;
-    if (part != 2 && tri_setup(u0, u1, u2, W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
-    if (part != 1 && tri_setup(u0, u2, __ldcg(sv + p.w), W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
+    if (slot < kBigListCap) big[slot] = 4 * t + e.part;
+    else sacc[6] = 1;
 }
 
 // Phase 2 over the tracker's primitive list (quadrilateral pairs and single
@@ -227,12 +198,11 @@ __device__ __forceinline__ void draw_deferred(const EvalArgs &a, int cull, const
 // shared out over the whole cluster (in eval_candidate).  `cull` leaves out
 // back faces.  Returns this thread's count of triangles culled for a flagged
 // vertex.
-template <bool kInlineFallback>
 __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::cluster_group &cluster, const int2 *snapc0,
                                           uint32_t *bm, int *big, int *sacc, int4 *queue, int lane, int warp, int nwarp)
 {
     const int W = a.cam.W, H = a.cam.H, Wq = a.cam.Wq;
-    const int NP = a.ch.n_inst * a.P, V = a.V, P = a.P, cap = a.qcap;
+    const int NP = a.ch.n_inst * a.P, cap = a.qcap;
     int culled = 0;
     int *ctr = cluster.map_shared_rank(&sacc[5], 0);
     int cur = chunk_ticket(ctr, lane), qn = 0;
@@ -251,7 +221,7 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::clust
                 if (make_entry(v0, v1, v2, v3, p.w >= 0, culled, e)) {
                     const int size = entry_size(e, W, H);
                     live = size == 1 && !(cull && back_small(e));
-                    if (size == 2) defer_large<kInlineFallback>(t, e, a, cull, bm, big, sacc);
+                    if (size == 2) defer_large(t, e, a, cull, big, sacc);
                 }
             }
             cur = __shfl_sync(0xffffffffu, tk, 0);
@@ -282,36 +252,26 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::clust
         if (last) break;
     }
     __syncthreads();
-    if (!kInlineFallback && sacc[6]) {
-        // the list overflowed: every large primitive of the candidate, a warp
-        // per triangle (drawing twice is harmless under the union); a primitive
-        // counts as large exactly as in the loop above
+    if (sacc[6]) {
+        // the list overflowed: every large primitive of the candidate (drawing
+        // twice is harmless under the union); a primitive counts as large
+        // exactly as in the loop above
         for (int base = warp * 32; base < NP; base += nwarp * 32) {
             const int tt = base + lane;
-            bool l1 = false, l2 = false;
+            PrimEntry e;
+            bool large = false;
             if (tt < NP) {
                 const int4 p = load_prim(a, tt);
                 int2 u0, u1, u2, u3 = make_int2(0, 0);
                 gather_prim(a, snapc0, tt, p, u0, u1, u2, u3);
-                PrimEntry e;
                 int dummy = 0;
-                if (make_entry(u0, u1, u2, u3, p.w >= 0, dummy, e) && entry_size(e, W, H) == 2) {
-                    l1 = e.part != 2;
-                    l2 = e.part != 1;
-                }
+                large = make_entry(u0, u1, u2, u3, p.w >= 0, dummy, e) && entry_size(e, W, H) == 2;
             }
-            for (int part = 1; part <= 2; ++part)
-                for (unsigned mm = __ballot_sync(0xffffffffu, part == 1 ? l1 : l2); mm; mm &= mm - 1) {
-                    const int tu = __shfl_sync(0xffffffffu, tt, __ffs(mm) - 1);
-                    const int b = tu >= P;
-                    const int4 p = a.prims[tu - b * P];
-                    const int2 *sv = snapc0 + b * V;
-                    const int2 u0 = __ldcg(sv + p.x);
-                    const int2 u1 = __ldcg(sv + (part == 1 ? p.y : p.z));
-                    const int2 u2 = __ldcg(sv + (part == 1 ? p.z : p.w));
-                    TriSetup ts;
-                    if (tri_setup(u0, u1, u2, W, H, cull, ts) == 1) raster_warp(ts, bm, Wq, lane);
-                }
+            const unsigned m = __ballot_sync(0xffffffffu, large);
+            const int pos = __popc(m & ((1u << lane) - 1u));
+            for (int b = 0; b < __popc(m); b += cap)
+                draw_rows_large(large && pos >= b && pos < b + cap, e.c0, e.c1, e.c2, e.c3, W, H, cull, bm, Wq, queue, cap,
+                                lane);
         }
     }
     return culled;
@@ -319,7 +279,7 @@ __device__ __forceinline__ int draw_prims(const EvalArgs &a, int cull, cg::clust
 
 // Phase 2 over plain triangles (tris[] of EvalArgs; the index-checked launch on
 // meshes in caller memory).  Deferred-list entries are triangle indices.
-template <bool kInlineFallback, bool kChecked>
+template <bool kChecked>
 __device__ __forceinline__ int draw_tris(const EvalArgs &a, cg::cluster_group &cluster, const int2 *snapc, uint32_t *bm,
                                       int *big, int *sacc, int lane, int warp, int nwarp)
 {
@@ -351,7 +311,7 @@ __device__ __forceinline__ int draw_tris(const EvalArgs &a, cg::cluster_group &c
             b2 = t2 >= a.T;
             tri2 = load_tri<kChecked>(a, t2);
         }
-        if (t0 < NT) culled += draw_one_tri<kInlineFallback>(v0, v1, v2, t0, a, a.cull, bm, big, sacc);
+        if (t0 < NT) culled += draw_one_tri(v0, v1, v2, t0, a, a.cull, bm, big, sacc);
         cur = nx1;
         t0 = t1;
         v0 = w0;
@@ -374,7 +334,7 @@ __device__ __forceinline__ int draw_tris(const EvalArgs &a, cg::cluster_group &c
         tri_setup(u0, u1, u2, W, H, a.cull, t);
         raster_warp(t, bm, Wq, lane);
     }
-    if (!kInlineFallback && sacc[6]) {  // the list overflowed: every large triangle of the candidate, a warp each (drawing twice is harmless)
+    if (sacc[6]) {  // the list overflowed: every large triangle of the candidate, a warp each (drawing twice is harmless)
         for (int base = warp * 32; base < NT; base += nwarp * 32) {
             const int tt = base + lane;
             bool large = false;
@@ -399,7 +359,7 @@ __device__ __forceinline__ int draw_tris(const EvalArgs &a, cg::cluster_group &c
     return culled;
 }
 
-template <bool kInlineFallback, bool kChecked = false, bool kQuads = true>
+template <bool kChecked = false, bool kQuads = true>
 __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const uint32_t *mask_override,
                                                unsigned tell_ctas, bool dependent_launch)
 {
@@ -490,9 +450,9 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     int cull = a.cull;
     if (kQuads && a.closed)
         cull |= !__any_sync(0xffffffffu, lane < K && *cluster.map_shared_rank(&sacc[8], lane < K ? lane : 0) != 0);
-    int culled = kQuads ? draw_prims<kInlineFallback>(a, cull, cluster, snapc, bm, big, sacc, queues + a.qcap * kQueueEntryBytes / 16 * warp, lane,
+    int culled = kQuads ? draw_prims(a, cull, cluster, snapc, bm, big, sacc, queues + a.qcap * kQueueEntryBytes / 16 * warp, lane,
                                                        warp, nwarp)
-                        : draw_tris<kInlineFallback, kChecked>(a, cluster, snapc, bm, big, sacc, lane, warp, nwarp);
+                        : draw_tris<kChecked>(a, cluster, snapc, bm, big, sacc, lane, warp, nwarp);
     cluster.sync();
     if (kQuads) {
         // the large primitives deferred by every CTA of the cluster, shared out
@@ -508,12 +468,34 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
         }
         const int total = __shfl_sync(0xffffffffu, incl, 7);
         if (total > 0) {  // the same in every CTA: the barrier below is uniform
+            // a ticket stands for `per` entries: one while there are warps enough
+            // (its rows go to the lanes), more when the list is long
             int *ctr = cluster.map_shared_rank(&sacc[7], 0);
-            for (int e = chunk_ticket(ctr, lane); e < total; e = chunk_ticket(ctr, lane)) {
-                const int r = __popc(__ballot_sync(0xffffffffu, lane < K && incl <= e));
-                const int start = __shfl_sync(0xffffffffu, incl - cnt, r);
-                const int ent = cluster.map_shared_rank(big, r)[e - start];
-                draw_deferred(a, cull, snapc, ent, bm, lane);
+            const int per = min(a.qcap, (total + K * nwarp - 1) / (K * nwarp));
+            for (int e0 = chunk_ticket(ctr, lane) * per; e0 < total; e0 = chunk_ticket(ctr, lane) * per) {
+                const int e = e0 + lane;
+                int r = 0, start = 0;
+                for (int q = 0; q < K; ++q) {
+                    const int v = __shfl_sync(0xffffffffu, incl, q);
+                    if (v <= e) {
+                        r = q + 1;
+                        start = v;
+                    }
+                }
+                const bool live = lane < per && e < total;
+                int2 c0 = make_int2(0, 0), c1 = c0, c2 = c0, c3 = make_int2(kSnapFlag, kSnapFlag);
+                if (live) {
+                    const int ent = cluster.map_shared_rank(big, r)[e - start], t = ent >> 2, part = ent & 3;
+                    const int b = t >= a.P;
+                    const int4 p = a.prims[t - b * a.P];
+                    const int2 *sv = snapc + b * a.V;
+                    c0 = __ldcg(sv + p.x);
+                    c1 = __ldcg(sv + (part == 2 ? p.z : p.y));
+                    c2 = __ldcg(sv + (part == 2 ? p.w : p.z));
+                    if (part == 0) c3 = __ldcg(sv + p.w);
+                }
+                draw_rows_large(live, c0, c1, c2, c3, a.cam.W, H, cull, bm, Wq, queues + a.qcap * kQueueEntryBytes / 16 * warp,
+                                a.qcap, lane);
             }
             cluster.sync();  // every deferred primitive drawn before the bitmaps are read
         }
@@ -604,14 +586,14 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
 __global__ void __launch_bounds__(256, 4) k_eval(EvalArgs a)
 {
     griddep_launch_dependents();
-    eval_candidate<false>(a, blockIdx.y, nullptr, gridDim.x * gridDim.y, true);
+    eval_candidate<>(a, blockIdx.y, nullptr, gridDim.x * gridDim.y, true);
 }
 
 // The same with index checks: meshes in the caller's device memory
 // (eval_population_noalloc), whose indices the host cannot validate.
 __global__ void __launch_bounds__(256, 4) k_eval_checked(EvalArgs a)
 {
-    eval_candidate<false, true, false>(a, blockIdx.y, nullptr, 0u, false);
+    eval_candidate<true, false>(a, blockIdx.y, nullptr, 0u, false);
 }
 
 // Persistent batched evaluation: a fixed grid of clusters pulls (instance,

@@ -386,18 +386,6 @@ static __device__ void raster_warp(const TriSetup &t, uint32_t *bm, int Wq, int 
     }
 }
 
-// One thread, int64, any size: the batched kernel's fallback when a CTA's
-// deferred list is full.
-static __device__ void raster_serial(const TriSetup &t, uint32_t *bm, int Wq)
-{
-    for (int i = t.i0; i <= t.i1; ++i)
-        for (int j = t.j0; j <= t.j1; ++j) {
-            long long Px = 256LL * j, Py = 256LL * i;
-            if ((edge64(t, 0, Px, Py) | edge64(t, 1, Px, Py) | edge64(t, 2, Px, Py)) >= 0)
-                atomicOr(bm + (size_t)i * Wq + (j >> 5), 1u << (j & 31));
-        }
-}
-
 // ----------------------------------------------------------------------------
 // Quadrilaterals: two mesh triangles T1 = (a, b, c) and T2 = (a, c, d) that share
 // the edge a-c.  The top-left rule covers a pixel centre p exactly when the
@@ -411,53 +399,12 @@ static __device__ void raster_serial(const TriSetup &t, uint32_t *bm, int Wq)
 // one bounding box instead of two.  Anything else (a fold at a silhouette edge,
 // a non-convex or degenerate pair, a flagged vertex) is drawn as two triangles.
 // ----------------------------------------------------------------------------
-struct QuadSetup {
-    int x[4], y[4];       // snapped corners, positive orientation
-    int j0, j1, i0, i1;   // pixel bbox clamped to the image
-    int spanx, spany;     // corner bbox extent in 1/256 px
-};
-
 // Twice the signed area of (p, q, r); exact in int32 when every coordinate
 // difference is below 2^15.
 __device__ __forceinline__ long long orient2(int2 p, int2 q, int2 r, bool narrow)
 {
     if (narrow) return (long long)((q.x - p.x) * (r.y - p.y) - (r.x - p.x) * (q.y - p.y));
     return (long long)(q.x - p.x) * (long long)(r.y - p.y) - (long long)(r.x - p.x) * (long long)(q.y - p.y);
-}
-
-// Returns 0 = nothing to draw (no pixel centre in the corners' clipped box, or
-// both triangles culled as back faces), 1 = draw the quadrilateral, 3 = draw the
-// two triangles separately (tri_setup on each; it also counts flagged ones).
-__device__ __forceinline__ int quad_setup(int2 a, int2 b, int2 c, int2 d, int W, int H, int cull, QuadSetup &q)
-{
-    if (a.x == kSnapFlag || b.x == kSnapFlag || c.x == kSnapFlag || d.x == kSnapFlag) return 3;
-    const int xmn = min(min(a.x, b.x), min(c.x, d.x)), xmx = max(max(a.x, b.x), max(c.x, d.x));
-    const int ymn = min(min(a.y, b.y), min(c.y, d.y)), ymx = max(max(a.y, b.y), max(c.y, d.y));
-    // each triangle's box lies inside this one: an empty box leaves both empty
-    q.j0 = max(0, (xmn + 255) >> 8);
-    q.j1 = min(W - 1, xmx >> 8);
-    q.i0 = max(0, (ymn + 255) >> 8);
-    q.i1 = min(H - 1, ymx >> 8);
-    if (q.j0 > q.j1 || q.i0 > q.i1) return 0;
-    q.spanx = xmx - xmn;
-    q.spany = ymx - ymn;
-    const bool narrow = q.spanx < (1 << 15) && q.spany < (1 << 15);
-    const long long A1 = orient2(a, b, c, narrow), A2 = orient2(a, c, d, narrow);
-    const long long Da = orient2(b, d, a, narrow), Dc = orient2(b, d, c, narrow);
-    // same non-zero orientation, and a, c strictly on opposite sides of b-d
-    const bool convex = ((A1 > 0 && A2 > 0) || (A1 < 0 && A2 < 0)) && ((Da > 0 && Dc < 0) || (Da < 0 && Dc > 0));
-    if (!convex) return 3;
-    if (cull && A1 > 0) return 0;
-    if (A1 < 0) {  // reverse the corner order: positive orientation
-        int2 t = b;
-        b = d;
-        d = t;
-    }
-    q.x[0] = a.x; q.y[0] = a.y;
-    q.x[1] = b.x; q.y[1] = b.y;
-    q.x[2] = c.x; q.y[2] = c.y;
-    q.x[3] = d.x; q.y[3] = d.y;
-    return 1;
 }
 
 // ----------------------------------------------------------------------------
@@ -638,6 +585,131 @@ __device__ __forceinline__ void draw_rows(bool live, int2 c0, int2 c1, int2 c2, 
             c1 = mid;
             c2 = end;
             A = orient_small(c0, c1, c2);
+        }
+    }
+}
+
+// floor(n / d) for 0 < d < 2^24, clamped to [-cap - 2, cap + 1] (cap < 2^21): a
+// quotient in FP32, once clamped within one of the floor, is put right by its
+// exact remainder.
+__device__ __forceinline__ int floor_div_clamped(long long n, int d, int cap)
+{
+    const float f = fminf(fmaxf((float)n * rcp_approx((float)d), (float)(-cap - 1)), (float)cap);
+    int q = (int)floorf(f);
+    const long long r = n - (long long)q * d;
+    if (r < 0) --q;
+    if (r >= d) ++q;
+    return q;
+}
+
+// The columns [lo, hi] of row i that the edge p -> q leaves covered (e >= 0, see
+// edge64): one floor of the edge function over its step.  An edge of no length
+// leaves all.
+__device__ __forceinline__ void clip_row(int2 p, int2 q, int i, int &lo, int &hi)
+{
+    const int dx = q.x - p.x, dy = q.y - p.y;
+    const int bias = (dy < 0 || (dy == 0 && dx > 0)) ? 0 : 1;
+    // e at column lo; e falls by 256 dy per column
+    const long long e = (long long)dx * (256 * i - p.y) - (long long)dy * (256 * lo - p.x) - bias;
+    if (dy == 0) {
+        if (dx != 0 && e < 0) hi = lo - 1;
+        return;
+    }
+    const int n = hi - lo + 1, f = floor_div_clamped(e >> 8, abs(dy), max(n, 0));
+    if (dy > 0) hi = min(hi, lo + f);      // columns up to lo + floor(e / 256 dy)
+    else lo = max(lo, lo - f);             // from lo + ceil(-e / 256 |dy|)
+}
+
+// draw_rows for primitives of any size: a row of pixels per lane again, but the
+// row's covered columns come from the edges (a convex polygon covers one run of
+// them) and are entered a word at a time.  The entries of the warp's table are
+// the corners (int4 [n] twice) and the first task and row (int2 [n]).
+// 1280x1024, two instruments of 40k triangles, 256 candidates: with a pixel per
+// lane and 64-bit edge functions at each, this phase took 76-160k cycles of the
+// kernel's 160-250k, now 8-11k of 90-100k (1.90 -> 1.03 ms a launch).
+static __device__ void draw_rows_large(bool live, int2 c0, int2 c1, int2 c2, int2 c3, int W, int H, int cull, uint32_t *bm,
+                                       int Wq, int4 *tab, int n, int lane)
+{
+    int4 *tab_a = tab, *tab_b = tab + n;
+    int2 *tab_m = reinterpret_cast<int2 *>(tab + 2 * n);
+    bool tri = c3.x == kSnapFlag, two = false;
+    const int2 mid = c2, end = c3;
+    long long A = 0;
+    if (live) {
+        A = orient2(c0, c1, c2, false);
+        if (!tri) {
+            const long long A2 = orient2(c0, c2, c3, false), Da = orient2(c1, c3, c0, false), Dc = orient2(c1, c3, c2, false);
+            // same non-zero orientation, and c0, c2 strictly on opposite sides of c1-c3
+            if (!(((A > 0 && A2 > 0) || (A < 0 && A2 < 0)) && ((Da > 0 && Dc < 0) || (Da < 0 && Dc > 0)))) tri = two = true;
+        }
+    }
+    for (;;) {
+        bool on = live && A != 0 && !(cull && A > 0);
+        int i0 = 0, rows = 0;
+        if (on) {
+            if (A < 0) {  // positive orientation
+                const int2 t = c1;
+                c1 = tri ? c2 : c3;
+                (tri ? c2 : c3) = t;
+            }
+            if (tri) c3 = c2;
+            i0 = max(0, (min(min(c0.y, c1.y), min(c2.y, c3.y)) + 255) >> 8);
+            const int i1 = min(H - 1, max(max(c0.y, c1.y), max(c2.y, c3.y)) >> 8);
+            on = i0 <= i1;
+            rows = on ? i1 - i0 + 1 : 0;
+        }
+        int incl = rows;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31), first = incl - rows;
+        const unsigned lm = __ballot_sync(0xffffffffu, on);
+        if (on) {
+            const int slot = __popc(lm & ((1u << lane) - 1u));
+            tab_a[slot] = make_int4(c0.x, c0.y, c1.x, c1.y);
+            tab_b[slot] = make_int4(c2.x, c2.y, c3.x, c3.y);
+            tab_m[slot] = make_int2(first, i0);
+        }
+        __syncwarp();
+        for (int base = 0; base < total; base += 32) {
+            // the polygon of task base + lane, as in draw_rows
+            const int rel = first - base;
+            const unsigned starts = __reduce_or_sync(0xffffffffu, on && rel >= 0 && rel < 32 ? 1u << rel : 0u);
+            const int before = __popc(__ballot_sync(0xffffffffu, on && rel < 0));
+            const int t = base + lane;
+            if (t < total) {
+                const int slot = before - 1 + __popc(starts & (0xffffffffu >> (31 - lane)));
+                const int4 pa = tab_a[slot], pb = tab_b[slot];
+                const int2 mv = tab_m[slot];
+                const int i = t - mv.x + mv.y;
+                int lo = max(0, (min(min(pa.x, pa.z), min(pb.x, pb.z)) + 255) >> 8);
+                int hi = min(W - 1, max(max(pa.x, pa.z), max(pb.x, pb.z)) >> 8);
+                clip_row(make_int2(pa.x, pa.y), make_int2(pa.z, pa.w), i, lo, hi);
+                clip_row(make_int2(pa.z, pa.w), make_int2(pb.x, pb.y), i, lo, hi);
+                clip_row(make_int2(pb.x, pb.y), make_int2(pb.z, pb.w), i, lo, hi);
+                clip_row(make_int2(pb.z, pb.w), make_int2(pa.x, pa.y), i, lo, hi);
+                if (lo <= hi) {
+                    uint32_t *w = bm + i * Wq;
+                    for (int k = lo >> 5; k <= hi >> 5; ++k) {
+                        uint32_t bits = 0xffffffffu;
+                        if (k == lo >> 5) bits &= 0xffffffffu << (lo & 31);
+                        if (k == hi >> 5) bits &= 0xffffffffu >> (31 - (hi & 31));
+                        atomicOr(w + k, bits);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (!__any_sync(0xffffffffu, two)) break;
+        live = two;  // the second triangles
+        two = false;
+        tri = true;
+        if (live) {
+            c1 = mid;
+            c2 = end;
+            A = orient2(c0, c1, c2, false);
         }
     }
 }
