@@ -199,10 +199,10 @@ static void tracker_free(trk_tracker *t)
     delete t;
 }
 
-static LaunchCfg auto_launch(const trk_tracker *t, const EvalArgs &a)
+static LaunchCfg auto_launch(const trk_tracker *t, const EvalArgs &a, int threads)
 {
-    LaunchCfg lc;
-    lc.threads = t->cfg.block_threads > 0 ? t->cfg.block_threads : 256;
+    LaunchCfg lc{};
+    lc.threads = t->cfg.block_threads > 0 ? t->cfg.block_threads : threads;
     if (t->cfg.cluster > 0) {
         lc.cluster = t->cfg.cluster;
     } else {
@@ -212,8 +212,9 @@ static LaunchCfg auto_launch(const trk_tracker *t, const EvalArgs &a)
         long long work = (long long)(t->V + t->T) * t->ch.n_inst;
         long long per_cta = (long long)lc.threads * 2;
         lc.cluster = (int)std::min<long long>(8, std::max<long long>(1, (work + per_cta - 1) / per_cta));
+        lc.work = work;
     }
-    lc.smem = eval_smem_bytes(a);
+    lc.smem = eval_smem_bytes(a, lc.threads);
     return lc;
 }
 
@@ -415,8 +416,8 @@ trk_status tracker_create(const trk_link_mesh *meshes, int32_t n_meshes, const t
     EvalArgs probe{};
     probe.ch = t->ch;
     probe.cam = t->cam;
-    t->lc = auto_launch(t, probe);
-    t->lc_front = t->lc;
+    t->lc = auto_launch(t, probe, eval_wide_threads(t->ch, t->cam));
+    t->lc_front = auto_launch(t, probe, 256);
     const bool binned_ok = binned_layout(t, probe);
     if (cfg->raster == TRK_RASTER_BINNED && !binned_ok) {
         tracker_free(t);
@@ -449,7 +450,8 @@ trk_status tracker_create(const trk_link_mesh *meshes, int32_t n_meshes, const t
             tracker_free(t);
             return inval("image too large for the shared-memory bitmap");
         }
-    } else if ((e = prepare_eval(t->lc.smem)) != cudaSuccess) {
+    } else if ((e = prepare_eval(t->lc.smem, t->lc.threads)) != cudaSuccess ||
+               (t->cfg.cluster == 0 && (e = eval_cluster_fit(t->lc)) != cudaSuccess)) {
         tracker_free(t);
         return cuda_fail(e, "eval kernel attributes");
     }
@@ -703,7 +705,7 @@ trk_status cmaes_create(trk_tracker *t, int32_t lam, const double *mean_host, co
         return cuda_fail(e, "cmaes upload");
     }
     if ((e = cudaMemset(es->done, 0, sizeof(unsigned))) != cudaSuccess ||
-        (t->raster == TRK_RASTER_CLUSTER && (e = prepare_eval(std::max(t->lc.smem, tell_smem_bytes()))) != cudaSuccess) ||
+        (t->raster == TRK_RASTER_CLUSTER && (e = prepare_eval(std::max(t->lc.smem, tell_smem_bytes()), t->lc.threads)) != cudaSuccess) ||
         (e = launch_cma_reset(es->k, es->st, es->mean0, false, nullptr, t->ch.n_inst, 0)) != cudaSuccess ||
         (e = cudaDeviceSynchronize()) != cudaSuccess) {
         cmaes_free(es);

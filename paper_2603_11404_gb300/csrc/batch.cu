@@ -44,6 +44,7 @@ struct trk_batch {
     struct Group {
         int item_off = 0, n_items = 0;
         size_t smem = 0;                // the largest bitmap of the group's instances
+        std::vector<int> insts;
         LaunchCfg lc{};
         int n_clusters = 0;
     };
@@ -101,7 +102,7 @@ static trk_status batch_configure(trk_batch *b, int cluster, int threads)
     size_t smem = 0;
     for (int i = 0; i < b->n; ++i) {
         max_inst = std::max(max_inst, b->tr[i]->ch.n_inst);
-        smem = std::max(smem, eval_smem_bytes(b->hdescs[i]));
+        smem = std::max(smem, eval_smem_bytes(b->hdescs[i], 256));
     }
     if (threads <= 0) threads = 256;
     if (threads > 256 || threads % 32 || threads < 32 * max_inst) return bfail(TRK_EINVAL, "batch threads");
@@ -111,12 +112,23 @@ static trk_status batch_configure(trk_batch *b, int cluster, int threads)
     int total = 0;
     for (trk_batch::Group &g : b->groups) {
         int maxc = 0;
-        cudaError_t e = prepare_eval_batch(g.smem, cluster, threads, &maxc);
+        g.lc = LaunchCfg{cluster, threads, g.smem, 0};
+        if (threads == 256) {
+            // wider CTAs where fewer than four fit an SM (see eval_wide_threads):
+            // the shape that every instance of the group allows
+            int wide = 1024;
+            for (int i : g.insts) wide = std::min(wide, eval_wide_threads(b->hdescs[i].ch, b->hdescs[i].cam));
+            if (wide > 256) {
+                g.lc.threads = wide;
+                g.lc.qcap = 32;
+                for (int i : g.insts)
+                    g.lc.qcap = std::min(g.lc.qcap, eval_queue_cap(b->hdescs[i].ch, b->hdescs[i].cam, wide));
+                for (int i : g.insts) g.lc.smem = std::max(g.lc.smem, eval_smem_bytes(b->hdescs[i], wide));
+            }
+        }
+        cudaError_t e = prepare_eval_batch(g.lc.smem, cluster, g.lc.threads, &maxc);
         if (e != cudaSuccess) return bfail(TRK_ECUDA, cudaGetErrorString(e));
         if (maxc <= 0) return bfail(TRK_EINVAL, "launch shape does not fit on the device");
-        g.lc.cluster = cluster;
-        g.lc.threads = threads;
-        g.lc.smem = g.smem;
         g.n_clusters = std::min(maxc, g.n_items);
         total += g.n_clusters;
     }
@@ -231,7 +243,7 @@ trk_status batch_create(trk_tracker *const *trackers, trk_cmaes *const *optimise
         set_last_error(cudaGetErrorString(e));
         return TRK_ECUDA;
     }
-    auto per_sm = [&](int i) { return (long long)sm_smem / (long long)(eval_smem_bytes(b->hdescs[i]) + 4096); };
+    auto per_sm = [&](int i) { return (long long)sm_smem / (long long)(eval_smem_bytes(b->hdescs[i], 256) + 4096); };
     auto cost = [&](int i) { return (long long)(b->tr[i]->V + b->tr[i]->T) * b->tr[i]->ch.n_inst; };
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
@@ -249,7 +261,8 @@ trk_status batch_create(trk_tracker *const *trackers, trk_cmaes *const *optimise
         }
         trk_batch::Group &g = b->groups.back();
         g.n_items += b->lam[i];
-        g.smem = std::max(g.smem, eval_smem_bytes(b->hdescs[i]));
+        g.smem = std::max(g.smem, eval_smem_bytes(b->hdescs[i], 256));
+        g.insts.push_back(i);
         for (int c = 0; c < b->lam[i]; ++c) items.push_back(make_int2(i, c));
     }
     const int G = (int)b->groups.size();

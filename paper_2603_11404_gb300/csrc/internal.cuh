@@ -110,9 +110,12 @@ struct __align__(16) EvalArgs {
 };
 
 struct LaunchCfg {
-    int cluster;           // CTAs per candidate
+    int cluster;           // CTAs per candidate (the most of them when fit[1] > 0)
     int threads;           // threads per CTA
     size_t smem;           // dynamic shared memory per CTA
+    int qcap;              // k_eval_batch_wide: drawing-queue entries per warp
+    int fit[9];            // k_eval: clusters of 1..8 CTAs resident at once (0: `cluster` as it is)
+    long long work;        // vertices and triangles of a candidate
 };
 
 // Constant-velocity Kalman filter on the frame estimates (temporal filtering,
@@ -196,9 +199,11 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
                               cudaStream_t s, const int *tell_last_dev = nullptr);
 cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_clusters);
 cudaError_t launch_pack_mask(const uint8_t *mask, uint32_t *packed, int W, int H, int Wq, cudaStream_t s);
-size_t eval_smem_bytes(const EvalArgs &a);
-int eval_queue_cap(const ChainDev &ch, const CamDev &cam);
-cudaError_t prepare_eval(size_t smem);
+size_t eval_smem_bytes(const EvalArgs &a, int threads);
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads);
+int eval_wide_threads(const ChainDev &ch, const CamDev &cam);
+cudaError_t prepare_eval(size_t smem, int threads);
+cudaError_t eval_cluster_fit(LaunchCfg &cfg);
 void set_last_error(const char *msg);  // the text tracker_last_error() returns
 int eval_max_threads();
 
@@ -271,7 +276,7 @@ inline void apply_mesh(trk::EvalArgs &a, const trk_tracker *t)
     a.prims = t->prims;
     a.P = t->P;
     a.closed = t->closed ? 1 : 0;
-    a.qcap = trk::eval_queue_cap(t->ch, t->cam);
+    a.qcap = trk::eval_queue_cap(t->ch, t->cam, 256);
 }
 
 // The tracker's keypoint term into a launch's arguments.

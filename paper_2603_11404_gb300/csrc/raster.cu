@@ -35,12 +35,13 @@ namespace cg = cooperative_groups;
 namespace trk {
 
 // Front of the dynamic shared memory: the composition's scratch and, once the
-// frames are composed, the warps' drawing queues (at most 8 warps).
+// frames are composed, the warps' drawing queues (room for 8 warps at least).
 constexpr int kQueueEntryBytes = 40;  // an entry of draw_rows' table; a queued primitive takes 32
 
-__host__ __device__ inline size_t front_smem_bytes(int n_inst, int qcap)
+__host__ __device__ inline size_t front_smem_bytes(int n_inst, int qcap, int threads)
 {
-    const size_t scr = (size_t)n_inst * kComposeScratch * sizeof(float2), q = (size_t)8 * qcap * kQueueEntryBytes;
+    const size_t warps = threads > 256 ? threads / 32 : 8;
+    const size_t scr = (size_t)n_inst * kComposeScratch * sizeof(float2), q = warps * qcap * kQueueEntryBytes;
     return scr > q ? scr : q;
 }
 
@@ -376,7 +377,7 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *scr = reinterpret_cast<float2 *>(smem);                           // [nI*kComposeScratch]
     int4 *queues = reinterpret_cast<int4 *>(smem);                            // [nwarp][qcap entries]: phase 2, over scr
-    uint32_t *bm = reinterpret_cast<uint32_t *>(smem + front_smem_bytes(nI, a.qcap));  // [H*Wq]
+    uint32_t *bm = reinterpret_cast<uint32_t *>(smem + front_smem_bytes(nI, a.qcap, blockDim.x));  // [H*Wq]
     float *sM = reinterpret_cast<float *>(bm + ((nwords + 3) & ~3));          // [nI*nF*24]
     int *big = reinterpret_cast<int *>(sM + nI * nF * 24);                    // [kBigListCap]
     // [kAccWords]: s I m culled, big-list count, chunk ticket counter, big-list
@@ -589,6 +590,13 @@ __global__ void __launch_bounds__(256, 4) k_eval(EvalArgs a)
     eval_candidate<>(a, blockIdx.y, nullptr, gridDim.x * gridDim.y, true);
 }
 
+// The same in CTAs of up to 1024 threads (see eval_wide_threads).
+__global__ void __launch_bounds__(1024, 1) k_eval_wide(EvalArgs a)
+{
+    griddep_launch_dependents();
+    eval_candidate<>(a, blockIdx.y, nullptr, gridDim.x * gridDim.y, true);
+}
+
 // The same with index checks: meshes in the caller's device memory
 // (eval_population_noalloc), whose indices the host cannot validate.
 __global__ void __launch_bounds__(256, 4) k_eval_checked(EvalArgs a)
@@ -606,10 +614,9 @@ __global__ void __launch_bounds__(256, 4) k_eval_checked(EvalArgs a)
 // rewrites between ticks (read with ld.cv, never from a cached line), and the
 // cluster that draws the launch's last ticket leaves the queue counter at zero
 // for the next tick.  Without kTell the updates are a separate launch.
-template <bool kTell>
-__global__ void __launch_bounds__(256, 3) k_eval_batch(const EvalArgs *descs, const uint32_t *const *masks,
-                                                       const int2 *items, int n_items, unsigned *next_item,
-                                                       const int *tell_last)
+template <bool kTell, bool kWide>
+__device__ __forceinline__ void eval_batch_body(const EvalArgs *descs, const uint32_t *const *masks, const int2 *items,
+                                                int n_items, unsigned *next_item, const int *tell_last, int wide_qcap)
 {
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ int s_item;
@@ -653,8 +660,27 @@ __global__ void __launch_bounds__(256, 3) k_eval_batch(const EvalArgs *descs, co
             __syncthreads();
             tell = (unsigned)s_args.lam * gridDim.x;  // every CTA of every candidate of the instance
         }
-        eval_candidate<true>(s_args, ic.y, masks ? masks[ic.x] : nullptr, tell, false);
+        if (kWide) {  // the descriptor's queues are sized for 256 threads
+            if (threadIdx.x == 0) s_args.qcap = wide_qcap;
+            __syncthreads();
+        }
+        eval_candidate<>(s_args, ic.y, masks ? masks[ic.x] : nullptr, tell, false);
     }
+}
+
+template <bool kTell>
+__global__ void __launch_bounds__(256, 3) k_eval_batch(const EvalArgs *descs, const uint32_t *const *masks,
+                                                       const int2 *items, int n_items, unsigned *next_item,
+                                                       const int *tell_last)
+{
+    eval_batch_body<kTell, false>(descs, masks, items, n_items, next_item, tell_last, 0);
+}
+
+__global__ void __launch_bounds__(1024, 1) k_eval_batch_wide(const EvalArgs *descs, const uint32_t *const *masks,
+                                                             const int2 *items, int n_items, unsigned *next_item,
+                                                             int qcap)
+{
+    eval_batch_body<false, true>(descs, masks, items, n_items, next_item, nullptr, qcap);
 }
 
 cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *masks_dev, const int2 *items_dev,
@@ -674,6 +700,9 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
     attr[0].val.clusterDim.z = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
+    if (cfg.threads > 256)  // batches only: the updates are a launch of their own
+        return cudaLaunchKernelEx(&lc, k_eval_batch_wide, descs_dev, masks_dev, items_dev, n_items, next_item_dev,
+                                  cfg.qcap);
     return tell_last_dev ? cudaLaunchKernelEx(&lc, k_eval_batch<true>, descs_dev, masks_dev, items_dev, n_items,
                                               next_item_dev, tell_last_dev)
                          : cudaLaunchKernelEx(&lc, k_eval_batch<false>, descs_dev, masks_dev, items_dev, n_items,
@@ -682,8 +711,9 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
 
 cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_clusters)
 {
-    cudaError_t e = ensure_smem_attr((const void *)k_eval_batch<false>, smem);
-    if (e == cudaSuccess) e = ensure_smem_attr((const void *)k_eval_batch<true>, smem);
+    const bool wide = threads > 256;
+    cudaError_t e = ensure_smem_attr(wide ? (const void *)k_eval_batch_wide : (const void *)k_eval_batch<false>, smem);
+    if (e == cudaSuccess && !wide) e = ensure_smem_attr((const void *)k_eval_batch<true>, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cluster, 1, 1);
@@ -696,6 +726,7 @@ cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_c
     attr[0].val.clusterDim.z = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
+    if (wide) return cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch_wide, &lc);
     // both forms (with and without the fused updates) must fit the shape
     int with_tell = 0;
     if ((e = cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch<false>, &lc)) != cudaSuccess ||
@@ -707,26 +738,97 @@ cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_c
 
 size_t tell_smem_bytes() { return sizeof(TellSmem); }
 
-size_t eval_smem_bytes(const EvalArgs &a)
-{
-    size_t nwords = (size_t)a.cam.H * a.cam.Wq;
-    return front_smem_bytes(a.ch.n_inst, eval_queue_cap(a.ch, a.cam)) + ((nwords + 3) & ~(size_t)3) * 4 +
-           (size_t)a.ch.n_inst * a.ch.n_frames * 24 * 4 + (size_t)kBigListCap * 4 + kAccWords * 4;
-}
-
-// Entries per warp of the drawing queue: one per lane, or what the composition
-// scratch has room for when the image's bitmap leaves no more.
-int eval_queue_cap(const ChainDev &ch, const CamDev &cam)
+// Shared memory of a CTA behind its front.
+static size_t eval_rest_bytes(const ChainDev &ch, const CamDev &cam)
 {
     const size_t nwords = (size_t)cam.H * cam.Wq;
-    const size_t rest = ((nwords + 3) & ~(size_t)3) * 4 + (size_t)ch.n_inst * ch.n_frames * 24 * 4 +
-                        (size_t)kBigListCap * 4 + kAccWords * 4;
-    return front_smem_bytes(ch.n_inst, 32) + rest <= 227 * 1024 ? 32 : 8;
+    return ((nwords + 3) & ~(size_t)3) * 4 + (size_t)ch.n_inst * ch.n_frames * 24 * 4 + (size_t)kBigListCap * 4 +
+           kAccWords * 4;
+}
+
+size_t eval_smem_bytes(const EvalArgs &a, int threads)
+{
+    return front_smem_bytes(a.ch.n_inst, eval_queue_cap(a.ch, a.cam, threads), threads) + eval_rest_bytes(a.ch, a.cam);
+}
+
+// CTAs of one shape that an SM holds: 1024 threads at the kernel's 64 registers,
+// 228 KB of shared memory (a KB per CTA is reserved, and a little is static).
+static int eval_ctas_per_sm(const ChainDev &ch, const CamDev &cam, int threads, int qcap)
+{
+    const size_t smem = front_smem_bytes(ch.n_inst, qcap, threads) + eval_rest_bytes(ch, cam) + 2048;
+    return (int)std::min<size_t>(1024 / threads, 228 * 1024 / smem);
+}
+
+// Entries per warp of the drawing queue: one per lane, or as many (16 at least)
+// as leave an SM as many CTAs: at 700x493 a full queue would cost it the fourth,
+// and with it a population of 64 the single wave of its clusters (51.6 us, with
+// 24 entries 37.7).  8 where the image's bitmap leaves no more.
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads)
+{
+    int cap = 32;
+    while (cap > 16 && eval_ctas_per_sm(ch, cam, threads, cap) < eval_ctas_per_sm(ch, cam, threads, 16)) cap -= 4;
+    return front_smem_bytes(ch.n_inst, cap, threads) + eval_rest_bytes(ch, cam) <= 227 * 1024 ? cap : 8;
+}
+
+// Threads per CTA that fill an SM (1024 at the kernel's 64 registers) when its
+// shared memory holds few of the image's bitmaps: 256 where four fit, 512 for
+// two or three, 1024 for one.  Two instruments of 40k triangles, 256 candidates,
+// one CTA each: 1280x1024 742 us with 256 threads, 470 with 512, 383 with 1024;
+// 960x768 410 and 350; 800x600 370 and 302 (320 threads, three to an SM: 352).
+int eval_wide_threads(const ChainDev &ch, const CamDev &cam)
+{
+    for (int n = 4; n; n /= 2)
+        if (eval_ctas_per_sm(ch, cam, 1024 / n, 16) == n) return 1024 / n;
+    return 256;
+}
+
+// Clusters of every size that are resident at once.
+cudaError_t eval_cluster_fit(LaunchCfg &cfg)
+{
+    for (int k = 1; k <= cfg.cluster; ++k) {
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(k, 1, 1);
+        lc.blockDim = dim3(cfg.threads, 1, 1);
+        lc.dynamicSmemBytes = cfg.smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = k;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        lc.attrs = attr;
+        lc.numAttrs = 1;
+        const cudaError_t e = cfg.threads > 256 ? cudaOccupancyMaxActiveClusters(&cfg.fit[k], k_eval_wide, &lc)
+                                                : cudaOccupancyMaxActiveClusters(&cfg.fit[k], k_eval, &lc);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// CTAs per candidate of a population of lam: as many as leave all its clusters
+// resident at once.  More CTAs shorten a candidate's way but cost it barriers and
+// bitmaps, so a second wave pays only with much work per thread and waves
+// nearly full.  20k triangles, CTAs 1/2/4/8 (us): 640x512 64 candidates 108/62/43/41, 128
+// candidates 108/70/62/69, 256 candidates 127/109/99/122; 960x768 91/56/56/83, 91/80/100/153,
+// 144/145/169/282; 1280x1024 90/61/93/206, 89/115/178/375, 170/222/341/717.
+static int eval_cluster(const LaunchCfg &cfg, int lam)
+{
+    int k = cfg.cluster;
+    if (cfg.fit[1] <= 0) return k;
+    while (k > 1 && lam > cfg.fit[k]) --k;
+    if (cfg.threads == 256 && k <= 2 && 2 * k <= cfg.cluster && lam <= cfg.fit[k] && cfg.fit[2 * k] > 0 &&
+        cfg.work >= 24LL * 2 * k * cfg.threads) {
+        const int fit = cfg.fit[2 * k], waves = (lam + fit - 1) / fit;
+        if (5 * lam >= 4 * waves * fit) k *= 2;
+    }
+    return k;
 }
 
 int eval_max_threads() { return 1024; }
 
-cudaError_t prepare_eval(size_t smem) { return ensure_smem_attr((const void *)k_eval, smem); }
+cudaError_t prepare_eval(size_t smem, int threads)
+{
+    return ensure_smem_attr(threads > 256 ? (const void *)k_eval_wide : (const void *)k_eval, smem);
+}
 
 cudaError_t launch_eval_checked(const EvalArgs &a, const LaunchCfg &cfg, cudaStream_t s)
 {
@@ -748,18 +850,21 @@ cudaError_t launch_eval_checked(const EvalArgs &a, const LaunchCfg &cfg, cudaStr
     return cudaLaunchKernelEx(&lc, k_eval_checked, a);
 }
 
-cudaError_t launch_eval(const EvalArgs &a, const LaunchCfg &cfg, cudaStream_t s)
+cudaError_t launch_eval(const EvalArgs &a0, const LaunchCfg &cfg, cudaStream_t s)
 {
-    if (a.lam == 0) return cudaSuccess;
-    if (!a.prims) return cudaErrorInvalidValue;  // k_eval draws the primitive records (apply_mesh)
+    if (a0.lam == 0) return cudaSuccess;
+    if (!a0.prims) return cudaErrorInvalidValue;  // k_eval draws the primitive records (apply_mesh)
+    EvalArgs a = a0;
+    a.qcap = eval_queue_cap(a.ch, a.cam, cfg.threads);
+    const int cluster = eval_cluster(cfg, a.lam);
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(cfg.cluster, a.lam, 1);
+    lc.gridDim = dim3(cluster, a.lam, 1);
     lc.blockDim = dim3(cfg.threads, 1, 1);
     lc.dynamicSmemBytes = cfg.smem;
     lc.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cfg.cluster;
+    attr[0].val.clusterDim.x = cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     // fused generations follow each other: overlap the next one's launch with
@@ -768,7 +873,7 @@ cudaError_t launch_eval(const EvalArgs &a, const LaunchCfg &cfg, cudaStream_t s)
     attr[1].val.programmaticStreamSerializationAllowed = a.cma_st ? 1 : 0;
     lc.attrs = attr;
     lc.numAttrs = 2;
-    return cudaLaunchKernelEx(&lc, k_eval, a);
+    return cfg.threads > 256 ? cudaLaunchKernelEx(&lc, k_eval_wide, a) : cudaLaunchKernelEx(&lc, k_eval, a);
 }
 
 // ----------------------------------------------------------------------------

@@ -201,6 +201,29 @@ def test_bimanual_launch_shapes_agree(api, cluster, threads, raster):
     _check_population(api, sc, P, M, wl.LOSS_ONE_MINUS_IOU, cluster=cluster, threads=threads, raster=raster)
 
 
+@pytest.mark.parametrize("W,H,n_inst", [(640, 512, 1), (700, 493, 2), (800, 600, 1), (960, 768, 2), (1280, 1024, 1),
+                                        (1280, 1280, 2)])
+def test_chosen_launch_shapes_agree(api, W, H, n_inst):
+    """Images whose bitmap leaves room for four, two or one CTA on an SM (the
+    tracker chooses 256, 512 or 1024 threads) and populations around one wave:
+    the counts and losses of a fixed narrow shape, and of the oracle for one
+    candidate."""
+    sc = wl.make_scene("c1", "c1", K=wl.Intrinsics(1.2 * W, 1.2 * W, W / 2, H / 2, W, H), n_instruments=n_inst)
+    rng = np.random.default_rng(W + H)
+    gt = np.concatenate([wl.sample_state(rng, sc.K) for _ in range(n_inst)])
+    M = random_mask(rng, H, W)
+    P = wl.population_around(rng, gt, 330)
+    auto = api.Tracker(sc, lambda_max=330)
+    fixed = api.Tracker(sc, lambda_max=330, cluster=2, block_threads=128)
+    Mp = auto.pack_mask(torch.from_numpy(M).cuda())
+    Pd = torch.from_numpy(np.ascontiguousarray(P, np.float32)).cuda()
+    want_loss, want = fixed.eval_population(Pd, Mp, counts=True)
+    for lam in (1, 19, 77, 153, 200, 330):
+        loss, counts = auto.eval_population(Pd[:lam], Mp, counts=True)
+        assert torch.equal(counts, want[:lam]) and torch.equal(loss, want_loss[:lam]), lam
+    _check_population(api, sc, P[:1], M)
+
+
 @pytest.mark.parametrize("raster", RASTERS)
 def test_large_triangles_warp_path(api, raster):
     """Near-camera close-up: triangles wider than 32 px go to the warp path."""
