@@ -123,9 +123,10 @@ typedef struct {
     float lambda_app;      /* appearance weight of Eq. render_loss (MSE_APP)     */
     int32_t cull_backfaces;/* 0: union of all faces (default)                    */
     int32_t lambda_max;    /* largest population eval_population will accept     */
-    int32_t cluster;       /* CTAs per candidate, 1..8 (0 = auto)                */
+    int32_t cluster;       /* CTAs per candidate, 1..8 (0 = by mesh and population) */
     int32_t block_threads; /* threads per CTA: multiple of 32, >= 32 per instrument,
-                              <= 256 (0 = auto)                                  */
+                              <= 256 (0 = 256, or 512 or 1024 where the image's
+                              bitmap leaves room for few CTAs on an SM)          */
     int32_t raster;        /* TRK_RASTER_* (0 = auto)                            */
 } trk_config;
 
@@ -397,7 +398,9 @@ typedef struct trk_batch trk_batch;
  * optimisers[i] (created on trackers[i]) for its populations; otherwise lam[i]
  * gives its population size.  Trackers may be shared between instances (the
  * batch owns its scratch).  cluster (CTAs per candidate, 1..8) and threads
- * (per CTA, multiple of 32, <= 256) may be 0 for the default (8, 256).
+ * (per CTA, multiple of 32, <= 256) may be 0 for the default (8, 256); with 256
+ * the groups of images whose bitmaps leave room for few CTAs on an SM take 512
+ * or 1024.
  * Synchronous (allocates and uploads the batch's tables). */
 trk_status batch_create(trk_tracker *const *trackers, trk_cmaes *const *optimisers, const int32_t *lam, int32_t n,
                         int32_t cluster, int32_t threads, trk_batch **out);

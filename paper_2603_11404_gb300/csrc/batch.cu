@@ -102,7 +102,7 @@ static trk_status batch_configure(trk_batch *b, int cluster, int threads)
     size_t smem = 0;
     for (int i = 0; i < b->n; ++i) {
         max_inst = std::max(max_inst, b->tr[i]->ch.n_inst);
-        smem = std::max(smem, eval_smem_bytes(b->hdescs[i], 256));
+        smem = std::max(smem, eval_smem_bytes(b->hdescs[i], 256, kBatchReserve));
     }
     if (threads <= 0) threads = 256;
     if (threads > 256 || threads % 32 || threads < 32 * max_inst) return bfail(TRK_EINVAL, "batch threads");
@@ -126,7 +126,7 @@ static trk_status batch_configure(trk_batch *b, int cluster, int threads)
                 for (int i : g.insts) g.lc.smem = std::max(g.lc.smem, eval_smem_bytes(b->hdescs[i], wide));
             }
         }
-        cudaError_t e = prepare_eval_batch(g.lc.smem, cluster, g.lc.threads, &maxc);
+        cudaError_t e = prepare_eval_batch(g.lc.smem, cluster, g.lc.threads, false, &maxc);
         if (e != cudaSuccess) return bfail(TRK_ECUDA, cudaGetErrorString(e));
         if (maxc <= 0) return bfail(TRK_EINVAL, "launch shape does not fit on the device");
         g.n_clusters = std::min(maxc, g.n_items);
@@ -243,7 +243,7 @@ trk_status batch_create(trk_tracker *const *trackers, trk_cmaes *const *optimise
         set_last_error(cudaGetErrorString(e));
         return TRK_ECUDA;
     }
-    auto per_sm = [&](int i) { return (long long)sm_smem / (long long)(eval_smem_bytes(b->hdescs[i], 256) + 4096); };
+    auto per_sm = [&](int i) { return (long long)sm_smem / (long long)(eval_smem_bytes(b->hdescs[i], 256, kBatchReserve) + 4096); };
     auto cost = [&](int i) { return (long long)(b->tr[i]->V + b->tr[i]->T) * b->tr[i]->ch.n_inst; };
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
@@ -261,7 +261,7 @@ trk_status batch_create(trk_tracker *const *trackers, trk_cmaes *const *optimise
         }
         trk_batch::Group &g = b->groups.back();
         g.n_items += b->lam[i];
-        g.smem = std::max(g.smem, eval_smem_bytes(b->hdescs[i], 256));
+        g.smem = std::max(g.smem, eval_smem_bytes(b->hdescs[i], 256, kBatchReserve));
         g.insts.push_back(i);
         for (int c = 0; c < b->lam[i]; ++c) items.push_back(make_int2(i, c));
     }

@@ -197,10 +197,12 @@ size_t tell_smem_bytes();
 cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *masks_dev, const int2 *items_dev,
                               int n_items, unsigned *next_item_dev, const LaunchCfg &cfg, int n_clusters,
                               cudaStream_t s, const int *tell_last_dev = nullptr);
-cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_clusters);
+cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, bool tell, int *max_clusters);
 cudaError_t launch_pack_mask(const uint8_t *mask, uint32_t *packed, int W, int H, int Wq, cudaStream_t s);
-size_t eval_smem_bytes(const EvalArgs &a, int threads);
-int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads);
+// Static and reserved shared memory of a CTA, as the shapes reckon with it (k_eval; k_eval_batch)
+constexpr size_t kEvalReserve = 2048, kBatchReserve = 3584;
+size_t eval_smem_bytes(const EvalArgs &a, int threads, size_t reserve = kEvalReserve);
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads, size_t reserve = kEvalReserve);
 int eval_wide_threads(const ChainDev &ch, const CamDev &cam);
 cudaError_t prepare_eval(size_t smem, int threads);
 cudaError_t eval_cluster_fit(LaunchCfg &cfg);
@@ -276,7 +278,7 @@ inline void apply_mesh(trk::EvalArgs &a, const trk_tracker *t)
     a.prims = t->prims;
     a.P = t->P;
     a.closed = t->closed ? 1 : 0;
-    a.qcap = trk::eval_queue_cap(t->ch, t->cam, 256);
+    a.qcap = trk::eval_queue_cap(t->ch, t->cam, 256, trk::kBatchReserve);
 }
 
 // The tracker's keypoint term into a launch's arguments.

@@ -14,13 +14,13 @@
 //            primitive records (edge-sharing triangle pairs, drawn as convex
 //            quadrilaterals where the projected corners allow, else as their
 //            triangles) from a counter in CTA 0's shared memory until none
-//            are left: integer setup (orientation, top-left bias, bbox), then
-//            small primitives are rasterised by one thread each with int32
-//            incremental edge functions; larger ones are deferred and, after
-//            a second cluster barrier, drawn by the warps of the whole
-//            cluster with int64 edge functions and __ballot_sync coverage
-//            words.  Coverage is OR-ed into the CTA's own full-image bitmap
-//            in shared memory.
+//            are left.  Primitives with a pixel centre in their box (on a
+//            closed mesh the front faces alone) enter the warp's queue, and a
+//            full queue is drawn a row of pixels per lane with int32 edge
+//            functions; larger ones are deferred and, after a second cluster
+//            barrier, drawn by the warps of the whole cluster, a row per lane
+//            from its edges' crossings.  Coverage is OR-ed into the CTA's own
+//            full-image bitmap in shared memory.
 //   phase 3  after a further cluster barrier CTA r ORs band r of all the
 //            cluster's bitmaps through distributed shared memory, ANDs with
 //            the observed mask, popcounts, and the cluster's counts meet in
@@ -614,6 +614,9 @@ __global__ void __launch_bounds__(256, 4) k_eval_checked(EvalArgs a)
 // rewrites between ticks (read with ld.cv, never from a cached line), and the
 // cluster that draws the launch's last ticket leaves the queue counter at zero
 // for the next tick.  Without kTell the updates are a separate launch.
+// Four CTAs to an SM with the updates, at 64 registers: eight streams at 640x512
+// take 7.45 ms for 32 frames, with three 7.90; a batch's frames of one CTA per
+// candidate are no faster with four (7.3 against 6.8 ms).
 template <bool kTell, bool kWide>
 __device__ __forceinline__ void eval_batch_body(const EvalArgs *descs, const uint32_t *const *masks, const int2 *items,
                                                 int n_items, unsigned *next_item, const int *tell_last, int wide_qcap)
@@ -669,9 +672,9 @@ __device__ __forceinline__ void eval_batch_body(const EvalArgs *descs, const uin
 }
 
 template <bool kTell>
-__global__ void __launch_bounds__(256, 3) k_eval_batch(const EvalArgs *descs, const uint32_t *const *masks,
-                                                       const int2 *items, int n_items, unsigned *next_item,
-                                                       const int *tell_last)
+__global__ void __launch_bounds__(256, kTell ? 4 : 3)
+    k_eval_batch(const EvalArgs *descs, const uint32_t *const *masks, const int2 *items, int n_items,
+                 unsigned *next_item, const int *tell_last)
 {
     eval_batch_body<kTell, false>(descs, masks, items, n_items, next_item, tell_last, 0);
 }
@@ -709,11 +712,13 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
                                               next_item_dev, tell_last_dev);
 }
 
-cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_clusters)
+cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, bool tell, int *max_clusters)
 {
     const bool wide = threads > 256;
-    cudaError_t e = ensure_smem_attr(wide ? (const void *)k_eval_batch_wide : (const void *)k_eval_batch<false>, smem);
-    if (e == cudaSuccess && !wide) e = ensure_smem_attr((const void *)k_eval_batch<true>, smem);
+    const cudaError_t e = ensure_smem_attr(wide   ? (const void *)k_eval_batch_wide
+                                           : tell ? (const void *)k_eval_batch<true>
+                                                  : (const void *)k_eval_batch<false>,
+                                           smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cluster, 1, 1);
@@ -726,14 +731,9 @@ cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, int *max_c
     attr[0].val.clusterDim.z = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    if (wide) return cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch_wide, &lc);
-    // both forms (with and without the fused updates) must fit the shape
-    int with_tell = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch<false>, &lc)) != cudaSuccess ||
-        (e = cudaOccupancyMaxActiveClusters(&with_tell, k_eval_batch<true>, &lc)) != cudaSuccess)
-        return e;
-    *max_clusters = std::min(*max_clusters, with_tell);
-    return cudaSuccess;
+    return wide   ? cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch_wide, &lc)
+           : tell ? cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch<true>, &lc)
+                  : cudaOccupancyMaxActiveClusters(max_clusters, k_eval_batch<false>, &lc);
 }
 
 size_t tell_smem_bytes() { return sizeof(TellSmem); }
@@ -746,16 +746,17 @@ static size_t eval_rest_bytes(const ChainDev &ch, const CamDev &cam)
            kAccWords * 4;
 }
 
-size_t eval_smem_bytes(const EvalArgs &a, int threads)
+size_t eval_smem_bytes(const EvalArgs &a, int threads, size_t reserve)
 {
-    return front_smem_bytes(a.ch.n_inst, eval_queue_cap(a.ch, a.cam, threads), threads) + eval_rest_bytes(a.ch, a.cam);
+    return front_smem_bytes(a.ch.n_inst, eval_queue_cap(a.ch, a.cam, threads, reserve), threads) +
+           eval_rest_bytes(a.ch, a.cam);
 }
 
 // CTAs of one shape that an SM holds: 1024 threads at the kernel's 64 registers,
 // 228 KB of shared memory (a KB per CTA is reserved, and a little is static).
-static int eval_ctas_per_sm(const ChainDev &ch, const CamDev &cam, int threads, int qcap)
+static int eval_ctas_per_sm(const ChainDev &ch, const CamDev &cam, int threads, int qcap, size_t reserve)
 {
-    const size_t smem = front_smem_bytes(ch.n_inst, qcap, threads) + eval_rest_bytes(ch, cam) + 2048;
+    const size_t smem = front_smem_bytes(ch.n_inst, qcap, threads) + eval_rest_bytes(ch, cam) + reserve;
     return (int)std::min<size_t>(1024 / threads, 228 * 1024 / smem);
 }
 
@@ -763,10 +764,12 @@ static int eval_ctas_per_sm(const ChainDev &ch, const CamDev &cam, int threads, 
 // as leave an SM as many CTAs: at 700x493 a full queue would cost it the fourth,
 // and with it a population of 64 the single wave of its clusters (51.6 us, with
 // 24 entries 37.7).  8 where the image's bitmap leaves no more.
-int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads)
+int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads, size_t reserve)
 {
     int cap = 32;
-    while (cap > 16 && eval_ctas_per_sm(ch, cam, threads, cap) < eval_ctas_per_sm(ch, cam, threads, 16)) cap -= 4;
+    while (cap > 16 &&
+           eval_ctas_per_sm(ch, cam, threads, cap, reserve) < eval_ctas_per_sm(ch, cam, threads, 16, reserve))
+        cap -= 4;
     return front_smem_bytes(ch.n_inst, cap, threads) + eval_rest_bytes(ch, cam) <= 227 * 1024 ? cap : 8;
 }
 
@@ -778,7 +781,7 @@ int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads)
 int eval_wide_threads(const ChainDev &ch, const CamDev &cam)
 {
     for (int n = 4; n; n /= 2)
-        if (eval_ctas_per_sm(ch, cam, 1024 / n, 16) == n) return 1024 / n;
+        if (eval_ctas_per_sm(ch, cam, 1024 / n, 16, kEvalReserve) == n) return 1024 / n;
     return 256;
 }
 

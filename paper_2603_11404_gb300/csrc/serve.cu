@@ -200,7 +200,7 @@ trk_status reconfigure(trk_server *v)
     int max_inst = 1;
     for (size_t i = 0; i < v->cs.size(); ++i)
         if (v->cs[i].open) {
-            smem = std::max(smem, std::max(eval_smem_bytes(v->hdescs[i], 256), tell_smem_bytes()));
+            smem = std::max(smem, std::max(eval_smem_bytes(v->hdescs[i], 256, kBatchReserve), tell_smem_bytes()));
             max_inst = std::max(max_inst, v->cs[i].es->t->ch.n_inst);
             // single-frame ticks launch the tracker's fused kernel on this device
             const trk_tracker *t = v->cs[i].es->t;
@@ -209,7 +209,7 @@ trk_status reconfigure(trk_server *v)
         }
     if (v->lc.threads < 32 * max_inst) return sfail(TRK_EINVAL, "threads too few for two instruments");
     int maxc = 0, maxw = 0;
-    SCU(prepare_eval_batch(smem, v->lc.cluster, v->lc.threads, &maxc), "server launch shape");
+    SCU(prepare_eval_batch(smem, v->lc.cluster, v->lc.threads, true, &maxc), "server launch shape");
     if (maxc <= 0) return sfail(TRK_EINVAL, "launch shape does not fit on the device");
     v->lc.smem = smem;
     v->max_clusters = maxc;
@@ -218,7 +218,7 @@ trk_status reconfigure(trk_server *v)
     // more CTAs per candidate shorten
     for (int c = 0; c <= 8; ++c) v->max_clusters_by_size[c] = 0;
     for (int c = v->lc.cluster + 1; c <= 8; ++c) {
-        SCU(prepare_eval_batch(smem, c, v->lc.threads, &maxw), "server wide launch shape");
+        SCU(prepare_eval_batch(smem, c, v->lc.threads, true, &maxw), "server wide launch shape");
         v->max_clusters_by_size[c] = maxw;
     }
     return TRK_OK;
