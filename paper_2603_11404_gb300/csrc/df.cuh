@@ -122,10 +122,17 @@ struct dfl2 {
 };
 
 // sin and cos of a double-float angle (|x| up to ~1e4 keeps the reduction
-// exact).  Kept out of line and with rolled loops: it is called from several
-// places once per candidate, so compact code matters more than a few cycles.
-static __device__ __noinline__ dfl2 df_sincos(dfl x)
+// exact) for the angles of lanes 0..15, called by a whole warp: lane l evaluates
+// the sine's polynomial for angle l, lane 16 + l the cosine's, and both lanes
+// get the pair.  One polynomial per lane is half of the arithmetic, which a warp
+// that composes frames by itself waits for.  Kept out of line: it is called from
+// several places once per candidate.
+static __device__ __noinline__ dfl2 df_sincos16(dfl x)
 {
+    const int lane = threadIdx.x & 31;
+    const bool cosine = lane >= 16;
+    x.hi = __shfl_sync(0xffffffffu, x.hi, lane & 15);
+    x.lo = __shfl_sync(0xffffffffu, x.lo, lane & 15);
     // pi/2 = P1 + P2 with P1 = 201/128 (8 significant bits) and P2 a double-float
     const float P1 = 1.5703125f;
     const dfl P2 = DFL_CONST(1.5707963267948966 - 1.5703125);
@@ -136,18 +143,17 @@ static __device__ __noinline__ dfl2 df_sincos(dfl x)
     // sin r = r * S(u), S(u) = sum_{j=0..8} s_j u^j;  cos r = C(u) = sum_{j=0..9} c_j u^j,
     // u = r^2, evaluated by Estrin's scheme (independent pairs, then powers
     // u^2, u^4, u^8) to keep the dependent chain short
+    auto pick = [&](dfl c, dfl s) { return dfl{cosine ? c.hi : s.hi, cosine ? c.lo : s.lo}; };
     const dfl u2 = df_mul(u, u), u4 = df_mul(u2, u2), u8 = df_mul(u4, u4);
-    dfl s01 = df_fma(TS1, u, TS0), s23 = df_fma(TS3, u, TS2);
-    dfl s45 = df_fma(TS5, u, TS4), s67 = df_fma(TS7, u, TS6);
-    dfl c01 = df_fma(TC1, u, TC0), c23 = df_fma(TC3, u, TC2);
-    dfl c45 = df_fma(TC5, u, TC4), c67 = df_fma(TC7, u, TC6), c89 = df_fma(TC9, u, TC8);
-    dfl s03 = df_fma(s23, u2, s01), s47 = df_fma(s67, u2, s45);
-    dfl c03 = df_fma(c23, u2, c01), c47 = df_fma(c67, u2, c45);
-    dfl ps = df_fma(TS8, u8, df_fma(s47, u4, s03));
-    dfl pc = df_fma(c89, u8, df_fma(c47, u4, c03));
-    dfl sr = df_mul(ps, r);
-    dfl cr = pc;
-    int q = ((int)n) & 3;
+    const dfl e01 = df_fma(pick(TC1, TS1), u, TC0), e23 = df_fma(pick(TC3, TS3), u, pick(TC2, TS2));
+    const dfl e45 = df_fma(pick(TC5, TS5), u, pick(TC4, TS4)), e67 = df_fma(pick(TC7, TS7), u, pick(TC6, TS6));
+    const dfl e89 = pick(df_fma(TC9, u, TC8), TS8);
+    const dfl e03 = df_fma(e23, u2, e01), e47 = df_fma(e67, u2, e45);
+    const dfl p = df_fma(e89, u8, df_fma(e47, u4, e03));
+    const dfl v = pick(p, df_mul(p, r));
+    const dfl sr = {__shfl_sync(0xffffffffu, v.hi, lane & 15), __shfl_sync(0xffffffffu, v.lo, lane & 15)};
+    const dfl cr = {__shfl_sync(0xffffffffu, v.hi, lane | 16), __shfl_sync(0xffffffffu, v.lo, lane | 16)};
+    const int q = ((int)n) & 3;
     dfl ss = (q & 1) ? cr : sr, cc = (q & 1) ? sr : cr;
     if (q == 1 || q == 2) cc = df_neg(cc);  // cos: +c, -s, -c, +s
     if (q >= 2) ss = df_neg(ss);            // sin: +s, +c, -s, -c

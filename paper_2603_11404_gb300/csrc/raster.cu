@@ -388,8 +388,9 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
     __shared__ float2 s_z[kMaxD];
     __shared__ int s_last;
 
+    const bool two_warps = nwarp > 2 * nI;  // an instrument's frames are composed by two warps
     {  // the warps that do not compose frames clear the bitmap (16-byte stores)
-        const int c0 = nwarp > nI ? 32 * nI : 0;
+        const int c0 = two_warps ? 64 * nI : nwarp > nI ? 32 * nI : 0;
         uint4 *bm4 = reinterpret_cast<uint4 *>(bm);
         for (int w = tid - c0; w >= 0 && w < (nwords + 3) >> 2; w += nthr - c0) bm4[w] = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -412,9 +413,15 @@ __device__ __forceinline__ void eval_candidate(const EvalArgs &a, int c, const u
             __syncthreads();
             par = s_par;
         }
-        if (warp < nI)
+        if (two_warps) {
+            if (warp < nI) compose_joints(a.ch, par + 9 * warp, scr + warp * kComposeScratch, lane);
+            else if (warp < 2 * nI) compose_pose(a.ch, a.cam, par + 9 * (warp - nI), scr + (warp - nI) * kComposeScratch, lane);
+            __syncthreads();
+            if (warp < nI) compose_chain(a.ch, sM + warp * nF * 24, scr + warp * kComposeScratch, lane);
+        } else if (warp < nI) {
             compose_frames_warp(a.ch, a.cam, par + 9 * warp, sM + warp * nF * 24, scr + warp * kComposeScratch,
                                 lane);
+        }
         if (rank == 0 && warp == nwarp - 1) check_state_finite(par, a.d, a.err, lane);
     }
     __syncthreads();

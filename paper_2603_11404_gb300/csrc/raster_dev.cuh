@@ -35,55 +35,66 @@ __device__ __forceinline__ dfl rot_entry(int axis, dfl s, dfl c, int i, int j)
     return neg ? df_neg(s) : s;
 }
 
-// Projective rows of every frame for one instrument state, computed by one
-// warp in double-float: rows (fx M0, fy M1, M2) of M = T_r^c T_f(q) with
+// Projective rows of every frame for one instrument state, in double-float, by
+// one warp or two (compose_joints and compose_pose side by side, a block barrier,
+// compose_chain): rows (fx M0, fy M1, M2) of M = T_r^c T_f(q) with
 // T_f = T_parent * [Rot(axis_f, coef_f q_joint) | offset_f] and q from the
 // inverse cosine map q = lb + (ub-lb)/2 (1 - cos(pi (qh-lb)/(ub-lb))),
 // written as hi/lo float pairs (24 floats per frame).  The pose rotation is
 // axis-angle, R = cos t I + sin t [k]x + (1 - cos t) k k^T with t = |r|,
 // k = r / t (I + [r]x when t < 1e-8), or look-at Ry(gamma) Rx(alpha) Rz(beta)
 // (Sec. III-A.3).  The lanes run the same code on different data: one
-// sine/cosine evaluation gives the three joint maps and the pose angles,
-// a second one the joint rotations, then the chain products, level by level
-// (frames at the same distance from the root in parallel).  The chain's root
-// starts from G = diag(fx, fy, 1) [R | t], so each product down the chain
+// sine/cosine evaluation gives the three joint maps, a second one the joint
+// rotations, a third one the pose, then the chain products, level by level
+// (frames at the same distance from the root in parallel).  All of it is latency
+// that the CTA waits for: 9.1k cycles with one warp and sine and cosine on every
+// lane, 6.8k with two warps and a polynomial per lane (640x512, 64 candidates:
+// 34.1 -> 32.9 us).  The chain's root starts from G = diag(fx, fy, 1) [R | t], so each product down the chain
 // yields the frame's scaled projective rows directly.
 // scr: kComposeScratch float2 (a multiple of two, so what follows stays
 // 16-byte aligned).
 constexpr int kComposeScratch = 4 + 12 + kMaxFrames * 9 + kMaxFrames * 12;
 
-static __device__ void compose_frames_warp(const ChainDev &ch, const CamDev &cam, const float *st, float *out,
-                                    float2 *scr, int lane)
+// The joint rotations (Js of the scratch): lanes 0-2 the joint maps, then lane f
+// frame f's rotation.
+static __device__ void compose_joints(const ChainDev &ch, const float *st, float2 *scr, int lane)
 {
-    float2 *qs = scr, *G = scr + 4, *Js = scr + 16, *Ts = scr + 16 + kMaxFrames * 9;
+    float2 *qs = scr, *Js = scr + 16;
     const int nF = ch.n_frames;
-    const bool lookat = ch.rot_param == TRK_ROT_LOOKAT;
-    const dfl r0 = df_from(st[0]), r1 = df_from(st[1]), r2 = df_from(st[2]);
-    const dfl t = lookat ? df_from(0.0f) : df_sqrt(dot3(r0, r0, r1, r1, r2, r2));
-    // step 1: lanes 0-2 the joint maps' angles, lane 3 the pose angle t (or
-    // the look-at angles gamma, alpha, beta on lanes 3-5)
     dfl arg = df_from(0.0f);
-    if (lane < 3)
-        arg = df_mul(df_sub(df_from(st[6 + lane]), dfc(ch.lb_df[lane])), dfc(ch.pi_over_range_df[lane]));
-    else if (lane == 3)
-        arg = lookat ? r2 : t;
-    else if (lane == 4 && lookat)
-        arg = r0;
-    else if (lane == 5 && lookat)
-        arg = r1;
-    const dfl2 sc = df_sincos(arg);
+    if (lane < 3) arg = df_mul(df_sub(df_from(st[6 + lane]), dfc(ch.lb_df[lane])), dfc(ch.pi_over_range_df[lane]));
+    const dfl2 sc = df_sincos16(arg);
     if (lane < 3) {
         const dfl q = df_fma(dfc(ch.half_range_df[lane]), df_sub(df_from(1.0f), sc.c), dfc(ch.lb_df[lane]));
         qs[lane] = make_float2(q.hi, q.lo);
-    } else if (lane < 6) {  // pose sines and cosines, parked in the chain scratch
-        Ts[2 * (lane - 3)] = make_float2(sc.s.hi, sc.s.lo);
-        Ts[2 * (lane - 3) + 1] = make_float2(sc.c.hi, sc.c.lo);
     }
     __syncwarp();
-    // step 2: joint rotations (lanes < nF) and the pose rotation (lanes 0-8)
     dfl ang = df_from(0.0f);
     if (lane < nF) ang = df_mul(dfc(ch.coef_df[lane]), dfc(qs[ch.joint[lane]]));
-    const dfl2 fsc = df_sincos(ang);
+    const dfl2 fsc = df_sincos16(ang);
+    if (lane < nF) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const dfl v = rot_entry(ch.axis[lane], fsc.s, fsc.c, e / 3, e % 3);
+            Js[9 * lane + e] = make_float2(v.hi, v.lo);
+        }
+    }
+}
+
+// G of the scratch, from the pose angle t = |r| (lane 0) or the look-at angles
+// gamma, alpha, beta (lanes 0-2); lanes 0-8 hold the rotation's entries.
+static __device__ void compose_pose(const ChainDev &ch, const CamDev &cam, const float *st, float2 *scr, int lane)
+{
+    float2 *G = scr + 4, *Ts = scr + 16 + kMaxFrames * 9;
+    const bool lookat = ch.rot_param == TRK_ROT_LOOKAT;
+    const dfl r0 = df_from(st[0]), r1 = df_from(st[1]), r2 = df_from(st[2]);
+    const dfl t = lookat ? df_from(0.0f) : df_sqrt(dot3(r0, r0, r1, r1, r2, r2));
+    const dfl2 sc = df_sincos16(lookat ? (lane == 0 ? r2 : lane == 1 ? r0 : r1) : t);
+    if (lane < 3) {  // sines and cosines, parked in the chain scratch
+        Ts[2 * lane] = make_float2(sc.s.hi, sc.s.lo);
+        Ts[2 * lane + 1] = make_float2(sc.c.hi, sc.c.lo);
+    }
+    __syncwarp();
     dfl Rv = df_from(0.0f);
     if (lane < 9) {
         const int i = lane / 3, j = lane - 3 * (lane / 3);
@@ -121,13 +132,6 @@ static __device__ void compose_frames_warp(const ChainDev &ch, const CamDev &cam
             }
         }
     }
-    if (lane < nF) {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const dfl v = rot_entry(ch.axis[lane], fsc.s, fsc.c, e / 3, e % 3);
-            Js[9 * lane + e] = make_float2(v.hi, v.lo);
-        }
-    }
     // G = diag(fx, fy, 1) [R | t], row-major 3 x 4: lanes 0-8 the rotation
     // entries, lanes 9-11 the translation
     if (lane < 12) {
@@ -137,7 +141,13 @@ static __device__ void compose_frames_warp(const ChainDev &ch, const CamDev &cam
         if (i == 1) g = df_mul(g, dfc(cam.fy_df));
         G[lane < 9 ? 4 * i + (lane - 3 * i) : 4 * i + 3] = make_float2(g.hi, g.lo);
     }
-    __syncwarp();
+}
+
+// The chain from G and the joint rotations to the frames' scaled rows.
+static __device__ void compose_chain(const ChainDev &ch, float *out, float2 *scr, int lane)
+{
+    float2 *G = scr + 4, *Js = scr + 16, *Ts = scr + 16 + kMaxFrames * 9;
+    const int nF = ch.n_frames;
     // the chain, level by level (a frame's level is its distance from the root):
     // the frames of one level are independent, two at a time (12 lanes each,
     // lane = 4 i + j within a frame)
@@ -174,6 +184,16 @@ static __device__ void compose_frames_warp(const ChainDev &ch, const CamDev &cam
         out[24 * f + 12 + r] = v.y;
     }
     __syncwarp();
+}
+
+// All of it by one warp.
+static __device__ void compose_frames_warp(const ChainDev &ch, const CamDev &cam, const float *st, float *out,
+                                           float2 *scr, int lane)
+{
+    compose_joints(ch, st, scr, lane);
+    compose_pose(ch, cam, st, scr, lane);
+    __syncwarp();
+    compose_chain(ch, out, scr, lane);
 }
 
 // ----------------------------------------------------------------------------
