@@ -356,6 +356,15 @@ def test_fused_generation_equals_separate_calls(api, scene_kw, lam, shape):
     assert sa["sigma"] == sb["sigma"] and sa["best_loss"] == sb["best_loss"] and sa["gen"] == sb["gen"] == 6
 
 
+@pytest.mark.parametrize("W,H,n_inst,lam", [(640, 512, 1, 160), (800, 600, 1, 16), (1280, 1024, 2, 24)])
+def test_fused_generation_in_chosen_shapes(api, W, H, n_inst, lam):
+    """The same in the shapes that the tracker chooses for larger images and
+    populations: the update runs with 256, 512 and 1024 threads."""
+    K = wl.Intrinsics(1.2 * W, 1.2 * W, W / 2, H / 2, W, H)
+    test_fused_generation_equals_separate_calls(api, {"mesh": "c1", "cam": "c1", "K": K, "n_instruments": n_inst}, lam,
+                                                (0, 0))
+
+
 @pytest.mark.parametrize("raster", [1, 2])
 def test_square_roots_after_a_tracked_frame(api, raster):
     """A tracked frame's last update leaves out C^(1/2) and C^(-1/2) (the next
