@@ -540,16 +540,15 @@ class SoftSilhouetteLoss(torch.autograd.Function):
         ctx.tracker, ctx.mask, ctx.sigma, ctx.with_grad = tracker, mask_packed, sigma, with_grad
         if with_grad:
             loss, g = tracker.soft_eval(p, mask_packed, sigma, grad=True)
-            ctx.save_for_backward(g)
+            ctx.save_for_backward(p, g)  # p too: autograd refuses the backward once it was changed in place
             return loss
         ctx.save_for_backward(p)
         return tracker.soft_eval(p, mask_packed, sigma)
 
     @staticmethod
     def backward(ctx, grad_loss):
-        (g,) = ctx.saved_tensors
-        if not ctx.with_grad:
-            _, g = ctx.tracker.soft_eval(g, ctx.mask, ctx.sigma, grad=True)
+        p, *saved = ctx.saved_tensors
+        g = saved[0] if ctx.with_grad else ctx.tracker.soft_eval(p, ctx.mask, ctx.sigma, grad=True)[1]
         return grad_loss.to(g.dtype)[:, None] * g, None, None, None, None
 
 

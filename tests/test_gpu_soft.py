@@ -224,3 +224,13 @@ def test_autograd_forms_give_the_same_bits(api):
             assert torch.equal(torch.autograd.grad(L, y, w)[0], g)
     with torch.no_grad():
         assert torch.equal(api.soft_silhouette_loss(torch.from_numpy(P).cuda().requires_grad_(True), tr, Mp), l0)
+
+
+def test_backward_after_an_inplace_change_is_refused(api):
+    sc, tr, M, Mp, P = _case(api, "c1", "c1", 1, None, 44, 3)
+    x = torch.from_numpy(P).cuda().requires_grad_(True)
+    for L in (api.soft_silhouette_loss(x, tr, Mp), api.SoftSilhouetteLoss.apply(x, tr, Mp)):
+        with torch.no_grad():
+            x += 0.0
+        with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+            L.sum().backward()
