@@ -43,8 +43,8 @@ ALGO_OPS_PER_VERT, ALGO_OPS_PER_TRI, ALGO_OPS_PER_BBOX_PX = 16, 40, 4
 # DRAM bytes (read + write) of one plain k_eval launch at 640x512, lambda = 64, from
 # the committed ncu capture of that kernel, valid for the kernel sources with this
 # digest; reported as null once those sources change.
-KEVAL_TRAFFIC_BYTES = 454144
-KEVAL_TRAFFIC_DIGEST = "a29b4c8e359ac077"
+KEVAL_TRAFFIC_BYTES = 503040
+KEVAL_TRAFFIC_DIGEST = "2b7915b9e5355ba9"
 KERNEL_SOURCES = ("raster.cu", "raster_dev.cuh", "cma_device.cuh", "df.cuh", "internal.cuh")
 
 
@@ -475,7 +475,7 @@ def bench_soft(a, rank, tr, sc, traj, init, packed, flush, n_frames: int = 60, r
     fwd_ms = timed(lambda: tr.soft_eval(P, Mp))
     bwd_ms = timed(lambda: tr.soft_eval(P, Mp, grad=True))
     hard_ms = timed(lambda: tr.eval_population(P, Mp))
-    # roofline of the soft form: the tile kernel evaluates every (pixel,
+    # roofline of the soft form: the method evaluates every (pixel,
     # triangle) pair inside the triangle's window of influence (its pixel box
     # grown by 14 sigma, clipped to the image): about 60 FP32 operations per
     # pair forward and 120 more for the gradient; the pairs are counted from

@@ -207,8 +207,9 @@ static LaunchCfg auto_launch(const trk_tracker *t, const EvalArgs &a, int thread
         lc.cluster = t->cfg.cluster;
     } else {
         // about 2 work items (vertices + triangles) per thread, at most 8 CTAs
-        // (2048 threads) per candidate: the kernel is latency-bound, so more
-        // threads per candidate help until the cluster barriers dominate
+        // per candidate: the kernel is latency-bound, so more threads per
+        // candidate help until the cluster barriers dominate (a large population
+        // takes fewer: eval_cluster_fit)
         long long work = (long long)(t->V + t->T) * t->ch.n_inst;
         long long per_cta = (long long)lc.threads * 2;
         lc.cluster = (int)std::min<long long>(8, std::max<long long>(1, (work + per_cta - 1) / per_cta));
@@ -424,7 +425,7 @@ trk_status tracker_create(const trk_link_mesh *meshes, int32_t n_meshes, const t
         return inval("image or mesh too large for the binned rasteriser");
     }
     // AUTO takes the cluster-bitmap kernel, the faster of the two on every
-    // workload measured (640 x 512, 20k triangles, 64 candidates: 43 us against
+    // workload measured (640 x 512, 20k triangles, 64 candidates: 33 us against
     // 72.5 us), and the binned form only for an image whose bitmap does not fit
     // one CTA's shared memory
     const bool cluster_fits = t->lc.smem <= 227 * 1024;

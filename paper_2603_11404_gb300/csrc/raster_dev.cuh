@@ -49,8 +49,8 @@ __device__ __forceinline__ dfl rot_entry(int axis, dfl s, dfl c, int i, int j)
 // (frames at the same distance from the root in parallel).  All of it is latency
 // that the CTA waits for: 9.1k cycles with one warp and sine and cosine on every
 // lane, 6.8k with two warps and a polynomial per lane (640x512, 64 candidates:
-// 34.1 -> 32.9 us).  The chain's root starts from G = diag(fx, fy, 1) [R | t], so each product down the chain
-// yields the frame's scaled projective rows directly.
+// 34.1 -> 32.9 us).  The chain's root starts from G = diag(fx, fy, 1) [R | t], so
+// each product down the chain yields the frame's scaled projective rows directly.
 // scr: kComposeScratch float2 (a multiple of two, so what follows stays
 // 16-byte aligned).
 constexpr int kComposeScratch = 4 + 12 + kMaxFrames * 9 + kMaxFrames * 12;
