@@ -50,7 +50,14 @@ constexpr int kBlkPx = kBlkW * kBlkH;
 constexpr int kSoftThreads = 256;
 constexpr int kFwdWarps = 4;           // warps that share a heavy block of the forward
 constexpr int kBwdWarps = 4;           // and of the backward
-constexpr int kHeavy = 48;             // groups within reach that make a block heavy
+// Groups within reach that make a block heavy.  On a small image there are too few
+// blocks to hide one warp's long block behind the others: at 12, 8 candidates at
+// 200x150 (loss and gradient, three scenes) take 329, 210 and 206 us, at 48 447, 243
+// and 267; 64 at 101x77 513, 352 and 421 against 661, 471 and 484.  At 640x512 sharing
+// costs more than it gives (64 candidates: 4.66, 2.24 and 2.42 ms against 4.29, 1.66
+// and 1.95).  A rule on the image alone: a candidate's bits do not depend on the
+// population it is called with.
+constexpr int kHeavy = 48, kHeavySmall = 12, kSmallBlocks = 1024;
 // With 1 + Q = prod (1 + exp): Q above kOne makes 1 - S < 2^-25, S is 1 in FP32
 // and the pixel's gradient factor 0, whatever the remaining triangles add.  The
 // forward stops early only at the larger kSaturated, so that a product formed
@@ -262,6 +269,7 @@ struct SoftArgs {
     float fx, fy, cx, cy, z_near, guard, sigma;
     int W, H, Wq;
     int nbx, nby;             // pixel blocks per row and column
+    int heavy;                // groups within reach that make a block heavy
     int ngroups, NTp;         // groups of 32 triangles (over all instruments), triangles padded to whole groups
     int nsup;                 // runs of 32 groups
     const float4 *verts;
@@ -477,9 +485,9 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_list(SoftArgs a)
     const int n0 = in ? cnt[0] : 0, n1 = in && by + 1 < a.nby ? cnt[a.nbx] : 0;
     const int2 v0 = make_int2(c, by << 16 | bx), v1 = make_int2(c, (by + 1) << 16 | bx);
     const int cap = a.lam * a.nby * a.nbx;
-    append(a, n0 > 0, n0 >= kHeavy, v0, kFwdHeavy, a.fwd, cap);
-    append(a, n1 > 0, n1 >= kHeavy, v1, kFwdHeavy, a.fwd, cap);
-    if (a.grad) append(a, n0 + n1 > 0, max(n0, n1) >= kHeavy, v0, kBwdHeavy, a.bwd, a.lam * nby2 * a.nbx);
+    append(a, n0 > 0, n0 >= a.heavy, v0, kFwdHeavy, a.fwd, cap);
+    append(a, n1 > 0, n1 >= a.heavy, v1, kFwdHeavy, a.fwd, cap);
+    if (a.grad) append(a, n0 + n1 > 0, max(n0, n1) >= a.heavy, v0, kBwdHeavy, a.bwd, a.lam * nby2 * a.nbx);
 }
 
 // The entries of a kernel's list: the heavy ones are taken by the whole block
@@ -1230,6 +1238,7 @@ void soft_shape(SoftArgs &a, const trk_tracker *t)
     a.Wq = t->cam.Wq;
     a.nbx = (a.W + kBlkW - 1) / kBlkW;
     a.nby = (a.H + kBlkH - 1) / kBlkH;
+    a.heavy = a.nbx * a.nby <= kSmallBlocks ? kHeavySmall : kHeavy;
     a.ngroups = (int)(((long long)a.nI * a.T + 31) / 32);
     a.NTp = 32 * a.ngroups;
     a.nsup = (a.ngroups + 31) / 32;
