@@ -863,27 +863,38 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
 // With c the closest boundary point, at parameter t of edge k, the signed
 // distance d changes with c by -(p - c) / d, and c follows the edge's ends by
 // 1 - t and t.  The sums are kept in the edges' frames: the parts along the
-// edge (U: only beyond an end) and across it (W), all of them and weighted by
-// the position of c on the edge (from its middle).
+// edge (only beyond an end: U, and V signed by the end) and across it (W, and Wt
+// weighted by the position of c on the edge, from its middle).
+// On the boundary p - c and d vanish together, but d is smooth there and the
+// derivative is their limit, one unit along the edge's normal: within kOnEdge of
+// an edge (in units of the cutoff: 3e-5 sigma, and more than FP32 leaves of the
+// distance of a centre that lies on the edge of a triangle some hundred pixels
+// across) the part across is the weight itself.  Where the derivative jumps (a
+// centre on a corner, or as far from two edges) the first of the nearest edges
+// takes the pixel, as in a comparison without rounding: distances count as equal
+// within kOnEdge, or one part in 2 / (kTie h) for edges of half length h -- the
+// rounding grows with the triangle, and a wider margin moved the gradient of
+// 20k triangles further from 64 bits.
 // The blocks are the forward's, two at a time (half the atomic additions for a
 // few more idle lanes); light and heavy ones as there.  Bound by issue: 1.03
 // and 2.53 ms for the forward's scenes above.  With the groups walking the whole
 // of their windows, one set of additions per triangle, 18-21 % of the lanes
 // had a pair within reach (here 60 %): 5.6 ms for the second scene.
 struct EdgeSums {
-    float U[3], Ut[3], W[3], Wt[3];
+    float U[3], V[3], W[3], Wt[3];
 };
+constexpr float kOnEdge = 1.0f / 524288.0f, kTie = 1.0f / 65536.0f;
 
-__device__ __forceinline__ void bwd_pixel(const BlockEdges &e, int px, float w, EdgeSums &s)
+__device__ __forceinline__ void bwd_pixel(const BlockEdges &e, int px, float w, float tie, EdgeSums &s)
 {
-    float d2[3], b[3], o[3], f[3];
+    float d2[3], b[3], over[3], o[3], f[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float a = fmaf((float)px, e.tx[k], e.a[k]);
         b[k] = fmaf(-(float)px, e.ty[k], e.b[k]);
-        const float over = __saturatef(fabsf(a) - e.h[k]);
-        d2[k] = fmaf(over, over, fmaf(b[k], b[k], 1e-30f));  // never zero
-        o[k] = with_sign(over, a);
+        over[k] = __saturatef(fabsf(a) - e.h[k]);
+        d2[k] = fmaf(over[k], over[k], fmaf(b[k], b[k], 1e-30f));  // never zero
+        o[k] = with_sign(over[k], a);
         f[k] = a - o[k];
     }
     const float m = min3(d2[0], d2[1], d2[2]);
@@ -891,37 +902,37 @@ __device__ __forceinline__ void bwd_pixel(const BlockEdges &e, int px, float w, 
     const float d = m * ir;
     const float sg = rcp_(1.0f + ex2(d * -kExpScale));
     // outside: d = -|p - c|, the sum grows along p - c; inside the other way
-    const float v = w * sg * -ir;
+    const bool on = m <= kOnEdge * kOnEdge;
+    const float q = w * sg;
+    const float v = on ? 0.0f : q * -ir, across = on ? -q : 0.0f;
+    const float nearest = fmaf(m, tie, kOnEdge * kOnEdge);
     // the nearest edge (the first of equal ones) takes it, none beyond the cutoff
     asm("{\n\t"
         ".reg .pred in, p0, r, p1, p2;\n\t"
-        ".reg .f32 u, x;\n\t"
+        ".reg .f32 x;\n\t"
         "setp.gt.f32 in, %12, 0fBF800000;\n\t"
-        "setp.eq.and.f32 p0|r, %13, %16, in;\n\t"
-        "setp.eq.and.f32 p1|p2, %14, %16, r;\n\t"
-        "@p0 mul.f32 u, %17, %18;\n\t"
-        "@p0 mul.f32 x, %17, %19;\n\t"
-        "@p0 add.f32 %0, %0, u;\n\t"
-        "@p0 fma.rn.f32 %3, u, %20, %3;\n\t"
+        "setp.le.and.f32 p0|r, %13, %16, in;\n\t"
+        "setp.le.and.f32 p1|p2, %14, %16, r;\n\t"
+        "@p0 fma.rn.f32 %0, %17, %18, %0;\n\t"
+        "@p0 fma.rn.f32 %3, %17, %19, %3;\n\t"
+        "@p0 fma.rn.f32 x, %17, %20, %15;\n\t"
         "@p0 add.f32 %6, %6, x;\n\t"
-        "@p0 fma.rn.f32 %9, x, %20, %9;\n\t"
-        "@p1 mul.f32 u, %17, %21;\n\t"
-        "@p1 mul.f32 x, %17, %22;\n\t"
-        "@p1 add.f32 %1, %1, u;\n\t"
-        "@p1 fma.rn.f32 %4, u, %23, %4;\n\t"
+        "@p0 fma.rn.f32 %9, x, %21, %9;\n\t"
+        "@p1 fma.rn.f32 %1, %17, %22, %1;\n\t"
+        "@p1 fma.rn.f32 %4, %17, %23, %4;\n\t"
+        "@p1 fma.rn.f32 x, %17, %24, %15;\n\t"
         "@p1 add.f32 %7, %7, x;\n\t"
-        "@p1 fma.rn.f32 %10, x, %23, %10;\n\t"
-        "@p2 mul.f32 u, %17, %24;\n\t"
-        "@p2 mul.f32 x, %17, %25;\n\t"
-        "@p2 add.f32 %2, %2, u;\n\t"
-        "@p2 fma.rn.f32 %5, u, %26, %5;\n\t"
+        "@p1 fma.rn.f32 %10, x, %25, %10;\n\t"
+        "@p2 fma.rn.f32 %2, %17, %26, %2;\n\t"
+        "@p2 fma.rn.f32 %5, %17, %27, %5;\n\t"
+        "@p2 fma.rn.f32 x, %17, %28, %15;\n\t"
         "@p2 add.f32 %8, %8, x;\n\t"
-        "@p2 fma.rn.f32 %11, x, %26, %11;\n\t"
+        "@p2 fma.rn.f32 %11, x, %29, %11;\n\t"
         "}"
-        : "+f"(s.U[0]), "+f"(s.U[1]), "+f"(s.U[2]), "+f"(s.Ut[0]), "+f"(s.Ut[1]), "+f"(s.Ut[2]), "+f"(s.W[0]),
+        : "+f"(s.U[0]), "+f"(s.U[1]), "+f"(s.U[2]), "+f"(s.V[0]), "+f"(s.V[1]), "+f"(s.V[2]), "+f"(s.W[0]),
           "+f"(s.W[1]), "+f"(s.W[2]), "+f"(s.Wt[0]), "+f"(s.Wt[1]), "+f"(s.Wt[2])
-        : "f"(d), "f"(d2[0]), "f"(d2[1]), "f"(d2[2]), "f"(m), "f"(v), "f"(o[0]), "f"(b[0]), "f"(f[0]), "f"(o[1]),
-          "f"(b[1]), "f"(f[1]), "f"(o[2]), "f"(b[2]), "f"(f[2]));
+        : "f"(d), "f"(d2[0]), "f"(d2[1]), "f"(across), "f"(nearest), "f"(v), "f"(o[0]), "f"(over[0]), "f"(b[0]),
+          "f"(f[0]), "f"(o[1]), "f"(over[1]), "f"(b[1]), "f"(f[1]), "f"(o[2]), "f"(over[2]), "f"(b[2]), "f"(f[2]));
 }
 
 constexpr int kBwdRows = 2 * kBlkH;  // the backward takes a block and the one below
@@ -959,13 +970,14 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_soft_bwd(SoftArgs a)
             const TriRec r = load_rec(a, tb + max(t, 0));
             more = col.next(lane, tn);
             BlockEdges e = block_edges(r, t >= 0, w.bx, w.by, unit);
+            const float tie = fmaf(kTie, fmaxf(e.h[0], fmaxf(e.h[1], e.h[2])), 1.0f);
             EdgeSums s{};
             for (int py = 0; py < kBwdRows; ++py) {
                 const unsigned row = (unsigned)(nz >> (kBlkW * py)) & ((1u << kBlkW) - 1u);
                 if (row) {
 #pragma unroll
                     for (int px = 0; px < kBlkW; ++px)
-                        if (row >> px & 1u) bwd_pixel(e, px, sw[kBlkW * py + px], s);
+                        if (row >> px & 1u) bwd_pixel(e, px, sw[kBlkW * py + px], tie, s);
                 }
                 e.down();
             }
@@ -975,8 +987,8 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_soft_bwd(SoftArgs a)
             for (int k = 0; k < 3; ++k) {
                 const int k1 = k == 2 ? 0 : k + 1;
                 const float h = 0.5f * r.L[k] * unit, i2h = h > 0.0f ? 0.5f / h : 0.0f;
-                // the ends' shares: t = (f + h) / 2h, and what is left
-                const float u1 = fmaf(h, s.U[k], s.Ut[k]) * i2h, u0 = s.U[k] - u1;
+                // the ends' shares: t = (f + h) / 2h, and what is left; beyond an end t is 0 or 1
+                const float u1 = 0.5f * (s.U[k] + s.V[k]), u0 = s.U[k] - u1;
                 const float w1 = fmaf(h, s.W[k], s.Wt[k]) * i2h, w0 = s.W[k] - w1;
                 gx[k] += r.tx[k] * u0 - r.ty[k] * w0;
                 gy[k] += r.ty[k] * u0 + r.tx[k] * w0;

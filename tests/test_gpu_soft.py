@@ -234,3 +234,43 @@ def test_backward_after_an_inplace_change_is_refused(api):
             x += 0.0
         with pytest.raises(RuntimeError, match="modified by an inplace operation"):
             L.sum().backward()
+
+
+# Pixel centres exactly on an edge: the signed distance is smooth there and such a
+# pixel carries the largest weight (a = 1/2).  Vertical, horizontal and diagonal
+# edges through centres, in every column of a block; in the last two also corners,
+# and in the last three bisectors, where the first of the nearest edges counts in
+# the kernel and in the oracle.  The bound is that of the tests above.
+@pytest.mark.parametrize("shift", range(8))
+@pytest.mark.parametrize("quad", ["vertical", "horizontal", "triangle", "diagonal", "corners", "square"])
+def test_soft_gradient_with_pixel_centres_on_edges(api, quad, shift):
+    from _helpers import tiny_scene
+    W, H, f = 64, 48, 100.0
+    tris = [[0, 1, 2], [0, 2, 3]]
+    if quad == "vertical":
+        p = [(16, 8.5), (40, 8.5), (40, 32.25), (16, 32.25)]
+    elif quad == "horizontal":
+        p = [(16.5, 8), (40.25, 8), (40.25, 32), (16.5, 32)]
+    elif quad == "diagonal":
+        p = [(15.5, 8.5), (39.5, 8.5), (39.5, 32.5), (15.5, 32.5)]
+    elif quad == "corners":
+        p, tris = [(16, 8), (48, 8), (16, 32)], [[0, 1, 2]]
+    elif quad == "square":
+        p = [(16, 8), (40, 8), (40, 32), (16, 32)]
+    else:
+        p, tris = [(16.25, 8), (47.5, 8), (16.25, 31.5)], [[0, 1, 2]]
+    verts = [[x + shift - W / 2, y - H / 2, 0.0] for x, y in p]  # at z = f a millimetre is a pixel
+    sc = tiny_scene(W, H, f, verts, tris)
+    M = np.zeros((H, W), np.uint8)
+    M[12:36, 19 + shift:46 + shift] = 1
+    tr = api.Tracker(sc, lambda_max=2)
+    Mp = tr.pack_mask(torch.from_numpy(M).cuda())
+    P = np.zeros((2, 9), np.float32)
+    P[:, 5] = f
+    P[1, 3] = 0.3125  # the same off the centres
+    loss, g = tr.soft_eval(torch.from_numpy(P).cuda(), Mp, grad=True)
+    s = wl.default_scales(9)
+    for c in range(2):
+        L, gref = soft.soft_grad(sc, P[c].astype(np.float64), M)
+        assert loss[c].item() == pytest.approx(L, rel=1e-4), c
+        assert _rel(g[c].cpu().numpy(), gref, s) < 1e-3, (c, g[c], gref)
