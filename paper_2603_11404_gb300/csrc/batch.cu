@@ -113,20 +113,25 @@ static trk_status batch_configure(trk_batch *b, int cluster, int threads)
     for (trk_batch::Group &g : b->groups) {
         int maxc = 0;
         g.lc = LaunchCfg{cluster, threads, g.smem, 0};
+        cudaError_t e = cudaSuccess;
         if (threads == 256) {
             // wider CTAs where fewer than four fit an SM (see eval_wide_threads):
             // the shape that every instance of the group allows
             int wide = 1024;
-            for (int i : g.insts) wide = std::min(wide, eval_wide_threads(b->hdescs[i].ch, b->hdescs[i].cam));
+            for (int i : g.insts)
+                wide = std::min(wide, eval_wide_threads(b->hdescs[i].ch, b->hdescs[i].cam, kBatchReserve));
             if (wide > 256) {
-                g.lc.threads = wide;
-                g.lc.qcap = 32;
-                for (int i : g.insts)
-                    g.lc.qcap = std::min(g.lc.qcap, eval_queue_cap(b->hdescs[i].ch, b->hdescs[i].cam, wide));
-                for (int i : g.insts) g.lc.smem = std::max(g.lc.smem, eval_smem_bytes(b->hdescs[i], wide));
+                LaunchCfg w{cluster, wide, g.smem, 32};
+                for (int i : g.insts) {
+                    w.qcap = std::min(w.qcap, eval_queue_cap(b->hdescs[i].ch, b->hdescs[i].cam, wide, kBatchReserve));
+                    w.smem = std::max(w.smem, eval_smem_bytes(b->hdescs[i], wide, kBatchReserve));
+                }
+                e = prepare_eval_batch(w.smem, cluster, wide, false, &maxc);
+                if (e == cudaSuccess && maxc > 0) g.lc = w;
+                else cudaGetLastError();  // 256 threads ask for less
             }
         }
-        cudaError_t e = prepare_eval_batch(g.lc.smem, cluster, g.lc.threads, false, &maxc);
+        if (g.lc.threads == threads) e = prepare_eval_batch(g.lc.smem, cluster, threads, false, &maxc);
         if (e != cudaSuccess) return bfail(TRK_ECUDA, cudaGetErrorString(e));
         if (maxc <= 0) return bfail(TRK_EINVAL, "launch shape does not fit on the device");
         g.n_clusters = std::min(maxc, g.n_items);

@@ -199,11 +199,13 @@ cudaError_t launch_eval_batch(const EvalArgs *descs_dev, const uint32_t *const *
                               cudaStream_t s, const int *tell_last_dev = nullptr);
 cudaError_t prepare_eval_batch(size_t smem, int cluster, int threads, bool tell, int *max_clusters);
 cudaError_t launch_pack_mask(const uint8_t *mask, uint32_t *packed, int W, int H, int Wq, cudaStream_t s);
-// Static and reserved shared memory of a CTA, as the shapes reckon with it (k_eval; k_eval_batch)
-constexpr size_t kEvalReserve = 2048, kBatchReserve = 3584;
+// Shared memory of a CTA beside the dynamic one, as the shapes reckon with it: the
+// kernel's static memory (k_eval and k_eval_wide 736 bytes; the batch kernels 2528,
+// their descriptor) and the KB that the device reserves for each CTA.
+constexpr size_t kEvalReserve = 2048, kBatchReserve = 3552;
 size_t eval_smem_bytes(const EvalArgs &a, int threads, size_t reserve = kEvalReserve);
 int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads, size_t reserve = kEvalReserve);
-int eval_wide_threads(const ChainDev &ch, const CamDev &cam);
+int eval_wide_threads(const ChainDev &ch, const CamDev &cam, size_t reserve = kEvalReserve);
 cudaError_t prepare_eval(size_t smem, int threads);
 cudaError_t eval_cluster_fit(LaunchCfg &cfg);
 void set_last_error(const char *msg);  // the text tracker_last_error() returns

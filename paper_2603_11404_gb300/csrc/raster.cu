@@ -785,10 +785,10 @@ int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads, size_t re
 // two or three, 1024 for one.  Two instruments of 40k triangles, 256 candidates,
 // one CTA each: 1280x1024 742 us with 256 threads, 470 with 512, 383 with 1024;
 // 960x768 410 and 350; 800x600 370 and 302 (320 threads, three to an SM: 352).
-int eval_wide_threads(const ChainDev &ch, const CamDev &cam)
+int eval_wide_threads(const ChainDev &ch, const CamDev &cam, size_t reserve)
 {
     for (int n = 4; n; n /= 2)
-        if (eval_ctas_per_sm(ch, cam, 1024 / n, 16, kEvalReserve) == n) return 1024 / n;
+        if (eval_ctas_per_sm(ch, cam, 1024 / n, 16, reserve) == n) return 1024 / n;
     return 256;
 }
 

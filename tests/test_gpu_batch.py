@@ -175,3 +175,33 @@ def test_batch_deferred_list_overflow(api):
     torch.cuda.synchronize()
     assert torch.equal(counts[0], rc) and torch.equal(losses[0].view(torch.int32), rl.view(torch.int32))
     assert 0.2 * W * H < rc[0, 0].item() < 0.9 * W * H
+
+
+def test_batch_takes_every_large_image(api):
+    """Heights of a 1280-pixel wide image at which the drawing queues of the wide
+    CTAs just fill an SM, the largest image among them, and one size down, where
+    two CTAs share it: each alone in a batch of one and two instruments, equal to
+    the single-tracker call; a tracked frame at the largest."""
+    P = {}
+    for ni, heights in ((1, (600, 1152, 1155, 1161, 1162, 1189, 1193, 1221, 1253, 1258, 1280)),
+                        (2, (597, 1150, 1154, 1158, 1186, 1190, 1218, 1250, 1254, 1279, 1280))):
+        for H in heights:
+            K = wl.Intrinsics(1600.0, 1600.0, 640.0, H / 2, 1280, H)
+            sc = wl.make_scene("800", "c2", n_instruments=ni, K=K)
+            rng = np.random.default_rng(H + ni)
+            if ni not in P:
+                P[ni] = np.concatenate([wl.sample_state(rng, K) for _ in range(ni)])
+            tr = api.Tracker(sc, loss_kind=wl.LOSS_ONE_MINUS_IOU, lambda_max=4)
+            Mp = tr.pack_mask(torch.from_numpy(random_mask(rng, H, 1280)).cuda())
+            p = torch.from_numpy(wl.population_around(rng, P[ni], 4)).cuda()
+            b = api.Batch([tr], lams=[4])
+            for shape in ((8, 256), (1, 256), (2, 128)):
+                b.set_launch(*shape)
+                losses, counts = b.eval([p], [Mp])
+                rl, rc = tr.eval_population(p, Mp, counts=True)
+                assert torch.equal(counts[0], rc) and torch.equal(losses[0].view(torch.int32), rl.view(torch.int32)), H
+    opt = [api.CMAES(tr, 4, P[2], wl.default_scales(18), seed=5, block_diag=True) for _ in range(2)]
+    b = api.Batch([tr], optimisers=opt[:1])
+    for _ in range(2):
+        (pose,) = b.track_frame([Mp], 2)
+        assert torch.equal(pose, opt[1].track_frame(Mp, 2))
