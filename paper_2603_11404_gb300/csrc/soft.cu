@@ -1182,18 +1182,19 @@ using namespace trk;
 
 namespace {
 
-// Scratch of one tracker: one allocation, laid out for `cap` candidates.
+// Scratch of one tracker: one allocation, which every call lays out for itself.
+// It is sized for a gradient whichever kind of call comes first: a gradient on as
+// many candidates then finds its memory (it may be under capture, and a captured
+// loss may still use what growing would free).
 struct SoftScratch {
-    int cap = 0;
-    bool grad = false;         // laid out with the backward's arrays
+    size_t bytes = 0;
     int fwd_grid = 0, bwd_grid = 0;
     void *mem = nullptr;
-    SoftArgs a{};              // the arrays
 };
 
-// A call on more candidates than this takes them in slices: the scratch stays
-// below about two gigabytes (the records and the per-pixel factors of a
-// 640x512, 20k-triangle candidate are about 3.5 MB).
+// A call on more candidates than the scratch holds takes them in slices; it grows
+// to two gigabytes, or one candidate's need (the records and the per-pixel
+// factors of a 640x512, 20k-triangle candidate are about 3.5 MB).
 constexpr size_t kSoftBudget = (size_t)2 << 30;
 
 struct RefineBuf {
@@ -1256,31 +1257,22 @@ void soft_shape(SoftArgs &a, const trk_tracker *t)
     a.nsup = (a.ngroups + 31) / 32;
 }
 
-// The largest slice of a call on lam candidates (at least one).
-int soft_slice(const trk_tracker *t, int lam, bool grad)
+// As many candidates (at least one) as `bytes` hold for this kind of call.
+int soft_fit(SoftArgs &a, int lam, bool grad, size_t bytes)
 {
-    SoftArgs a{};
-    soft_shape(a, t);
-    const size_t per = soft_layout(a, 1, grad, nullptr);
-    return (int)std::max<size_t>(1, std::min<size_t>((size_t)lam, kSoftBudget / std::max<size_t>(per, 1)));
+    return (int)std::max<size_t>(1, std::min<size_t>((size_t)lam, bytes / soft_layout(a, 1, grad, nullptr)));
 }
 
-trk_status soft_scratch(trk_tracker *t, int lam, bool grad, SoftScratch **out)
+trk_status soft_scratch(trk_tracker *t, size_t bytes, SoftScratch **out)
 {
     SoftScratch *s = static_cast<SoftScratch *>(t->soft);
-    if (s && s->cap >= lam && (s->grad || !grad)) {
+    if (s && s->bytes >= bytes) {
         *out = s;
         return TRK_OK;
-    }
-    if (s) {  // grow: keep what either kind of call needs
-        lam = std::max(lam, s->cap);
-        grad |= s->grad;
     }
     soft_free(t);
     s = new SoftScratch();
     t->soft = s;
-    soft_shape(s->a, t);
-    const size_t bytes = soft_layout(s->a, lam, grad, nullptr);
     cudaError_t e;
     int fwd = 0, bwd = 0, sms = 0;
     if ((e = cudaMalloc(&s->mem, bytes)) != cudaSuccess ||
@@ -1290,9 +1282,7 @@ trk_status soft_scratch(trk_tracker *t, int lam, bool grad, SoftScratch **out)
         soft_free(t);
         return soft_fail(e == cudaErrorMemoryAllocation ? TRK_ENOMEM : TRK_ECUDA, cudaGetErrorString(e));
     }
-    soft_layout(s->a, lam, grad, static_cast<char *>(s->mem));
-    s->cap = lam;
-    s->grad = grad;
+    s->bytes = bytes;
     s->fwd_grid = std::max(1, fwd) * sms;
     s->bwd_grid = std::max(1, bwd) * sms;
     *out = s;
@@ -1303,11 +1293,14 @@ trk_status soft_launch(trk_tracker *t, const float *params, int lam, const uint3
                        float *grad, cudaStream_t st)
 {
     if (lam == 0) return TRK_OK;
-    const int slice = soft_slice(t, lam, grad != nullptr);
+    SoftArgs a{};
+    soft_shape(a, t);
+    int slice = soft_fit(a, lam, true, kSoftBudget);
     SoftScratch *s = nullptr;
-    trk_status r = soft_scratch(t, slice, grad != nullptr, &s);
+    trk_status r = soft_scratch(t, soft_layout(a, slice, true, nullptr), &s);
     if (r != TRK_OK) return r;
-    SoftArgs a = s->a;
+    slice = std::max(slice, soft_fit(a, lam, grad != nullptr, s->bytes));  // a loss alone needs less
+    soft_layout(a, slice, grad != nullptr, static_cast<char *>(s->mem));
     a.fx = (float)t->cam.fx;
     a.fy = (float)t->cam.fy;
     a.cx = (float)(t->cam.cx256 / 256.0);

@@ -274,3 +274,51 @@ def test_soft_gradient_with_pixel_centres_on_edges(api, quad, shift):
         L, gref = soft.soft_grad(sc, P[c].astype(np.float64), M)
         assert loss[c].item() == pytest.approx(L, rel=1e-4), c
         assert _rel(g[c].cpu().numpy(), gref, s) < 1e-3, (c, g[c], gref)
+
+
+@pytest.mark.parametrize("first", ["loss", "gradient"])
+def test_soft_scratch_stays_within_its_bound(api, first):
+    """A loss of 1024 candidates and a gradient of eight on one tracker, in either
+    order: the scratch stays below its two gigabytes (a candidate of the largest
+    image holds about 8 MB), and the results are those of a tracker of their own."""
+    sc = wl.make_scene("c1", "c2", K=wl.Intrinsics(1600.0, 1600.0, 640.0, 640.0, 1280, 1280))
+    rng = np.random.default_rng(97)
+    gt = wl.sample_state(rng, sc.K)
+    P = torch.from_numpy(wl.population_around(rng, gt, 1024)).cuda()
+    fresh = api.Tracker(sc, lambda_max=1)
+    Mp = fresh.pack_mask(api.unpack_mask(fresh.render(torch.from_numpy(gt.astype(np.float32)).cuda()), 1280))
+    want = [x.clone() for x in fresh.soft_eval(P[:8].contiguous(), Mp, grad=True)]
+    del fresh
+    tr = api.Tracker(sc, lambda_max=1)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    for kind in ("loss", "gradient") if first == "loss" else ("gradient", "loss"):
+        if kind == "loss":
+            loss = tr.soft_eval(P, Mp)
+        else:
+            got = tr.soft_eval(P[:8].contiguous(), Mp, grad=True)
+    torch.cuda.synchronize()
+    assert free0 - torch.cuda.mem_get_info()[0] < (2 << 30) + (64 << 20)
+    for a, b in zip(got, want):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+    assert torch.equal(loss[:8].view(torch.int32), want[0].view(torch.int32))
+
+
+def test_soft_calls_of_both_kinds_under_capture(api):
+    """After a loss on a population, a gradient on as many candidates can be
+    captured, and a captured loss stays valid after it."""
+    sc, tr, M, Mp, P = _case(api, "c1", "c1", 1, None, 98, 6)
+    Pd = torch.from_numpy(P).cuda()
+    want_l = tr.soft_eval(Pd, Mp)
+    graphs, outs = [], []
+    for grad in (False, True):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            outs.append(tr.soft_eval(Pd, Mp, grad=grad))
+        graphs.append(g)
+    l1, g1 = tr.soft_eval(Pd, Mp, grad=True)
+    for g in graphs + graphs:
+        g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], want_l) and torch.equal(l1, want_l)
+    assert torch.equal(outs[1][0], want_l) and torch.equal(outs[1][1], g1)
