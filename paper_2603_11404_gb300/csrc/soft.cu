@@ -63,6 +63,9 @@ constexpr int kHeavy = 48, kHeavySmall = 12, kSmallBlocks = 1024;
 // forward stops early only at the larger kSaturated, so that a product formed
 // in another order cannot fall below kOne again.
 constexpr float kOne = 3.4e7f, kSaturated = 6.6e7f;
+// A product over no triangle: nothing beside the smallest term (8e-7), and not
+// zero, so that Q fma'd with an infinite product gives infinity, never NaN.
+constexpr float kEmpty = 1e-30f;
 // Gradient sums are accumulated in 64-bit fixed point, exact and so independent
 // of the order of the (atomic) additions: dL/d(u, v) per vertex in units of
 // 2^-36 (|sum| < 2^27: with x_t = softplus(d_t / sigma) >= sigmoid, a pixel adds
@@ -791,12 +794,12 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
         const int j = w.bx * kBlkW + (lane & (kBlkW - 1)), i = w.by * kBlkH + lane / kBlkW;
         const bool on = j < a.W && i < a.H;
         if (w.heavy) {
-            part[warp][lane] = 0.0f;
+            part[warp][lane] = kEmpty;
             __syncthreads();
         }
         float Q[kBlkPx];
 #pragma unroll
-        for (int p = 0; p < kBlkPx; ++p) Q[p] = 1e-30f;  // nothing beside the smallest term (8e-7), and not zero
+        for (int p = 0; p < kBlkPx; ++p) Q[p] = kEmpty;
         Collector<kBlkH> col(a, c, w.bx, w.by, warp, w.heavy ? kFwdWarps : 1, queue[warp]);
         int t, batches = 0;
         bool more = col.next(lane, t);
