@@ -302,7 +302,8 @@ enum { kFwdHeavy, kFwdLight, kBwdHeavy, kBwdLight, kTicket, kFwdExit = kTicket +
 
 // Edge record of a drawable triangle, positively oriented, in image pixels: the
 // corners, the edges' unit directions and lengths, and
-// +1 / -1 for the mesh's corner order / the reverse (0: not drawn).
+// +1 / -1 for the mesh's corner order / the reverse, +2 / -2 when all corners
+// are on the lattice of 1/256 px.
 struct TriRec {
     float x[3], y[3], tx[3], ty[3], L[3], orient;
 };
@@ -384,6 +385,9 @@ __device__ __forceinline__ float4 soft_project(const SoftArgs &a, const float *M
     return o;
 }
 
+// x to the lattice of 1/256 px (|x| < 2^14; coarser beyond).
+__device__ __forceinline__ float rint256(float x) { return __fadd_rn(__fadd_rn(x, 49152.0f), -49152.0f); }
+
 // A warp per group of 32 triangles.  Every lane projects its triangle's three
 // corners itself: cheaper than a pass of its own over the vertices and a gather.
 __global__ void __launch_bounds__(kSoftThreads) k_soft_tris(SoftArgs a)
@@ -428,7 +432,10 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_tris(SoftArgs a)
             a.rec[ti] = make_float4(x[0], y[0], x[1], y[1]);
             a.rec[n + ti] = make_float4(x[2], y[2], tx[0], ty[0]);
             a.rec[2 * n + ti] = make_float4(tx[1], ty[1], tx[2], ty[2]);
-            a.rec[3 * n + ti] = make_float4(L[0], L[1], L[2], A > 0.0f ? 1.0f : -1.0f);
+            bool lattice = true;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) lattice &= rint256(x[k]) == x[k] && rint256(y[k]) == y[k];
+            a.rec[3 * n + ti] = make_float4(L[0], L[1], L[2], (A > 0.0f ? 1.0f : -1.0f) * (lattice ? 2.0f : 1.0f));
             lox = fminf(x[0], fminf(x[1], x[2]));
             hix = fmaxf(x[0], fmaxf(x[1], x[2]));
             loy = fminf(y[0], fminf(y[1], y[2]));
@@ -874,10 +881,12 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
 // distance of a centre that lies on the edge of a triangle some hundred pixels
 // across) the part across is the weight itself.  Where the derivative jumps (a
 // centre on a corner, or as far from two edges) the first of the nearest edges
-// takes the pixel, as in a comparison without rounding: distances count as equal
-// within kOnEdge, or one part in 2 / (kTie h) for edges of half length h -- the
-// rounding grows with the triangle, and a wider margin moved the gradient of
-// 20k triangles further from 64 bits.
+// takes the pixel, as in a comparison without rounding: squared distances count
+// as equal within kOnEdge^2, and for a triangle with all corners on the lattice of
+// 1/256 px, whose bisectors run through pixel centres, within the rounding's part,
+// kTie h for edges of half length h.  Of other triangles the nearest edge counts as
+// FP32 has it: a margin assigned more pixels to the wrong edge than it put right
+// (gradients of 20k triangles 1.0e-6 -> 5.0e-6 from 64 bits at worst).
 // The blocks are the forward's, two at a time (half the atomic additions for a
 // few more idle lanes); light and heavy ones as there.  Bound by issue: 1.03
 // and 2.53 ms for the forward's scenes above.  With the groups walking the whole
@@ -973,7 +982,7 @@ __global__ void __launch_bounds__(32 * kBwdWarps, 5) k_soft_bwd(SoftArgs a)
             const TriRec r = load_rec(a, tb + max(t, 0));
             more = col.next(lane, tn);
             BlockEdges e = block_edges(r, t >= 0, w.bx, w.by, unit);
-            const float tie = fmaf(kTie, fmaxf(e.h[0], fmaxf(e.h[1], e.h[2])), 1.0f);
+            const float tie = fabsf(r.orient) > 1.0f ? fmaf(kTie, fmaxf(e.h[0], fmaxf(e.h[1], e.h[2])), 1.0f) : 1.0f;
             EdgeSums s{};
             for (int py = 0; py < kBwdRows; ++py) {
                 const unsigned row = (unsigned)(nz >> (kBlkW * py)) & ((1u << kBlkW) - 1u);
