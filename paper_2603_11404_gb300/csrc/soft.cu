@@ -76,7 +76,11 @@ constexpr float kEmpty = 1e-30f;
 constexpr float kGvScale = 68719476736.0f;
 constexpr float kRestScale = 4294967296.0f;
 constexpr float kGScale = 16777216.0f;
-constexpr double kLossScale = 4294967296.0;  // the loss, in units of 2^-32
+// The loss in units of 2^-41 (TRK_MAX_PIXELS of them stay below 2^62) and the
+// blocks' remainders in units of 2^-73: an instrument that reaches into the image
+// by its fringe alone has a loss of 1e-6 and less.
+constexpr int kLossBits = 41;
+constexpr float kLossScale = 2199023255552.0f;
 // (a power of two times a float is exact in FP32: no FP64 arithmetic needed)
 __device__ __forceinline__ long long to_fixed(float x, float scale) { return __float2ll_rn(x * scale); }
 
@@ -293,7 +297,7 @@ struct SoftArgs {
     unsigned *rdone;          // [lam] finished blocks of k_soft_reduce
     longlong2 *gv;            // [lam * nI * V]: dL/du, dL/dv in fixed point (units of 2^-36)
     unsigned long long *G;    // [lam * nI * nF * 12][2] fixed point, units of 2^-24 and of 2^-56
-    unsigned long long *lsum; // [lam] loss in fixed point, units of 2^-32
+    unsigned long long *lsum; // [lam][2] loss in fixed point, units of 2^-41 and of 2^-73
     float *loss;              // [lam]
     float *grad;              // [lam * d] or NULL
 };
@@ -366,7 +370,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fk(SoftArgs a)
         }
     }
     __syncthreads();
-    if (b == 0 && tid == 0) a.lsum[c] = (unsigned long long)s_m << 32;
+    if (b == 0 && tid < 2) a.lsum[2 * c + tid] = tid ? 0ull : (unsigned long long)s_m << kLossBits;
 }
 
 // Projection of a mesh vertex: (u - cx, v - cy, Z, flag).  Explicit roundings:
@@ -851,9 +855,12 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
         if (a.grad) a.wp[(((size_t)c * a.nby + w.by) * a.nbx + w.bx) * kBlkPx + lane] = wpx;
         const int m = __popc(__ballot_sync(0xffffffffu, mv));
         for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if (lane == 0)  // squared error minus the mask pixels counted in advance: exact sums, in any order
-            atomicAdd(a.lsum + c, (unsigned long long)__double2ll_rn((double)l * kLossScale) -
-                                      ((unsigned long long)m << 32));
+        if (lane == 0) {  // squared error minus the mask pixels counted in advance: exact sums, in any order
+            const float q = l * kLossScale, h = rintf(q);
+            const long long rest = to_fixed(q - h, kRestScale);
+            atomicAdd(a.lsum + 2 * c, (unsigned long long)__float2ll_rn(h) - ((unsigned long long)m << kLossBits));
+            if (rest) atomicAdd(a.lsum + 2 * c + 1, (unsigned long long)rest);
+        }
     }
     // the last block to run out of work writes the losses
     __syncthreads();
@@ -865,7 +872,8 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
     if (s_it) {
         __threadfence();
         for (int c = tid; c < a.lam; c += blockDim.x)
-            a.loss[c] = (float)((double)(long long)__ldcg(a.lsum + c) * (1.0 / kLossScale));
+            a.loss[c] = (float)(((double)(long long)__ldcg(a.lsum + 2 * c) +
+                                 (double)(long long)__ldcg(a.lsum + 2 * c + 1) * (1.0 / kRestScale)) * (1.0 / kLossScale));
     }
 }
 
@@ -1238,7 +1246,7 @@ size_t soft_layout(SoftArgs &a, int lam, bool grad, char *base)
     take(a.fwd, L * nb);
     take(a.ctl, kCtl);
     take(a.rdone, L);
-    take(a.lsum, L);
+    take(a.lsum, 2 * L);
     take(a.Tf, fr * 12);
     take(a.dT, fr * 9 * 12);
     if (grad) {

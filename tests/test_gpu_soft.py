@@ -322,3 +322,22 @@ def test_soft_calls_of_both_kinds_under_capture(api):
     torch.cuda.synchronize()
     assert torch.equal(outs[0], want_l) and torch.equal(l1, want_l)
     assert torch.equal(outs[1][0], want_l) and torch.equal(outs[1][1], g1)
+
+
+def test_soft_losses_of_the_fringe_keep_their_digits(api):
+    """An instrument outside the image whose fringe reaches into it, no mask: losses
+    from 3 down to 7e-10, within the bound of the tests above (and approx's own 1e-12:
+    corners lie whole pixels away, and a pixel exactly at the cutoff adds 7e-13)."""
+    from _helpers import tiny_scene
+    W, H, f = 64, 48, 100.0
+    verts = [[x - 10.0, y - 10.0, 0.0] for x, y in ((0, 0), (20, 1), (19, 22), (1, 20))]
+    sc = tiny_scene(W, H, f, verts, [[0, 1, 2], [0, 2, 3]])
+    tr = api.Tracker(sc, lambda_max=1)
+    Mp = tr.pack_mask(torch.zeros((H, W), dtype=torch.uint8, device="cuda"))
+    P = np.zeros((8, 9), np.float32)
+    P[:, 5] = f
+    P[:, 3] = [-42.3, -46.0, -48.0, -50.0, -51.0, -52.0, -53.0, -54.0]
+    loss = tr.soft_eval(torch.from_numpy(P).cuda(), Mp).cpu().numpy()
+    for c in range(8):
+        L = soft.soft_loss(sc, P[c].astype(np.float64), np.zeros((H, W)))
+        assert loss[c] == pytest.approx(L, rel=1e-4), c
