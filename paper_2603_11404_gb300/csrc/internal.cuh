@@ -204,6 +204,7 @@ cudaError_t launch_pack_mask(const uint8_t *mask, uint32_t *packed, int W, int H
 // their descriptor) and the KB that the device reserves for each CTA.
 constexpr size_t kEvalReserve = 2048, kBatchReserve = 3552;
 size_t eval_smem_bytes(const EvalArgs &a, int threads, size_t reserve = kEvalReserve);
+size_t eval_checked_smem_bytes(const EvalArgs &a, int threads);
 int eval_queue_cap(const ChainDev &ch, const CamDev &cam, int threads, size_t reserve = kEvalReserve);
 int eval_wide_threads(const ChainDev &ch, const CamDev &cam, size_t reserve = kEvalReserve);
 cudaError_t prepare_eval(size_t smem, int threads);

@@ -155,7 +155,7 @@ trk_status eval_population_noalloc(const float *verts_dev, int32_t n_verts, cons
         long long per_cta = (long long)lc.threads * 2;
         lc.cluster = (int)std::min<long long>(8, std::max<long long>(1, (work + per_cta - 1) / per_cta));
     }
-    lc.smem = eval_smem_bytes(a, 256);
+    lc.smem = eval_checked_smem_bytes(a, lc.threads);
     if (lc.smem > 227 * 1024) return fail(TRK_EINVAL, "image too large for the shared-memory bitmap");
     // the index-checked kernel: the mesh is in the caller's device memory; its
     // dynamic shared-memory limit is a kernel attribute, not an allocation

@@ -759,6 +759,12 @@ size_t eval_smem_bytes(const EvalArgs &a, int threads, size_t reserve)
            eval_rest_bytes(a.ch, a.cam);
 }
 
+// k_eval_checked has no drawing queues (EvalArgs::qcap is 0 there).
+size_t eval_checked_smem_bytes(const EvalArgs &a, int threads)
+{
+    return front_smem_bytes(a.ch.n_inst, a.qcap, threads) + eval_rest_bytes(a.ch, a.cam);
+}
+
 // CTAs of one shape that an SM holds: 1024 threads at the kernel's 64 registers,
 // 228 KB of shared memory (a KB per CTA is reserved, and a little is static).
 static int eval_ctas_per_sm(const ChainDev &ch, const CamDev &cam, int threads, int qcap, size_t reserve)
