@@ -14,7 +14,8 @@ namespace trk {
 constexpr int kMaxFrames = TRK_MAX_FRAMES;
 constexpr int kMaxD = TRK_MAX_D;
 constexpr int kSnapFlag = INT32_MIN;          // snapped x of a flagged vertex
-constexpr int kBigListCap = 1024;              // large triangles deferred per CTA
+constexpr int kBigListCap = 1020;              // large primitives deferred per CTA (with the counters 4128
+                                               // bytes; four more entries would cost the largest images)
 constexpr double kGuardPx = 16384.0;           // |u - cx|, |v - cy| limit (2^14 px)
 
 // Kinematic chain of one instrument in device-friendly form (Sec. III-A.2).

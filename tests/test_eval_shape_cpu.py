@@ -10,7 +10,7 @@ from paper_2603_11404_gb300 import build
 
 KB = 1024
 CTA_LIMIT, SM_LIMIT = 227 * KB, 228 * KB  # static and dynamic memory of a CTA; all of an SM, with a KB per CTA
-SCRATCH, LIST = (16 + 16 * 21) * 8, 1024 * 4  # composition scratch per instrument, deferred list
+SCRATCH = (16 + 16 * 21) * 8  # composition scratch per instrument
 
 
 def constant(name, file):
@@ -41,6 +41,7 @@ def test_reserves_cover_the_static_memory():
         assert b + KB <= r["kBatchReserve" if "k_eval_batch" in name else "kEvalReserve"], name
 
 
+LIST = 4 * constant("kBigListCap", "internal.cuh")  # deferred list
 ACC = 4 * constant("kAccWords", "raster.cu")
 
 

@@ -547,3 +547,29 @@ def test_front_face_rule_and_its_exceptions(api, kind, cull, cluster):
     counts, _, _ = _check_population(api, sc, P, M, cull=cull, cluster=cluster, fk_tol=1e-3)
     if kind == "closed":
         assert (counts[:, 3] > 0).any() and (counts[:, 3] == 0).any() and counts[:, 0].max() > 50
+
+
+def test_image_whose_bitmap_fills_the_shared_memory(api):
+    """29 pixels wide and as tall as one CTA's shared memory holds (56072 rows of a
+    five-frame instrument; 55624 in a batch): accepted to the last word, counts
+    equal to the oracle's, with a vertex behind the camera in the second candidate."""
+    for H, batch in ((56069, False), (56072, False), (55621, True), (55624, True)):
+        K = wl.Intrinsics(200.0, 200.0, 14.5, 60.0, 29, H)
+        sc = wl.make_scene("800", "c1", K=K)
+        rng = np.random.default_rng(H)
+        P = wl.population_around(rng, wl.sample_state(rng, wl.Intrinsics(200.0, 200.0, 80.0, 64.0, 160, 128)), 2)
+        P[1, 5] = 12.0
+        M = np.zeros((H, 29), np.uint8)
+        M[:400] = random_mask(rng, 400, 29)
+        M[-3:] = 1
+        tr = api.Tracker(sc, lambda_max=2)
+        Mp = tr.pack_mask(torch.from_numpy(M).cuda())
+        Pd = torch.from_numpy(P).cuda()
+        loss, counts, snap, _ = tr.eval_population_debug(Pd, Mp)
+        for c in range(2):
+            s, I, m, culled, _ = oracle_counts_from_snapped(sc, snap[c].cpu().numpy(), M)
+            assert tuple(counts[c].tolist()) == (s, I, m, culled), (H, c)
+        if batch:
+            b = api.Batch([tr], lams=[2])
+            lb, cb = b.eval([Pd], [Mp])
+            assert torch.equal(cb[0], counts) and torch.equal(lb[0], loss)
