@@ -530,8 +530,8 @@ class SoftSilhouetteLoss(torch.autograd.Function):
     The gradient kernels need the forward's per-pixel factors, so with
     with_grad the forward call also computes the gradient (9 floats per
     instrument and candidate, saved for the backward) and the backward runs no
-    kernel of its own: one forward pass less, 1.7 instead of 2.2 ms for 64
-    candidates at 640x512.  Without it (or under no_grad) the forward computes
+    kernel of its own: one forward pass less, 1.75 instead of 2.32 ms for 64
+    candidates at 640x512 (4.43 instead of 5.96 seen end-on).  Without it (or under no_grad) the forward computes
     the loss alone and the backward evaluates both."""
 
     @staticmethod

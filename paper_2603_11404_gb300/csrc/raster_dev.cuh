@@ -419,11 +419,9 @@ static __device__ void raster_warp(const TriSetup &t, uint32_t *bm, int Wq, int 
 // one bounding box instead of two.  Anything else (a fold at a silhouette edge,
 // a non-convex or degenerate pair, a flagged vertex) is drawn as two triangles.
 // ----------------------------------------------------------------------------
-// Twice the signed area of (p, q, r); exact in int32 when every coordinate
-// difference is below 2^15.
-__device__ __forceinline__ long long orient2(int2 p, int2 q, int2 r, bool narrow)
+// Twice the signed area of (p, q, r).
+__device__ __forceinline__ long long orient2(int2 p, int2 q, int2 r)
 {
-    if (narrow) return (long long)((q.x - p.x) * (r.y - p.y) - (r.x - p.x) * (q.y - p.y));
     return (long long)(q.x - p.x) * (long long)(r.y - p.y) - (long long)(r.x - p.x) * (long long)(q.y - p.y);
 }
 
@@ -656,9 +654,9 @@ static __device__ void draw_rows_large(bool live, int2 c0, int2 c1, int2 c2, int
     const int2 mid = c2, end = c3;
     long long A = 0;
     if (live) {
-        A = orient2(c0, c1, c2, false);
+        A = orient2(c0, c1, c2);
         if (!tri) {
-            const long long A2 = orient2(c0, c2, c3, false), Da = orient2(c1, c3, c0, false), Dc = orient2(c1, c3, c2, false);
+            const long long A2 = orient2(c0, c2, c3), Da = orient2(c1, c3, c0), Dc = orient2(c1, c3, c2);
             // same non-zero orientation, and c0, c2 strictly on opposite sides of c1-c3
             if (!(((A > 0 && A2 > 0) || (A < 0 && A2 < 0)) && ((Da > 0 && Dc < 0) || (Da < 0 && Dc > 0)))) tri = two = true;
         }
@@ -729,7 +727,7 @@ static __device__ void draw_rows_large(bool live, int2 c0, int2 c1, int2 c2, int
         if (live) {
             c1 = mid;
             c2 = end;
-            A = orient2(c0, c1, c2, false);
+            A = orient2(c0, c1, c2);
         }
     }
 }

@@ -779,13 +779,14 @@ __device__ __forceinline__ float combine_lanes(const float (&Q)[kBlkPx], int lan
 // Persistent blocks over the listed pixel blocks.  A light block of pixels is
 // one warp's (no barrier, at most one batch that is not full); a heavy one (a
 // shaft seen end-on puts thousands of triangles within its reach) is shared by
-// the block's warps, every fourth group to a warp.  Bound by issue (72 % of the
-// cycles; half of the instructions evaluate pairs, a third collect them).
-// 640x512, 20k triangles, 64 candidates (two scenes): 0.52 and 1.54 ms; with
-// every block shared by four warps 0.92 and 1.93 ms, with one warp each 0.56
-// and 1.44 ms -- but then 8 candidates, where the heaviest blocks decide, take
-// 1.52 instead of 1.03 ms for a loss and a gradient.  (A pixel per thread with
-// the triangles in shared memory, about 180 instructions per pair: 12 ms.)
+// the block's warps, every fourth group to a warp.  Bound by issue (65 % of the
+// cycles; half of the instructions evaluate pairs, a third collect them).  The
+// loss of 64 candidates at 640x512, 20k triangles, takes 0.61 and 0.67 ms in two
+// scenes and 1.57 ms in one seen end-on.  With every block shared by four warps
+// this kernel takes 1.3 to 1.8 times as long; with one warp each about as long,
+// but then 8 candidates, where the heaviest blocks decide, take half as long again
+// for a loss and a gradient.  (A pixel per thread with the triangles in shared
+// memory, about 180 instructions per pair, was 8 to 20 times slower.)
 // Every kCheck batches a warp looks whether the pixels are saturated (see
 // kSaturated) by its own products and the last ones the other warps left in
 // shared memory: those only grow, so a decision made on them holds, and the
@@ -896,10 +897,11 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
 // FP32 has it: a margin assigned more pixels to the wrong edge than it put right
 // (gradients of 20k triangles 1.0e-6 -> 5.0e-6 from 64 bits at worst).
 // The blocks are the forward's, two at a time (half the atomic additions for a
-// few more idle lanes); light and heavy ones as there.  Bound by issue: 1.03
-// and 2.53 ms for the forward's scenes above.  With the groups walking the whole
-// of their windows, one set of additions per triangle, 18-21 % of the lanes
-// had a pair within reach (here 60 %): 5.6 ms for the second scene.
+// few more idle lanes); light and heavy ones as there.  Bound by issue (70 % of
+// the cycles); a loss and its gradient in the forward's three scenes: 1.75, 2.05
+// and 4.43 ms.  With the groups walking the whole of their windows, one set of
+// additions per triangle, 18-21 % of the lanes had a pair within reach (here
+// 60 %) and this kernel took 2.2 times as long.
 struct EdgeSums {
     float U[3], V[3], W[3], Wt[3];
 };
