@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 5) k_soft_fwd(SoftArgs a)
 // FP32 has it: a margin assigned more pixels to the wrong edge than it put right
 // (gradients of 20k triangles 1.0e-6 -> 5.0e-6 from 64 bits at worst).
 // The blocks are the forward's, two at a time (half the atomic additions for a
-// few more idle lanes); light and heavy ones as there.  Bound by issue (70 % of
+// few more idle lanes); light and heavy ones as there.  Bound by issue (67 % of
 // the cycles); a loss and its gradient in the forward's three scenes: 1.75, 2.05
 // and 4.43 ms.  With the groups walking the whole of their windows, one set of
 // additions per triangle, 18-21 % of the lanes had a pair within reach (here
